@@ -128,8 +128,8 @@ typedef struct {
 
 /* Options of the B index (the sky partition of paper §2.3). The index cuts
  * the sphere into declination zones of height zone_height_arcsec, each zone
- * into RA cells about as wide as they are high; B sources are sorted by
- * (zone, RA). 0 selects 20 arcsec. build_fp64 also stores float64 unit
+ * into RA cells about as wide as they are high; B sources are filed by zone
+ * and RA. 0 selects 20 arcsec. build_fp64 also stores float64 unit
  * vectors, which the FP64 path reads (it falls back to computing them). */
 typedef struct {
     double zone_height_arcsec;
@@ -222,9 +222,9 @@ XM_API xm_status xm_prof_entry(int32_t i, const char** kernel, double* total_ms,
 /* ---- the B index (paper §2.3, sky partitioning) ------------------------ */
 
 /* Builds the resident, immutable index of catalogue B: ingest (longitude
- * normalisation, validity), zone and RA key per source, a stable radix sort
- * on (zone, RA key), per-zone offsets, and per-source float32 tangent-plane
- * offsets from float64 cell centres. The index keeps B's frame; an A
+ * normalisation, validity), zone and RA key per source, a partition of the
+ * sources into zones and RA buckets with the buckets' table, and per-source
+ * float32 tangent-plane offsets from float64 cell centres. The index keeps B's frame; an A
  * catalogue in another frame is rotated into it at match time. Synchronises
  * `stream` once. Errors: XM_EINVAL (bad opts or coordinates), XM_ENOMEM,
  * XM_ECUDA. */
@@ -646,14 +646,14 @@ XM_API xm_status xm_measure_peak(int32_t what, double* value, void* stream);
 
 /* ---- test hook (no counterpart in the paper) ----------------------------- */
 
-/* Sets the look-back of the radix sort's counting passes for tests of its
- * bounded waits: spin_limit is the number of polls after which a look-back
+/* Sets the look-backs of the radix sort's counting passes and of the index
+ * build's prefix sums for tests of their bounded waits: spin_limit is the number of polls after which a look-back
  * gives up (0 restores the default, one to two seconds of polling), and
  * silent_tile (-1 = none) is a tile that publishes none of its status words,
  * so the look-backs after it wait on words nobody writes. A look-back that
- * gives up lets its kernel finish (that pass's output is then not sorted)
- * and the call that ran the sort returns XM_ETIMEOUT; the device stays
- * usable. The setting holds for every later sort in the process until it is
+ * gives up lets its kernel finish (what it computes is then not used) and
+ * the call that ran it returns XM_ETIMEOUT; the device stays
+ * usable. The setting holds for every later call in the process until it is
  * reset; it is for tests, not for production use. Errors: XM_EINVAL. */
 XM_API xm_status xm_debug_lookback(int32_t spin_limit, int32_t silent_tile);
 

@@ -2,23 +2,27 @@
 //
 // The paper files every source of the second catalogue under a sky cell so a
 // source of the first catalogue need only look at nearby cells. Here the
-// partition is a set of equal-height declination zones cut into RA cells,
-// realised by a stable radix sort of the sources on (zone, RA key):
-//   k_zone_geom   per zone: centre, its sin/cos, number and width of RA cells
-//                 (once per device and zone count, then copied)
-//   k_ingest_b    per source, input order: validity, fixed-point position,
-//                 sort key, the float32 offsets in its cell; exact position
-//                 kept by row
-//   index sort    (xm_sort.cu) on a plan k_ingest_b narrows: the zone range
-//                 and the RA bits that vary, so a catalogue of a small sky
-//                 area sorts in fewer passes; the offsets ride along
-//   k_zone_start  first sorted source of each zone (binary search)
-//   k_zone_rows   rows of each zone, size of its RA bucket table (one to two
-//                 buckets per source); prefix sum; k_zone_lut the offsets
-//   k_gather_b    the 16-byte records in (zone, RA) order (float32 offsets
-//                 in the cell's tangent frame, RA key, row) from the sorted
-//                 arrays, and the bucket tables
-//   k_gap_fill    the long runs of the bucket tables
+// partition is a set of equal-height declination zones cut into RA buckets.
+// Within a bucket the order of the sources is free, so the build is not a
+// sort but a partition that ends in shared memory: it reads and writes a
+// source's 16-byte record two or three times.
+//   k_zone_geom    per zone: sin/cos of its centre, number and width of RA
+//                  cells (once per device and zone count)
+//   k_zone_count   sources of each zone
+//   k_zone_bins    (large catalogues) first row of each zone; bins of
+//                  consecutive zones holding a few hundredths of the rows
+//   k_ingest_b     validity, fixed-point position, the record (float32
+//                  offsets in its cell, RA key, row), exact position kept by
+//                  row; records leave grouped by bin
+//   k_zone_parts   (large catalogues) zones of many sources cut into RA parts
+//   k_cell_count   (large catalogues) sources of each cell: zone or part
+//   k_cell_units   first row of each cell; units of consecutive cells that
+//                  fit one block's shared memory
+//   k_split        (large catalogues) records of a bin grouped by unit
+//   k_place_b      per unit: RA buckets counted in shared memory, the zones'
+//                  bucket tables and the records in bucket order written
+// Up to about a million sources the bins are the units themselves and the
+// steps marked "large catalogues" are left out.
 #include <math.h>
 #include <string.h>
 
@@ -26,7 +30,7 @@
 #include <new>
 #include <vector>
 
-#include "xm_internal.cuh"
+#include "xm_lookback.cuh"
 
 namespace xm {
 
@@ -34,67 +38,397 @@ namespace {
 
 constexpr int kBlock = 256;
 
-__global__ void k_zone_geom(int32_t nz, ZoneInfo* __restrict__ zones) {
+// Units: consecutive cells whose first rows fall in the same window of
+// 2^kUnitRowBits rows, of zones in the same kUnitZones, form one unit; a part
+// of a zone, and a cell of more rows than a window, begins a unit (which ends
+// with it: the next cell begins in a later window). So a unit of several
+// cells holds fewer than two windows' rows, and only a unit of one cell can
+// hold more than k_place_b stages. Zones of more than kPartMin sources are cut
+// into parts of half of kPartRows to kPartRows on average, so nearly every
+// unit fits the stage. (Unstaged, a block per zone reading its records twice
+// from L2, the placing of 2e8 records took 2.3 ms in zones of 7400 and 4 to 5
+// ms in zones of 22000 and more, whose records no longer stay in L2.)
+constexpr int kUnitRowBits = 9, kUnitZoneBits = 6;
+constexpr int kUnitZones = 1 << kUnitZoneBits;
+constexpr uint32_t kPartMin = 896, kPartRows = 800;
+
+// Digits of a split: the units of a small catalogue, or the bins of the first
+// of two splits, or the units of a bin in the second. A bin covers zones with
+// the same z >> kBinZoneBits (records carry the low bits of their zone).
+constexpr int kMaxUnits = 2048, kMaxBins = 1024, kMaxDigits = 1536;
+constexpr int kBinZoneBits = 11;
+
+// Three blocks of 384 threads an SM, 3072 records a tile. Bound by latency and
+// instruction issue (all-sky index, 2e8 sources: ingest 3.57 ms, second split
+// 2.20 ms, at 0.4 of the copy bandwidth by their 48 and 32 bytes a source); two
+// blocks of 512 with 4096 records measured within 7 % of it.
+constexpr int kSplitThreads = 384;
+constexpr int kTileItems = 8;
+constexpr int kTile = kSplitThreads * kTileItems;  // records of a tile
+constexpr int kCursorStep = 8;   // cursors lie 32 bytes apart: on one cache line
+                                 // they slowed each other down 5 to 10 times
+constexpr int kCellSlots = 4096;  // cells of a bin counted in shared memory
+constexpr int kCountChunk = 8;    // tiles a k_cell_count block takes
+constexpr size_t kCountSmem = 220 * 1024;  // k_zone_count's counters at most
+
+__global__ void k_zone_geom(int32_t nz, ZoneGeo* __restrict__ geo) {
     pdl_wait();
     const int32_t z = blockIdx.x * blockDim.x + threadIdx.x;
     if (z >= nz) return;
     const double h = kPi / nz;
     const double lo = -kHalfPi + z * h;
     const double hi = lo + h;
-    ZoneInfo Z;
-    memset(&Z, 0, sizeof(Z));
-    Z.dec_c = -kHalfPi + (z + 0.5) * h;
-    sincos(Z.dec_c, &Z.sin_c, &Z.cos_c);
-    Z.sin_cf = (float)Z.sin_c;
-    Z.cos_cf = (float)Z.cos_c;
+    double sin_c, cos_c;
+    sincos(-kHalfPi + (z + 0.5) * h, &sin_c, &cos_c);
     // widest edge of the zone: its cells are at most h wide there
     const double cos_edge = (lo <= 0.0 && hi >= 0.0) ? 1.0 : cos(fmin(fabs(lo), fabs(hi)));
     double nb = ceil(kTwoPi * cos_edge / h);
     if (nb < 1) nb = 1;
     if (nb > 1073741824.0) nb = 1073741824.0;
+    ZoneGeo Z;
+    Z.sin_cf = (float)sin_c;
+    Z.cos_cf = (float)cos_c;
+    Z.binw_f = (float)(kTwoPi / nb);
     Z.nbins = (uint32_t)nb;
-    Z.binw = kTwoPi / nb;
-    Z.binw_f = (float)Z.binw;
-    zones[z] = Z;
+    geo[z] = Z;
 }
 
-// Narrows the sort plan to a block's keys: warp reductions, one lane per warp
-// through shared memory, then an atomic only where the block widens what the
-// plan already holds (a stale read costs one redundant atomic, never a miss).
-__device__ __forceinline__ void plan_accumulate(bool has, uint32_t z, uint32_t ra,
-                                                SortPlan* plan) {
-    __shared__ uint32_t red[4][kBlock / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t zlo = __reduce_min_sync(0xFFFFFFFFu, has ? z : 0xFFFFFFFFu);
-    const uint32_t zhi = __reduce_max_sync(0xFFFFFFFFu, has ? z : 0u);
-    const uint32_t rand_ = __reduce_and_sync(0xFFFFFFFFu, has ? ra : 0xFFFFFFFFu);
-    const uint32_t ror = __reduce_or_sync(0xFFFFFFFFu, has ? ra : 0u);
-    if (lane == 0) {
-        red[0][warp] = zlo;
-        red[1][warp] = zhi;
-        red[2][warp] = rand_;
-        red[3][warp] = ror;
+__device__ __forceinline__ ZoneGeo load_geo(const ZoneGeo* p) {
+    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
+    ZoneGeo Z;
+    Z.sin_cf = __uint_as_float(u.x);
+    Z.cos_cf = __uint_as_float(u.y);
+    Z.binw_f = __uint_as_float(u.z);
+    Z.nbins = u.w;
+    return Z;
+}
+
+// What the ingest reads of a source's zone, in one load: the geometry, and
+// above the RA cells (fewer than 2^21: zones are at least 1 arcsec high) the
+// digit of the first split, a bin or a unit.
+constexpr int kDigitShift = 21;
+static_assert(kMaxUnits <= 1 << (32 - kDigitShift), "a digit fits above the RA cells");
+
+__device__ __forceinline__ void write_zone_in(const ZoneGeo* geo, uint4* zin, int64_t z, uint32_t digit) {
+    uint4 u = __ldg(reinterpret_cast<const uint4*>(geo + z));
+    u.w |= digit << kDigitShift;
+    zin[z] = u;
+}
+
+// A latitude the index accepts (the others count as 0 and fail the call). A
+// source's zone depends on its latitude alone, valid longitude or not, so that
+// the counts hold for every row.
+__device__ __forceinline__ double lat_or_zero(double lat) {
+    const uint64_t b = (uint64_t)__double_as_longlong(lat) & 0x7FFFFFFFFFFFFFFFull;
+    return keep_or_zero(lat, b <= 0x4056800000000000ull);  // bits of 90.0
+}
+
+__device__ __forceinline__ bool build_failed(const int32_t* err) {
+    return (*(const volatile int32_t*)err & kErrTimeout) != 0;
+}
+
+// Sources per zone. WIDE 0: counters in global memory (few sources, or more
+// zones than shared memory holds counters for); 1: a 32-bit counter per zone
+// in shared memory; 2: 16-bit counters, folded into the global ones before
+// they can overflow. On 2e8 sources in 27,000 zones the shared form takes
+// 0.41 ms (the 8 bytes it reads per source), global atomics 2.1 ms.
+template <int WIDE>
+__global__ void __launch_bounds__(1024) k_zone_count(const double* __restrict__ lat, int64_t n,
+                                                     int32_t nz, uint32_t* __restrict__ zcnt) {
+    pdl_wait();
+    extern __shared__ uint32_t h[];
+    if (WIDE) {
+        for (int i = threadIdx.x; i < (WIDE == 1 ? nz : (nz + 1) / 2); i += blockDim.x) h[i] = 0;
+        __syncthreads();
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t a = red[0][0], b = red[1][0], c = red[2][0], d = red[3][0];
-        for (int w = 1; w < kBlock / 32; w++) {
-            a = min(a, red[0][w]);
-            b = max(b, red[1][w]);
-            c &= red[2][w];
-            d |= red[3][w];
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * step) {
+        double la[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) la[k] = i0 + k * step < n ? lat[i0 + k * step] : 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if (i0 + k * step >= n) break;
+            const int32_t z = zone_of_lat(lat_or_zero(la[k]), nz);
+            if (WIDE == 0) {
+                atomicAdd(&zcnt[z], 1u);
+            } else if (WIDE == 1) {
+                atomicAdd(&h[z], 1u);
+            } else {
+                const int sh = 16 * (z & 1);
+                if (((atomicAdd(&h[z >> 1], 1u << sh) >> sh) & 0xFFFFu) == 0x7FFFu) {
+                    atomicSub(&h[z >> 1], 0x8000u << sh);
+                    atomicAdd(&zcnt[z], 0x8000u);
+                }
+            }
         }
-        const volatile SortPlan* vp = plan;
-        if (a < vp->zmin) atomicMin(&plan->zmin, a);
-        if (b > vp->zmax) atomicMax(&plan->zmax, b);
-        if (~c & vp->ra_and) atomicAnd(&plan->ra_and, c);
-        if (d & ~vp->ra_or) atomicOr(&plan->ra_or, d);
+    }
+    if (!WIDE) return;
+    __syncthreads();
+    for (int z = threadIdx.x; z < nz; z += blockDim.x) {
+        const uint32_t v = WIDE == 1 ? h[z] : (h[z >> 1] >> (16 * (z & 1))) & 0xFFFFu;
+        if (v) atomicAdd(&zcnt[z], v);
     }
 }
+
+// ---- prefix sums over zones and cells (256 threads x 4 elements a tile)
+
+constexpr int kPreItems = 4;
+constexpr int kPreTile = kBlock * kPreItems;
+
+struct PreTile {
+    int64_t warp_tot[kBlock / 32];
+    int64_t prefix;
+    unsigned int tile;
+};
+
+__device__ __forceinline__ int64_t take_tile(PreTile& S, unsigned int* counter) {
+    if (threadIdx.x == 0) S.tile = atomicAdd(counter, 1u);
+    __syncthreads();
+    return S.tile;
+}
+
+// Exclusive prefix of v[0] of this thread over the block (thread t holds
+// elements 4t .. 4t + 3, v their values) and the block's total.
+__device__ __forceinline__ int64_t block_prefix(PreTile& S, const int64_t* v, int64_t* all) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int64_t sum = 0;
+#pragma unroll
+    for (int k = 0; k < kPreItems; k++) sum += v[k];
+    int64_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) S.warp_tot[warp] = incl;
+    __syncthreads();
+    int64_t woff = 0, tot = 0;
+#pragma unroll
+    for (int w = 0; w < kBlock / 32; w++) {
+        if (w < warp) woff += S.warp_tot[w];
+        tot += S.warp_tot[w];
+    }
+    __syncthreads();
+    *all = tot;
+    return woff + incl - sum;
+}
+
+// The same over the whole grid.
+__device__ __forceinline__ int64_t tile_prefix(PreTile& S, int64_t tile, const int64_t* v,
+                                               uint64_t* status, Lookback lb, int32_t* err) {
+    int64_t all;
+    const int64_t mine = block_prefix(S, v, &all);
+    if (threadIdx.x < 32) {
+        const int64_t p = lookback_warp(status, tile, all, lb.spin_limit, tile == lb.silent_tile, err);
+        if (threadIdx.x == 0) S.prefix = p;
+    }
+    __syncthreads();
+    return S.prefix + mine;
+}
+
+// First row of each zone, and the bins of the first split (two splits):
+// zones whose first rows share row >> kb, and whose numbers share
+// z >> kBinZoneBits.
+__global__ void __launch_bounds__(kBlock) k_zone_bins(
+    const uint32_t* __restrict__ zcnt, int32_t nz, int64_t n, int kb,
+    const ZoneGeo* __restrict__ geo, uint4* __restrict__ zin, uint32_t* __restrict__ bin_start, uint32_t* __restrict__ bin_zone, uint32_t* __restrict__ bcur,
+    int32_t nbins, uint64_t* status, unsigned int* counter, Lookback lb, int32_t* err) {
+    pdl_wait();
+    __shared__ PreTile S;
+    const int64_t tile = take_tile(S, counter);
+    const int64_t z0 = tile * kPreTile + threadIdx.x * kPreItems;
+    int64_t v[kPreItems];
+#pragma unroll
+    for (int k = 0; k < kPreItems; k++) v[k] = z0 + k < nz ? zcnt[z0 + k] : 0;
+    int64_t start = tile_prefix(S, tile, v, status, lb, err);
+    int64_t before = z0 > 0 && z0 < nz ? start - zcnt[z0 - 1] : 0;
+#pragma unroll
+    for (int k = 0; k < kPreItems; k++) {
+        const int64_t z = z0 + k;
+        if (z >= nz) break;
+        const int32_t b = (int32_t)(start >> kb) + (int32_t)(z >> kBinZoneBits);
+        const int32_t bp = z == 0 ? -1 : (int32_t)(before >> kb) + (int32_t)((z - 1) >> kBinZoneBits);
+        write_zone_in(geo, zin, z, (uint32_t)b);
+        for (int32_t i = bp + 1; i <= b && i < nbins; i++) {  // (ids before b without a zone: empty)
+            bin_start[i] = (uint32_t)start;
+            bin_zone[i] = (uint32_t)z;
+            bcur[i * kCursorStep] = (uint32_t)start;
+        }
+        if (z == nz - 1)
+            for (int32_t i = b + 1; i <= nbins; i++) {
+                bin_start[i] = (uint32_t)n;
+                if (i < nbins) bin_zone[i] = 0;
+            }
+        before = start;
+        start += v[k];
+    }
+}
+
+// What the ingest narrows: the range of the top 16 bits of the RA key, as
+// maxima (of 65535 - key and of key) so that zeroed memory is the empty range.
+struct KeyRange {
+    uint32_t not_min, max;
+};
+
+// Zone z's cells: its parts are (key >> (16 + shift)) - p0, cell first + part.
+struct __align__(16) ZoneCells {
+    uint32_t first;  // first cell
+    uint32_t parts;
+    uint32_t p0;
+    uint32_t shift;  // RA bits (of the top 16) below a part number
+};
+
+__device__ __forceinline__ ZoneCells load_cells(const ZoneCells* p) {
+    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
+    return ZoneCells{u.x, u.y, u.z, u.w};
+}
+
+__device__ __forceinline__ uint32_t cell_of(const ZoneCells& Z, uint32_t ra_key) {
+    return Z.first + ((ra_key >> kIndexRaShift) >> Z.shift) - Z.p0;
+}
+
+// Zones of many sources into RA parts; the last block lays out the tiles of
+// the second split and the chunks of the cell count (those of the bins before
+// it, per bin).
+__global__ void __launch_bounds__(kBlock) k_zone_parts(
+    const uint32_t* __restrict__ zcnt, int32_t nz, const KeyRange* range,
+    ZoneCells* __restrict__ zcells, uint32_t* __restrict__ cell_zone,
+    uint32_t* __restrict__ cell_split, uint32_t cells_cap, uint32_t* n_cells,
+    const uint32_t* __restrict__ bin_start, int32_t nbins, uint32_t* __restrict__ bin_tile,
+    uint32_t* __restrict__ bin_chunk,
+    uint64_t* status, unsigned int* counter, Lookback lb, int32_t* err) {
+    pdl_wait();
+    if (build_failed(err)) return;
+    __shared__ PreTile S;
+    if (blockIdx.x == gridDim.x - 1) {  // (takes no tile)
+        static_assert(kMaxBins <= kPreTile, "a thread holds kPreItems bins");
+        for (int which = 0; which < 2; which++) {
+            const uint32_t rows = which ? kCountChunk * kTile : kTile;
+            uint32_t* out = which ? bin_chunk : bin_tile;
+            int64_t v[kPreItems], all;
+#pragma unroll
+            for (int k = 0; k < kPreItems; k++) {
+                const int b = threadIdx.x * kPreItems + k;
+                v[k] = b < nbins ? (bin_start[b + 1] - bin_start[b] + rows - 1) / rows : 0;
+            }
+            int64_t run = block_prefix(S, v, &all);
+#pragma unroll
+            for (int k = 0; k < kPreItems; k++) {
+                const int b = threadIdx.x * kPreItems + k;
+                if (b < nbins) out[b] = (uint32_t)run;
+                run += v[k];
+            }
+            if (threadIdx.x == 0) out[nbins] = (uint32_t)all;
+        }
+        return;
+    }
+    const int64_t tile = take_tile(S, counter);
+    const int64_t z0 = tile * kPreTile + threadIdx.x * kPreItems;
+    const uint32_t kmin = 65535u - range->not_min, kmax = range->max;
+    const uint64_t width = kmax >= kmin ? kmax - kmin + 1 : 1;
+    uint32_t sh[kPreItems];
+    int64_t v[kPreItems];  // cells, and above bit 31 the unit boundaries of parts
+#pragma unroll
+    for (int k = 0; k < kPreItems; k++) {
+        const uint32_t m = z0 + k < nz ? zcnt[z0 + k] : 0;
+        uint32_t s = 16, parts = 1;
+        if (m > kPartMin) {
+            s = 0;
+            while (s < 16 && ((uint64_t)m << (s + 1)) <= kPartRows * width) s++;
+            parts = (kmax >> s) - (kmin >> s) + 1;
+            if (parts == 1) s = 16;
+        }
+        sh[k] = s;
+        v[k] = z0 + k < nz ? (int64_t)parts + (parts > 1 ? (int64_t)(parts + 1) << 31 : 0) : 0;
+    }
+    int64_t run = tile_prefix(S, tile, v, status, lb, err);
+#pragma unroll
+    for (int k = 0; k < kPreItems; k++) {
+        const int64_t z = z0 + k;
+        if (z >= nz) break;
+        const uint32_t first = (uint32_t)(run & 0x7FFFFFFF), split = (uint32_t)(run >> 31);
+        const uint32_t parts = (uint32_t)(v[k] & 0x7FFFFFFF);
+        zcells[z] = ZoneCells{first, parts, parts > 1 ? kmin >> sh[k] : 0, sh[k]};
+        for (uint32_t p = 0; p < parts && first + p < cells_cap; p++) {
+            cell_zone[first + p] = (uint32_t)z;
+            // parts are units of their own: each part (marked in the top
+            // bit), and the zone after them, starts a unit
+            cell_split[first + p] = parts > 1 ? (split + p + 1) | 0x80000000u : split;
+        }
+        run += v[k];
+        if (z == nz - 1) *n_cells = min((uint32_t)(run & 0x7FFFFFFF), cells_cap);
+    }
+}
+
+// First row of each cell and the units. A cell is a zone when cell_zone is
+// NULL (the cells are then the zones, in order, and the ingest splits by unit:
+// zin).
+__global__ void __launch_bounds__(kBlock) k_cell_units(
+    const uint32_t* __restrict__ cnt, uint32_t n_cells, const uint32_t* n_cells_dev,
+    const uint32_t* __restrict__ cell_zone, const uint32_t* __restrict__ cell_split, int64_t n,
+    const ZoneGeo* __restrict__ geo, uint4* __restrict__ zin, uint32_t* __restrict__ cell_start,
+    uint32_t* __restrict__ cell_unit,
+    uint4* __restrict__ unit, uint32_t* __restrict__ ucur, uint32_t unit_cap,
+    uint32_t* n_units, uint64_t* status, unsigned int* counter, Lookback lb, int32_t* err) {
+    pdl_wait();
+    if (n_cells_dev) {
+        if (build_failed(err)) return;
+        n_cells = *n_cells_dev;
+    }
+    __shared__ PreTile S;
+    // a cell's rows, and above bit 31 whether it begins a unit by its size
+    // (a part does so anyway)
+    auto sums = [&](int64_t c) {
+        const uint32_t m = cnt[c];
+        const bool wide = m > (1u << kUnitRowBits) && !(cell_split && cell_split[c] >> 31);
+        return (int64_t)m | (wide ? 1ll << 31 : 0);
+    };
+    const int64_t tile = take_tile(S, counter);
+    if (tile * kPreTile >= n_cells) return;
+    const int64_t c0 = tile * kPreTile + threadIdx.x * kPreItems;
+    int64_t v[kPreItems];
+#pragma unroll
+    for (int k = 0; k < kPreItems; k++) v[k] = c0 + k < n_cells ? sums(c0 + k) : 0;
+    const int64_t before = tile_prefix(S, tile, v, status, lb, err);
+    int64_t start = before & 0x7FFFFFFF, wide = before >> 31;
+    // (first row of cell c, wide cells up to and with it)
+    auto unit_of = [&](int64_t c, int64_t first_row, int64_t n_wide) {
+        const uint32_t z = cell_zone ? cell_zone[c] : (uint32_t)c;
+        return (first_row >> kUnitRowBits) + (z >> kUnitZoneBits) + n_wide +
+               (cell_split ? cell_split[c] & 0x7FFFFFFFu : 0);
+    };
+    int64_t up = c0 > 0 && c0 < n_cells ? unit_of(c0 - 1, start - cnt[c0 - 1], wide) : -1;
+#pragma unroll
+    for (int k = 0; k < kPreItems; k++) {
+        const int64_t c = c0 + k;
+        if (c >= n_cells) break;
+        wide += v[k] >> 31;
+        const int64_t u = unit_of(c, start, wide);
+        cell_start[c] = (uint32_t)start;
+        cell_unit[c] = (uint32_t)u;
+        if (zin) write_zone_in(geo, zin, c, (uint32_t)u);
+        const uint32_t z = cell_zone ? cell_zone[c] : (uint32_t)c;
+        for (int64_t i = up + 1; i <= u && i < unit_cap; i++) {  // (ids skipped: empty units)
+            unit[i] = make_uint4((uint32_t)c, z, (uint32_t)start, 0);
+            ucur[i * kCursorStep] = (uint32_t)start;
+        }
+        if (c == (int64_t)n_cells - 1) {
+            cell_start[n_cells] = (uint32_t)n;
+            const int64_t nu = min(u + 1, (int64_t)unit_cap);
+            unit[nu] = make_uint4(n_cells, 0, (uint32_t)n, 0);
+            *n_units = (uint32_t)nu;
+        }
+        up = u;
+        start += v[k] & 0x7FFFFFFF;
+    }
+}
+
+// ---- records
 
 // The float32 offsets (xi, eta) of a source in the tangent frame of its cell
 // (zone centre line, RA cell centre), from its exact fixed-point position k.
-__device__ __forceinline__ void cell_offsets(const PosKey& k, float h_f, const ZoneInfo& Z,
+__device__ __forceinline__ void cell_offsets(const PosKey& k, float h_f, const ZoneGeo& Z,
                                              float* xi, float* eta) {
     const uint32_t ra_key = (uint32_t)(k.key64 >> 32) & kRaKeyMask;
     const uint32_t bin = bin_of(ra_key, Z.nbins);
@@ -105,244 +439,714 @@ __device__ __forceinline__ void cell_offsets(const PosKey& k, float h_f, const Z
     *eta = fmaf(L.cd * Z.sin_cf, hav_a, L.sdd);
 }
 
-// Ingest of B, one source per thread in input order: validity, longitude
-// mod 360, the exact position kept by row, the sort key (zone above the RA
-// key to 2^-24 of a turn; the sort orders on the zone and the top 16 RA
-// bits only), and the record's float32 offsets in its cell as the sort's
-// payload (x in the low word, y in the high word), so the records are
-// formed in index order without reading positions at random rows.
-__global__ void __launch_bounds__(kBlock) k_ingest_b(
-    const double* __restrict__ lon, const double* __restrict__ lat, int64_t n, int32_t nz,
-    float h_f, const ZoneInfo* __restrict__ zones, uint64_t* __restrict__ keys,
-    uint32_t* __restrict__ vals, uint64_t* __restrict__ pay, double2* __restrict__ pos,
-    double* __restrict__ px, double* __restrict__ py, double* __restrict__ pz, SortPlan* plan,
-    int32_t* err) {
-    pdl_wait();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool has = i < n;
-    uint32_t z = 0, ra = 0;
-    if (has) {
-        double lo = lon[i], la = lat[i];
-        const bool ok = coord_ok(lo, la);
-        if (!ok) atomicOr(err, kErrCoord);
-        lo = keep_or_zero(lo, ok);
-        la = keep_or_zero(la, ok);
-        lo = lon_mod360(lo);
-        const PosKey k = pos_key(lo, la, nz);
-        z = (uint32_t)k.z;
-        const uint32_t rk = (uint32_t)(k.key64 >> 32) & kRaKeyMask;
-        ra = (rk & kIndexRaMask) >> kIndexSortBeginBit;
-        keys[i] = ((uint64_t)z << 32) | rk;
-        vals[i] = (uint32_t)i;
-        float xi, eta;
-        cell_offsets(k, h_f, zones[z], &xi, &eta);
-        pay[i] = (uint64_t)__float_as_uint(xi) | ((uint64_t)__float_as_uint(eta) << 32);
-        pos[i] = make_double2(lo, la);
-        if (px) unit64_deg(lo, la, &px[i], &py[i], &pz[i]);
+// On their way records carry the low bits of their zone where a finished
+// record has zeros: 8 bits in the low byte of the RA key, and between the two
+// splits 3 more in the top exponent bits of the offsets (which are below 2 in
+// size) and the sign of the row.
+__device__ __forceinline__ uint4 tag_record(float xi, float eta, uint32_t ra24, uint32_t row,
+                                            uint32_t z, bool wide) {
+    uint4 r = make_uint4(__float_as_uint(xi), __float_as_uint(eta), ra24 | (z & 255u), row);
+    if (wide) {
+        r.x |= ((z >> 8) & 1u) << 30;
+        r.y |= ((z >> 9) & 1u) << 30;
+        r.w |= ((z >> 10) & 1u) << 31;
     }
-    plan_accumulate(has, z, ra, plan);
+    return r;
 }
 
-// The sorted keys and rows of an index build: where the plan's passes left
-// them.
-struct Sorted {
-    const uint64_t* k0;
-    const uint32_t* v0;
-    const uint64_t* p0;
-    const uint64_t* k1;
-    const uint32_t* v1;
-    const uint64_t* p1;
-    const SortPlan* plan;
-    __device__ __forceinline__ const uint64_t* keys() const { return sorted_in_scratch(plan) ? k1 : k0; }
-    __device__ __forceinline__ const uint32_t* vals() const { return sorted_in_scratch(plan) ? v1 : v0; }
-    __device__ __forceinline__ const uint64_t* pays() const { return sorted_in_scratch(plan) ? p1 : p0; }
-};
+__device__ __forceinline__ uint32_t wide_tag(const uint4& r) {
+    return (r.z & 255u) | ((r.x >> 30) & 1u) << 8 | ((r.y >> 30) & 1u) << 9 | (r.w >> 31) << 10;
+}
 
-__global__ void k_zone_start(Sorted S, int64_t n, int32_t nz, int64_t* __restrict__ zone_start) {
+__device__ __forceinline__ uint4 narrow_record(uint4 r) {
+    r.x &= ~(1u << 30);
+    r.y &= ~(1u << 30);
+    r.w &= ~(1u << 31);
+    return r;
+}
+
+// Shared memory of a tile that leaves grouped by digit: staged records, their
+// digits, digit counts (then starts), and where each digit's run goes.
+template <int ITEMS, int DIGITS>
+struct SplitSmem {
+    uint4 rec[kSplitThreads * ITEMS];
+    uint32_t cnt[DIGITS];
+    uint32_t to[DIGITS];
+    uint16_t dig[kSplitThreads * ITEMS];
+    uint32_t warp_tot[kSplitThreads / 32];
+};
+constexpr uint32_t kNoRecord = 0xFFFFFFFFu;
+
+// The tile's records to memory, grouped by digit (dr: digit << 16 | rank of
+// each record, or kNoRecord): ranks are those of the counting atomics (any
+// order within a digit), a run of each digit is claimed from its cursor by
+// one atomic, and consecutive threads then store consecutive records of a
+// run. (Records waiting in shared memory instead of registers, for more
+// blocks per SM, measured slower: the shared-memory pipe limits it.)
+template <int ITEMS, int DIGITS>
+__device__ __forceinline__ void split_tile(SplitSmem<ITEMS, DIGITS>& S, const uint4 (&r)[ITEMS],
+                                           const uint32_t (&dr)[ITEMS], int nd, uint32_t* cursors,
+                                           int64_t n, uint4* __restrict__ out) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __syncthreads();
+    // digit starts within the tile: thread t sums digits [t * per, ...)
+    const int per = (nd + kSplitThreads - 1) / kSplitThreads;
+    uint32_t sum = 0;
+    for (int k = 0; k < per; k++) {
+        const int d = tid * per + k;
+        if (d < nd) sum += S.cnt[d];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) S.warp_tot[warp] = incl;
+    __syncthreads();
+    uint32_t run = incl - sum, total = 0;
+#pragma unroll
+    for (int w = 0; w < kSplitThreads / 32; w++) {
+        if (w < warp) run += S.warp_tot[w];
+        total += S.warp_tot[w];
+    }
+    for (int k = 0; k < per; k++) {
+        const int d = tid * per + k;
+        if (d >= nd) break;
+        const uint32_t c = S.cnt[d];
+        S.cnt[d] = run;
+        if (c) S.to[d] = atomicAdd(&cursors[(int64_t)d * kCursorStep], c) - run;
+        run += c;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < ITEMS; k++) {
+        if (dr[k] == kNoRecord) continue;
+        const uint32_t p = S.cnt[dr[k] >> 16] + (dr[k] & 0xFFFFu);
+        S.rec[p] = r[k];
+        S.dig[p] = (uint16_t)(dr[k] >> 16);
+    }
+    __syncthreads();
+    for (uint32_t p = tid; p < total; p += kSplitThreads) {
+        const uint32_t g = S.to[S.dig[p]] + p;
+        if (g < n) out[g] = S.rec[p];
+    }
+}
+
+// Counts a record under its digit; digit << 16 | its rank there. (Lanes that
+// all hold one digit, as in a catalogue stored by position, add it once.)
+__device__ __forceinline__ uint32_t count_digit(uint32_t* cnt, int32_t d) {
+    if (__all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {
+        if (d < 0) return kNoRecord;
+        const int lane = threadIdx.x & 31;
+        uint32_t base = 0;
+        if (lane == 0) base = atomicAdd(&cnt[d], 32u);
+        return (uint32_t)d << 16 | (__shfl_sync(0xffffffffu, base, 0) + lane);
+    }
+    return d < 0 ? kNoRecord : (uint32_t)d << 16 | atomicAdd(&cnt[d], 1u);
+}
+
+// Ingest of B: validity, longitude mod 360, the exact position kept by row,
+// the record, and the records grouped by digit. WIDE: two splits (the digits
+// are bins; wide tags; the key range narrowed); otherwise the digits are
+// the units.
+template <int ITEMS, bool WIDE, int DIGITS>
+__global__ void __launch_bounds__(kSplitThreads, 3) k_ingest_b(
+    const double* __restrict__ lon, const double* __restrict__ lat, int64_t n, int32_t nz,
+    float h_f, const uint4* __restrict__ zin, int nd, uint32_t* cursors, uint4* __restrict__ out,
+    double2* __restrict__ pos, double* __restrict__ px, double* __restrict__ py,
+    double* __restrict__ pz, KeyRange* range, int32_t* err) {
     pdl_wait();
-    const int32_t z = blockIdx.x * blockDim.x + threadIdx.x;
-    if (z > nz) return;
-    const uint64_t* __restrict__ keys = S.keys();
-    const uint64_t target = (uint64_t)z << 32;
-    int64_t lo = 0, hi = n;
-    while (lo < hi) {
-        const int64_t mid = lo + ((hi - lo) >> 1);
-        if (keys[mid] < target) lo = mid + 1;
+    if (build_failed(err)) return;
+    extern __shared__ __align__(16) unsigned char split_smem[];
+    auto& S = *reinterpret_cast<SplitSmem<ITEMS, DIGITS>*>(split_smem);
+    const int64_t base = (int64_t)blockIdx.x * (kSplitThreads * ITEMS) + threadIdx.x;
+    // (the coordinates wait where the records will be)
+    uint4 r[ITEMS];
+#pragma unroll
+    for (int k = 0; k < ITEMS; k++) {
+        const int64_t i = base + k * kSplitThreads;
+        if (i < n) {
+            const int2 a = __ldcs(reinterpret_cast<const int2*>(lon) + i);
+            const int2 b = __ldcs(reinterpret_cast<const int2*>(lat) + i);
+            r[k] = make_uint4((uint32_t)a.x, (uint32_t)a.y, (uint32_t)b.x, (uint32_t)b.y);
+        }
+    }
+    for (int d = threadIdx.x; d < nd; d += kSplitThreads) S.cnt[d] = 0;
+    __syncthreads();
+    uint32_t dr[ITEMS];
+    uint32_t not_min = 0, kmax = 0;
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < ITEMS; k++) {
+        const int64_t i = base + k * kSplitThreads;
+        int32_t dig = -1;
+        if (i < n) {
+            const double lo = __hiloint2double((int)r[k].y, (int)r[k].x);
+            const double la = __hiloint2double((int)r[k].w, (int)r[k].z);
+            const bool ok = coord_ok(lo, la);
+            bad |= !ok;
+            const double lat_k = lat_or_zero(la);
+            const double lon_k = lon_mod360(keep_or_zero(lo, ok));
+            const PosKey key = pos_key(lon_k, lat_k, nz);
+            const uint4 zu = __ldg(zin + key.z);
+            dig = (int32_t)(zu.w >> kDigitShift);
+            ZoneGeo Z;
+            Z.sin_cf = __uint_as_float(zu.x);
+            Z.cos_cf = __uint_as_float(zu.y);
+            Z.binw_f = __uint_as_float(zu.z);
+            Z.nbins = zu.w & ((1u << kDigitShift) - 1u);
+            __stcs(&pos[i], make_double2(lon_k, lat_k));
+            if (px) unit64_deg(lon_k, lat_k, &px[i], &py[i], &pz[i]);
+            const uint32_t ra = (uint32_t)(key.key64 >> 32) & kRaKeyMask;
+            if (WIDE) {
+                not_min = max(not_min, 65535u - (ra >> kIndexRaShift));
+                kmax = max(kmax, ra >> kIndexRaShift);
+            }
+            float xi, eta;
+            cell_offsets(key, h_f, Z, &xi, &eta);
+            r[k] = tag_record(xi, eta, ra, (uint32_t)i, (uint32_t)key.z, WIDE);
+        }
+        dr[k] = count_digit(S.cnt, dig);
+    }
+    if (bad) atomicOr(err, kErrCoord);
+    if (WIDE) {  // (a stale read of the range costs one redundant atomic, never a miss)
+        not_min = __reduce_max_sync(0xffffffffu, not_min);
+        kmax = __reduce_max_sync(0xffffffffu, kmax);
+        if ((threadIdx.x & 31) == 0) {
+            const volatile KeyRange* v = range;
+            if (not_min > v->not_min) atomicMax(&range->not_min, not_min);
+            if (kmax > v->max) atomicMax(&range->max, kmax);
+        }
+    }
+    split_tile<ITEMS, DIGITS>(S, r, dr, nd, cursors, n, out);
+}
+
+// Chunk t of the bins' chunks: its bin (the last whose first chunk is <= t).
+__device__ __forceinline__ int bin_of_chunk(const uint32_t* __restrict__ bin_chunk, int nbins, uint32_t t) {
+    int lo = 0, hi = nbins;  // bin_chunk[lo] <= t < bin_chunk[hi]
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(bin_chunk + mid) <= t) lo = mid;
         else hi = mid;
     }
-    zone_start[z] = lo;
+    return lo;
 }
 
-__global__ void k_zone_rows(int32_t nz, const int64_t* __restrict__ zone_start, Sorted S,
-                            ZoneInfo* __restrict__ zones, int32_t* __restrict__ lut_cnt) {
+// Sources per cell, a chunk of one bin's records per block, counted in shared
+// memory (cells past what that holds: in global memory). The block also lists
+// its tiles for the second split: first row, row after the bin, bin.
+__global__ void __launch_bounds__(kSplitThreads) k_cell_count(
+    const uint4* __restrict__ rec, const uint32_t* __restrict__ bin_start,
+    const uint32_t* __restrict__ bin_chunk, int nbins, const uint32_t* __restrict__ bin_zone,
+    const ZoneCells* __restrict__ zcells, const uint32_t* n_cells,
+    uint32_t* __restrict__ ccnt, const uint32_t* __restrict__ bin_tile, uint4* __restrict__ tiles,
+    const int32_t* err) {
     pdl_wait();
-    const int32_t z = blockIdx.x * blockDim.x + threadIdx.x;
-    if (z >= nz) return;
-    const uint64_t* __restrict__ keys = S.keys();
-    ZoneInfo& Z = zones[z];
-    Z.start = zone_start[z];
-    Z.end = zone_start[z + 1];
-    // RA buckets over the zone's own key range: a power of two, one to two
-    // per source (a window's candidates are the rows of the buckets it
-    // touches), at most 2^24
-    const int64_t m = Z.end - Z.start;
-    int lg = 0;
-    while (lg < 24 && ((int64_t)1 << lg) < m) lg++;
-    uint32_t kmin = 0, range = 0;
-    if (m > 0) {  // (the keys are in order of their top 16 RA bits only)
-        kmin = (uint32_t)keys[Z.start] & kIndexRaMask;
-        range = ((uint32_t)keys[Z.end - 1] & kIndexRaMask) - kmin;
+    if (build_failed(err) || blockIdx.x >= bin_chunk[nbins]) return;
+    __shared__ uint32_t h[kCellSlots];
+    for (int i = threadIdx.x; i < kCellSlots; i += kSplitThreads) h[i] = 0;
+    __syncthreads();
+    const int b = bin_of_chunk(bin_chunk, nbins, blockIdx.x);
+    const uint32_t zhi = bin_zone[b] >> kBinZoneBits << kBinZoneBits;
+    const uint32_t lo = bin_start[b] + (blockIdx.x - bin_chunk[b]) * (kCountChunk * kTile);
+    const uint32_t hi = min(bin_start[b + 1], lo + kCountChunk * kTile);
+    const uint32_t first = zcells[bin_zone[b]].first;  // of the bin's cells
+    if (threadIdx.x < kCountChunk && lo + threadIdx.x * kTile < hi)
+        tiles[bin_tile[b] + (blockIdx.x - bin_chunk[b]) * kCountChunk + threadIdx.x] =
+            make_uint4(lo + threadIdx.x * kTile, bin_start[b + 1], (uint32_t)b, 0);
+    for (uint32_t i0 = lo + threadIdx.x; i0 < hi; i0 += kSplitThreads * 4) {
+        uint4 r[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            if (i0 + k * kSplitThreads < hi) r[k] = __ldg(rec + i0 + k * kSplitThreads);
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if (i0 + k * kSplitThreads >= hi) break;
+            const uint32_t c = cell_of(load_cells(zcells + (zhi + wide_tag(r[k]))), r[k].z);
+            if (c - first < kCellSlots) atomicAdd(&h[c - first], 1u);
+            else atomicAdd(&ccnt[c], 1u);
+        }
     }
-    const int bits = range ? 32 - __clz(range) : 0;
-    // buckets no finer than the order of the sorted keys (which keep only
-    // the top bits of the RA key), then as many as range >> shift needs
-    int shift = bits > lg ? bits - lg : 0;
-    if (shift < kIndexSortBeginBit) shift = kIndexSortBeginBit;
-    lg = bits > shift ? bits - shift : 0;  // range >> shift < 2^lg
-    Z.lut_shift = (uint32_t)shift;
-    Z.lut_kmin = kmin;
-    Z.lut_nb = 1u << lg;
-    lut_cnt[z] = (1 << lg) + 1;
+    __syncthreads();
+    const uint32_t nc = *n_cells;
+    for (int i = threadIdx.x; i < kCellSlots && first + i < nc; i += kSplitThreads)
+        if (h[i]) atomicAdd(&ccnt[first + i], h[i]);
 }
 
-__global__ void k_zone_lut(int32_t nz, const int64_t* __restrict__ lut_off,
-                           ZoneInfo* __restrict__ zones, ZoneHot* __restrict__ zhot,
-                           uint32_t* __restrict__ lut) {
+// The second split: a tile of one bin's records grouped by unit. (A bin of
+// more units than a tile counts claims every record's place by itself.)
+__global__ void __launch_bounds__(kSplitThreads, 3) k_split(
+    const uint4* __restrict__ rec, const uint4* __restrict__ tiles, const uint32_t* n_tiles, int nbins,
+    const uint32_t* __restrict__ bin_zone, const ZoneCells* __restrict__ zcells,
+    const uint32_t* __restrict__ cell_unit, const uint32_t* n_units, int64_t n, uint32_t* ucur,
+    uint4* __restrict__ out, const int32_t* err) {
     pdl_wait();
-    const int32_t z = blockIdx.x * blockDim.x + threadIdx.x;
-    if (z >= nz) return;
-    const int64_t base = lut_off[z];
-    zones[z].lut_base = base;
-    const ZoneInfo& Z = zones[z];
+    if (build_failed(err) || blockIdx.x >= *n_tiles) return;
+    extern __shared__ __align__(16) unsigned char split_smem[];
+    auto& S = *reinterpret_cast<SplitSmem<kTileItems, kMaxDigits>*>(split_smem);
+    const int tid = threadIdx.x;
+    const uint4 tile = __ldg(tiles + blockIdx.x);
+    const uint32_t lo = tile.x, hi = tile.y;
+    const int b = (int)tile.z;
+    uint4 r[kTileItems];
+#pragma unroll
+    for (int k = 0; k < kTileItems; k++) {
+        const uint32_t i = lo + tid + k * kSplitThreads;
+        if (i < hi) r[k] = __ldcs(rec + i);
+    }
+    const uint32_t z0 = bin_zone[b], zhi = z0 >> kBinZoneBits << kBinZoneBits;
+    // the bin's units (a unit lies in one bin): those from its first zone on
+    // that come before the next bin's first zone (0: there is none)
+    const uint32_t u0 = cell_unit[zcells[z0].first];
+    const uint32_t z1 = b + 1 < nbins ? bin_zone[b + 1] : 0;
+    const uint32_t nd = (z1 > z0 ? cell_unit[zcells[z1].first] : *n_units) - u0;
+    if (nd > kMaxDigits) {  // (rare: every record claims its place by itself)
+#pragma unroll
+        for (int k = 0; k < kTileItems; k++) {
+            if (lo + tid + k * kSplitThreads >= hi) break;
+            const ZoneCells Z = load_cells(zcells + (zhi + wide_tag(r[k])));
+            const uint32_t u = __ldg(cell_unit + cell_of(Z, r[k].z));
+            const uint32_t g = atomicAdd(&ucur[(int64_t)u * kCursorStep], 1u);
+            if (g < n) out[g] = narrow_record(r[k]);
+        }
+        return;
+    }
+    for (uint32_t d = tid; d < nd; d += kSplitThreads) S.cnt[d] = 0;
+    __syncthreads();
+    uint32_t dr[kTileItems];
+#pragma unroll
+    for (int k = 0; k < kTileItems; k++) {
+        int32_t dig = -1;
+        if (lo + tid + k * kSplitThreads < hi) {
+            const ZoneCells Z = load_cells(zcells + (zhi + wide_tag(r[k])));
+            dig = (int32_t)(__ldg(cell_unit + cell_of(Z, r[k].z)) - u0);
+            r[k] = narrow_record(r[k]);
+        }
+        dr[k] = count_digit(S.cnt, dig);
+    }
+    split_tile<kTileItems, kMaxDigits>(S, r, dr, (int)nd, ucur + (int64_t)u0 * kCursorStep, n, out);
+}
+
+// ---- the zones' buckets
+
+constexpr int kPlaceThreads = 128, kPlaceItems = 8;
+constexpr uint32_t kPlaceCap = kPlaceThreads * kPlaceItems;  // records staged
+constexpr uint32_t kPlaceCtr = 2 * kPlaceCap + 2 * kUnitZones;  // 16-bit bucket counters
+constexpr uint32_t kBigCtr = kPlaceCtr / 2 + 4 * kPlaceCap;  // 32-bit ones, with the stage's room
+constexpr int kPlaceBlocks = 8;  // per SM
+
+struct PlaceSmem {
+    uint4 stage[kPlaceCap];
+    uint32_t ctr[kPlaceCtr / 2];  // two 16-bit counters a word (directly after the stage)
+    uint32_t zmin[kUnitZones], zmax[kUnitZones];  // keys of each zone, top 16 bits
+    uint32_t zkmin[kUnitZones], zshift[kUnitZones], zlb[kUnitZones + 1];
+    uint32_t warp_tot[kPlaceThreads / 32];
+};
+// (a unit of several cells holds fewer than two windows' rows)
+static_assert(kPlaceCap >= 2u << kUnitRowBits, "units of several cells fit the stage");
+
+// What a build leaves for k_place_b.
+struct PlaceArgs {
+    const uint4* rec;            // grouped by unit
+    const uint4* unit;           // first cell, its zone and its first row, of each unit
+    const uint32_t* n_units;
+    const uint32_t* cell_start;  // first row of each cell
+    const uint32_t* cell_zone;   // NULL: cells are zones
+    const ZoneCells* zcells;     // NULL: cells are zones
+    const KeyRange* range;
+    const ZoneGeo* geo;
+    int32_t nz;
+    int64_t n;
+    BRec* out;
+    uint32_t* lut;
+    ZoneHot* zhot;
+    const int32_t* err;
+};
+
+// Buckets of a zone of m rows whose keys span [kmin, kmax] (top 16 bits in
+// place): one to two per row, never finer than kIndexRaShift bits. With
+// `aligned`, buckets begin at multiples of their width and are at most 2^most
+// wide, so that the bounds of the zone's parts are bounds of buckets.
+struct Buckets {
+    uint32_t kmin, shift, last;
+};
+
+__device__ __forceinline__ Buckets buckets_of(uint32_t m, uint32_t kmin, uint32_t kmax, bool aligned,
+                                              uint32_t most) {
+    Buckets B{kmin, (uint32_t)kIndexRaShift, 0};
+    if (m == 0 || kmax < kmin) {
+        B.kmin = 0;
+        return B;
+    }
+    const int lg = m > 1 ? 32 - __clz(m - 1) : 0;  // 2^lg >= m
+    for (int s = kIndexRaShift;; s++) {
+        const uint32_t lo = aligned ? kmin >> s << s : kmin;
+        const uint32_t last = (kmax - lo) >> s;
+        if (last < (1u << lg) || s >= (int)most) {
+            B.kmin = lo;
+            B.shift = (uint32_t)s;
+            B.last = last;
+            return B;
+        }
+    }
+}
+
+__device__ __forceinline__ void write_zone(const PlaceArgs& P, uint32_t z, uint32_t start,
+                                           uint32_t rel, const Buckets& B) {
+    const ZoneGeo Z = load_geo(P.geo + z);
     ZoneHot H;
-    H.start = (uint32_t)Z.start;
-    H.lut_rel = (int32_t)(base - 2 * Z.start);
-    H.lut_kmin = Z.lut_kmin;
-    H.shift_lg = Z.lut_shift | ((uint32_t)(__ffs(Z.lut_nb) - 1) << 8);
+    H.start = start;
+    H.lut_rel = (int32_t)rel;
+    H.lut_kmin = B.kmin;
+    H.shift_last = B.shift | (B.last << 8);
     H.nbins = Z.nbins;
     H.sin_cf = Z.sin_cf;
     H.cos_cf = Z.cos_cf;
     H.binw_f = Z.binw_f;
-    zhot[z] = H;
-    if (zones[z].end == zones[z].start) {  // empty zone: one empty bucket
-        lut[base] = 0;
-        lut[base + 1] = 0;
+    P.zhot[z] = H;
+}
+
+// Block-wide exclusive prefix of one value per thread.
+__device__ __forceinline__ uint32_t block_offset(uint32_t sum, uint32_t* warp_tot) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
     }
+    if (lane == 31) warp_tot[warp] = incl;
+    __syncthreads();
+    uint32_t run = incl - sum;
+#pragma unroll
+    for (int w = 0; w < kPlaceThreads / 32; w++)
+        if (w < warp) run += warp_tot[w];
+    return run;
 }
 
-__device__ __forceinline__ uint32_t bucket_of(uint64_t key, const ZoneInfo& Z) {
-    return (((uint32_t)key & kIndexRaMask) - Z.lut_kmin) >> Z.lut_shift;
+// Inclusive prefix, plus `add`, of n 32-bit counters in place. GLOBAL: they
+// lie in global memory, counted by atomics (read past L1).
+template <bool GLOBAL>
+__device__ __forceinline__ void scan_counters(uint32_t* c, uint32_t n, uint32_t add,
+                                              uint32_t* warp_tot) {
+    const uint32_t per = ((n + kPlaceThreads - 1) / kPlaceThreads) | 1u;
+    const uint32_t lo = min(n, threadIdx.x * per), hi = min(n, lo + per);
+    uint32_t sum = 0;
+    for (uint32_t i = lo; i < hi; i++) sum += GLOBAL ? __ldcg(c + i) : c[i];
+    uint32_t run = add + block_offset(sum, warp_tot);
+    for (uint32_t i = lo; i < hi; i++) {
+        run += GLOBAL ? __ldcg(c + i) : c[i];
+        c[i] = run;
+    }
+    __syncthreads();
 }
 
-// A run of bucket-table entries that take one value, too long for the
-// thread that found it (filled by k_gap_fill).
-struct LutGap {
-    int64_t first;   // index into the table array
-    uint32_t count;  // entries
-    uint32_t value;  // row (relative to the zone)
-};
+// Exclusive prefix of 16-bit counters, two in each of n words, in place (the
+// total fits 16 bits). A thread takes an odd number of consecutive words: no
+// bank conflicts.
+__device__ __forceinline__ void scan_pairs(uint32_t* c, uint32_t n, uint32_t* warp_tot) {
+    const uint32_t per = ((n + kPlaceThreads - 1) / kPlaceThreads) | 1u;
+    const uint32_t lo = min(n, threadIdx.x * per), hi = min(n, lo + per);
+    uint32_t sum = 0;
+    for (uint32_t i = lo; i < hi; i++) sum += c[i];
+    sum = (sum & 0xFFFFu) + (sum >> 16);
+    uint32_t run = block_offset(sum, warp_tot);
+    for (uint32_t i = lo; i < hi; i++) {
+        const uint32_t v = c[i], a = run + (v & 0xFFFFu);
+        c[i] = run | a << 16;
+        run = a + (v >> 16);
+    }
+    __syncthreads();
+}
 
-constexpr uint32_t kGapInline = 32;  // longest run written by the finding thread
+__device__ __forceinline__ uint32_t clean(uint32_t key) { return key & kRaKeyMask; }
 
-// Records into index order, and each zone's RA bucket table: bucket k holds
-// the first row (relative to the zone) whose key reaches it. The first row of
-// each run of equal buckets writes the entries from just after the previous
-// row's bucket up to its own; the zone's last row also writes the entries
-// after its bucket (the value: the zone's row count). Runs longer than
-// kGapInline go to a list for k_gap_fill.
-__global__ void k_gather_b(Sorted S, int64_t n, const ZoneInfo* __restrict__ zones,
-                           uint32_t* __restrict__ lut, BRec* __restrict__ rec,
-                           LutGap* __restrict__ gaps, unsigned long long* __restrict__ n_gaps,
-                           long long gap_cap, int32_t* err) {
-    pdl_wait();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint64_t* __restrict__ keys = S.keys();
-    const uint64_t key = keys[i];
-    const ZoneInfo& Z = zones[key >> 32];
-    const uint64_t off = S.pays()[i];
-    BRec r;
-    r.xi = __uint_as_float((uint32_t)off);
-    r.eta = __uint_as_float((uint32_t)(off >> 32));
-    r.ra_key = (uint32_t)key;
-    r.row = (int32_t)S.vals()[i];
-    rec[i] = r;
-    const int64_t rows = Z.end - Z.start, rel = i - Z.start;
-    const int64_t b = bucket_of(key, Z);
-    const int64_t pb = rel == 0 ? -1 : (int64_t)bucket_of(keys[i - 1], Z);
-    auto run = [&](int64_t first, int64_t count, uint32_t value) {
-        if (count <= 0) return;
-        if (count <= kGapInline) {
-            for (int64_t k = 0; k < count; k++) lut[Z.lut_base + first + k] = value;
-        } else {
-            const unsigned long long g = atomicAdd(n_gaps, 1ull);
-            if ((long long)g < gap_cap) gaps[g] = LutGap{Z.lut_base + first, (uint32_t)count, value};
-            else atomicOr(err, kErrOverflow);
+// Rows [s, e) of one cell, too many to stage (or of too many buckets): counted,
+// then moved one by one. B: the zone's buckets, of which the cell holds
+// [b0, b1); `base` is the table place of b0. Buckets past the counters in
+// shared memory are counted in the table itself.
+__device__ __noinline__ void place_large(const PlaceArgs& P, PlaceSmem& S, uint32_t s, uint32_t e,
+                            const Buckets& B, uint32_t b0, uint32_t b1, int64_t base) {
+    const uint32_t nb = b1 - b0;
+    uint32_t* const L = P.lut + base;
+    uint32_t* const c = nb <= kBigCtr ? reinterpret_cast<uint32_t*>(S.stage) : L;
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < nb; i += kPlaceThreads) c[i] = 0;
+    __syncthreads();
+    for (uint32_t i0 = s + threadIdx.x; i0 < e; i0 += kPlaceThreads * 4) {
+        uint32_t key[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            key[k] = i0 + k * kPlaceThreads < e ? __ldg(&P.rec[i0 + k * kPlaceThreads].z) : 0;
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            if (i0 + k * kPlaceThreads < e)
+                atomicAdd(&c[((clean(key[k]) - B.kmin) >> B.shift) - b0], 1u);
+    }
+    __syncthreads();
+    if (c != L) scan_counters<false>(c, nb, s, S.warp_tot);  // c[b]: the row after bucket b
+    else scan_counters<true>(c, nb, s, S.warp_tot);
+    for (uint32_t i0 = s + threadIdx.x; i0 < e; i0 += kPlaceThreads * 4) {
+        uint4 r[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            if (i0 + k * kPlaceThreads < e) r[k] = __ldg(&P.rec[i0 + k * kPlaceThreads]);
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if (i0 + k * kPlaceThreads >= e) break;
+            r[k].z = clean(r[k].z);
+            const uint32_t p = atomicSub(&c[((r[k].z - B.kmin) >> B.shift) - b0], 1u) - 1u;
+            reinterpret_cast<uint4*>(P.out)[p] = r[k];
         }
-    };
-    run(pb + 1, b - pb, (uint32_t)rel);
-    if (rel == rows - 1) run(b + 1, (int64_t)Z.lut_nb - b, (uint32_t)rows);
+    }
+    __syncthreads();  // (c[b]: the first row of bucket b)
+    if (c != L)
+        for (uint32_t i = threadIdx.x; i < nb; i += kPlaceThreads) L[i] = c[i];
+    __syncthreads();
 }
 
-// The long runs of the bucket tables, one block per run.
-__global__ void k_gap_fill(const LutGap* __restrict__ gaps, const unsigned long long* n_gaps,
-                           long long gap_cap, uint32_t* __restrict__ lut) {
+// Units, a block each: the records of consecutive zones, or of one part of a
+// zone, into the order of their buckets, with the zones' bucket tables. A
+// unit's records pass through registers and shared memory once: each takes a
+// rank in its bucket by a shared-memory atomic, the buckets' counts become
+// their first rows, the records go to their places in the stage, and table and
+// stage leave in order. The tables of a unit's zones lie one after the other
+// from 2 * (its first row) + 3 z + 2 c on, z its first zone and c its first
+// cell: a zone of m rows has at most 2 m + 1 entries, or one per part and one
+// more. Bound by latency and instruction issue: 3.0 ms on the all-sky index
+// (2e8 rows), 0.22 ms on 1.2e7; 384 threads with units twice as large took
+// 3.24 and 0.27 ms, 512 threads with four times as large 3.3 and 0.21 ms.
+__global__ void __launch_bounds__(kPlaceThreads, kPlaceBlocks) k_place_b(PlaceArgs P) {
     pdl_wait();
-    const long long ng = min((long long)*n_gaps, gap_cap);
-    for (long long g = blockIdx.x; g < ng; g += gridDim.x) {
-        const LutGap G = gaps[g];
-        for (uint32_t k = threadIdx.x; k < G.count; k += blockDim.x) lut[G.first + k] = G.value;
+    extern __shared__ __align__(16) unsigned char place_smem[];
+    PlaceSmem& S = *reinterpret_cast<PlaceSmem*>(place_smem);
+    if (build_failed(P.err)) {  // an index that holds nothing
+        if (blockIdx.x == 0 && threadIdx.x < 2) P.lut[threadIdx.x] = 0;
+        for (int64_t z = (int64_t)blockIdx.x * kPlaceThreads + threadIdx.x; z < P.nz;
+             z += (int64_t)gridDim.x * kPlaceThreads)
+            write_zone(P, (uint32_t)z, 0, 0, Buckets{0, 31, 0});
+        return;
+    }
+    const uint32_t n_units = *P.n_units;
+    const uint32_t tid = threadIdx.x;
+    uint4 d{}, d1{};  // this unit's first cell, zone and row, and the next's
+    if (blockIdx.x < n_units) {
+        d = __ldg(P.unit + blockIdx.x);
+        d1 = __ldg(P.unit + blockIdx.x + 1);
+    }
+    for (uint32_t u = blockIdx.x; u < n_units; u += gridDim.x) {
+        const uint32_t c0 = d.x, z0 = d.y, s = d.z, c1 = d1.x, e = d1.z;
+        if (u + gridDim.x < n_units) {
+            d = __ldg(P.unit + u + gridDim.x);
+            d1 = __ldg(P.unit + u + gridDim.x + 1);
+        }
+        if (c0 == c1) continue;  // an id without cells
+        const uint32_t m = e - s, nzones = c1 - c0;
+        bool large = m > kPlaceCap;
+        uint4 r[kPlaceItems];
+        if (!large) {
+#pragma unroll
+            for (int k = 0; k < kPlaceItems; k++) {
+                if (k * kPlaceThreads >= m) break;
+                const uint32_t i = tid + k * kPlaceThreads;
+                if (i < m) r[k] = __ldcs(P.rec + s + i);
+            }
+        }
+        ZoneCells Z{c0, 1, 0, 16};
+        if (P.zcells) Z = load_cells(P.zcells + z0);
+        const bool part = Z.parts > 1;
+        const uint32_t rel0 = P.zcells ? 3 * z0 + 2 * Z.first : 5 * z0;
+        uint32_t nb = 0;                        // counters, and table entries written
+        int64_t base = 2 * (int64_t)s + rel0;   // place of the first
+        Buckets B{};
+        uint32_t b0 = 0;
+        __syncthreads();  // (the last unit's stage and tables are out)
+        if (part) {
+            const uint32_t zs = P.cell_start[Z.first];
+            const uint32_t mz = P.cell_start[Z.first + Z.parts] - zs;
+            B = buckets_of(mz, (65535u - P.range->not_min) << 16, P.range->max << 16, true,
+                           Z.shift + kIndexRaShift);
+            const uint32_t p = c0 - Z.first;
+            const uint32_t at = Z.p0 + p, sh = Z.shift + 16;
+            b0 = p == 0 ? 0 : ((at << sh) - B.kmin) >> B.shift;
+            nb = (p + 1 == Z.parts ? B.last + 1 : (((at + 1) << sh) - B.kmin) >> B.shift) - b0;
+            base = 2 * (int64_t)zs + rel0 + b0;
+            large |= nb > kPlaceCtr;
+            if (tid == 0) {
+                if (p == 0) write_zone(P, z0, zs, rel0, B);
+                if (p + 1 == Z.parts) P.lut[base + nb] = e;
+                S.zkmin[0] = B.kmin;
+                S.zshift[0] = B.shift;
+                S.zlb[0] = 0u - b0;
+            }
+        } else if (large) {  // one zone
+            uint32_t kmin = 0xFFFFu, kmax = 0;
+            for (uint32_t i = s + tid; i < e; i += kPlaceThreads) {
+                const uint32_t key = __ldg(&P.rec[i].z) >> 16;
+                kmin = min(kmin, key);
+                kmax = max(kmax, key);
+            }
+            kmin = __reduce_min_sync(0xffffffffu, kmin);
+            kmax = __reduce_max_sync(0xffffffffu, kmax);
+            if (tid == 0) {
+                S.zmin[0] = 0xFFFFu;
+                S.zmax[0] = 0;
+            }
+            __syncthreads();
+            if ((tid & 31) == 0) {
+                atomicMin(&S.zmin[0], kmin);
+                atomicMax(&S.zmax[0], kmax);
+            }
+            __syncthreads();
+            B = buckets_of(m, S.zmin[0] << 16, S.zmax[0] << 16, false, 32);
+            nb = B.last + 1;
+            if (tid == 0) {
+                write_zone(P, z0, s, rel0, B);
+                P.lut[base + nb] = e;
+            }
+        }
+        if (large) {
+            place_large(P, S, s, e, B, b0, b0 + nb, base);
+            continue;
+        }
+        if (!part) {
+            if (tid < nzones) {
+                S.zmin[tid] = 0xFFFFu;
+                S.zmax[tid] = 0;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < kPlaceItems; k++) {
+                if (k * kPlaceThreads >= m) break;
+                if (tid + k * kPlaceThreads < m) {
+                    const uint32_t l = (r[k].z - z0) & 255u, key = r[k].z >> 16;
+                    if (key < S.zmin[l]) atomicMin(&S.zmin[l], key);
+                    if (key > S.zmax[l]) atomicMax(&S.zmax[l], key);
+                }
+            }
+            __syncthreads();
+            // zone l's buckets, and its table's place among the unit's
+            uint32_t zs = 0, entries = 0;
+            if (tid < nzones) {
+                zs = P.cell_start[c0 + tid];
+                B = buckets_of(P.cell_start[c0 + tid + 1] - zs, S.zmin[tid] << 16, S.zmax[tid] << 16,
+                               false, 32);
+                entries = B.last + 2;
+            }
+            static_assert(kUnitZones <= kPlaceThreads, "a thread per zone");
+            const uint32_t lb = block_offset(entries, S.warp_tot);
+            if (tid < nzones) {
+                S.zkmin[tid] = B.kmin;
+                S.zshift[tid] = B.shift;
+                S.zlb[tid] = lb;
+                if (tid + 1 == nzones) S.zlb[nzones] = lb + entries;
+                write_zone(P, z0 + tid, zs, rel0 + lb - 2 * (zs - s), B);
+            }
+            __syncthreads();
+            nb = S.zlb[nzones];
+        }
+        for (uint32_t i = tid; i < (nb + 1) / 2; i += kPlaceThreads) S.ctr[i] = 0;
+        __syncthreads();
+        uint32_t at[kPlaceItems];  // the record's counter, its rank there above
+#pragma unroll
+        for (int k = 0; k < kPlaceItems; k++) {
+            if (k * kPlaceThreads >= m) break;
+            if (tid + k * kPlaceThreads < m) {
+                const uint32_t l = (r[k].z - z0) & 255u;  // (0 in a part)
+                r[k].z &= kRaKeyMask;
+                const uint32_t c = S.zlb[l] + ((r[k].z - S.zkmin[l]) >> S.zshift[l]);
+                const uint32_t sh = 16 * (c & 1u);
+                at[k] = c | ((atomicAdd(&S.ctr[c >> 1], 1u << sh) >> sh) & 0xFFFFu) << 16;
+            }
+        }
+        __syncthreads();
+        scan_pairs(S.ctr, (nb + 1) / 2, S.warp_tot);
+        const uint16_t* const first = reinterpret_cast<const uint16_t*>(S.ctr);
+#pragma unroll
+        for (int k = 0; k < kPlaceItems; k++) {
+            if (k * kPlaceThreads >= m) break;
+            if (tid + k * kPlaceThreads < m) S.stage[first[at[k] & 0xFFFFu] + (at[k] >> 16)] = r[k];
+        }
+        for (uint32_t i = tid; i < nb; i += kPlaceThreads) P.lut[base + i] = s + first[i];
+        __syncthreads();
+        for (uint32_t i = tid; i < m; i += kPlaceThreads)
+            reinterpret_cast<uint4*>(P.out)[s + i] = S.stage[i];
     }
 }
 
 // Zone geometry depends only on the zone count: it is computed once per
-// (device, zone count) into a table kept for the life of the process and
-// copied into each new index.
+// (device, zone count) into a table kept for the life of the process (at most
+// 64 of them; past that, into `own`, the caller's memory).
 struct GeomCache {
     int device;
     int32_t nz;
-    ZoneInfo* zones;
+    ZoneGeo* geo;
 };
 
-xm_status zone_geometry(int32_t nz, ZoneInfo* zones, cudaStream_t s) {
+xm_status zone_geometry(int32_t nz, ZoneGeo* own, const ZoneGeo** out, cudaStream_t s) {
     static std::mutex mu;
     static std::vector<GeomCache> cache;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
-    const ZoneInfo* src = nullptr;
     {
         std::lock_guard<std::mutex> g(mu);
         for (const GeomCache& c : cache)
-            if (c.device == dev && c.nz == nz) src = c.zones;
-        if (!src && cache.size() < 64) {
-            ZoneInfo* t = nullptr;
-            if (cudaMalloc(&t, (size_t)nz * sizeof(ZoneInfo)) == cudaSuccess) {
+            if (c.device == dev && c.nz == nz) {
+                *out = c.geo;
+                return XM_OK;
+            }
+        if (cache.size() < 64) {
+            ZoneGeo* t = nullptr;
+            if (cudaMalloc(&t, (size_t)nz * sizeof(ZoneGeo)) == cudaSuccess) {
                 k_zone_geom<<<(unsigned)((nz + kBlock - 1) / kBlock), kBlock>>>(nz, t);
                 if (cudaDeviceSynchronize() == cudaSuccess) {
                     cache.push_back(GeomCache{dev, nz, t});
-                    src = t;
-                } else {
-                    cudaFree(t);
+                    *out = t;
+                    return XM_OK;
                 }
+                cudaFree(t);
             }
             cudaGetLastError();
         }
     }
-    if (src) {
-        e = cudaMemcpyAsync(zones, src, (size_t)nz * sizeof(ZoneInfo), cudaMemcpyDeviceToDevice, s);
-        return e == cudaSuccess ? XM_OK : cuda_fail(e, "zone geometry copy");
-    }
-    XM_LAUNCH("k_zone_geom", (unsigned)((nz + kBlock - 1) / kBlock), kBlock, 0, s, k_zone_geom, nz,
-              zones);
+    XM_LAUNCH("k_zone_geom", (unsigned)((nz + kBlock - 1) / kBlock), kBlock, 0, s, k_zone_geom, nz, own);
+    *out = own;
     return XM_OK;
 }
 
-int bits_for(int64_t v) {
-    int b = 0;
-    while (v > 0) { b++; v >>= 1; }
-    return b;
+// Shared-memory limits of the build's kernels, set once per device.
+void prepare_build() {
+    static std::mutex mu;
+    static bool done[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> g(mu);
+    if (dev < 0 || dev >= 64 || done[dev]) return;
+    auto set = [](auto k, size_t bytes) {
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    set(k_zone_count<1>, kCountSmem);
+    set(k_zone_count<2>, kCountSmem);
+    set(k_ingest_b<2, false, kMaxUnits>, sizeof(SplitSmem<2, kMaxUnits>));
+    set(k_ingest_b<4, false, kMaxUnits>, sizeof(SplitSmem<4, kMaxUnits>));
+    set(k_ingest_b<kTileItems, true, kMaxBins>, sizeof(SplitSmem<kTileItems, kMaxBins>));
+    set(k_split, sizeof(SplitSmem<kTileItems, kMaxDigits>));
+    set(k_place_b, sizeof(PlaceSmem));
+    done[dev] = true;
 }
+
+// Slices of one allocation, each 256-byte aligned.
+struct Slices {
+    size_t bytes = 0;
+    template <typename T>
+    size_t add(int64_t count) {
+        const size_t at = bytes;
+        bytes += ((size_t)(count > 0 ? count : 1) * sizeof(T) + 255) & ~size_t(255);
+        return at;
+    }
+};
 
 }  // namespace
 
@@ -381,30 +1185,54 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
     const bool deferred = opts && opts->deferred_check;
     const int64_t nn = n > 0 ? n : 1;
 
+    // The bins of one split are the units; past kMaxUnits units there are two
+    // splits, into 384 to 767 bins of 2^kb rows (at least a unit's window, so
+    // that units do not straddle bins) and those into units.
+    int64_t cells_cap = X->nz;
+    int64_t units_cap = 2 * (n >> kUnitRowBits) + (X->nz >> kUnitZoneBits) + 1;
+    const bool two = units_cap > kMaxUnits;
+    int kb = kUnitRowBits;
+    while (two && (n >> (kb + 1)) >= 384) kb++;
+    const int nbins = two ? (int)((n >> kb) + (X->nz >> kBinZoneBits) + 1) : 0;
+    if (two) {  // parts of zones: of half of kPartRows rows or more, of zones past kPartMin
+        cells_cap += n / 200 + 16;
+        units_cap += n / 160 + 16;
+    }
+
     xm_status st = XM_OK;
-    // temporaries
+    // temporaries: one block, the part that starts as zeros first
+    Slices W;
+    const size_t o_zcnt = W.add<uint32_t>(X->nz);
+    const size_t o_ccnt = W.add<uint32_t>(two ? cells_cap : 0);
+    const int64_t pre_z = (X->nz + kPreTile - 1) / kPreTile;
+    const int64_t pre_c = (cells_cap + kPreTile - 1) / kPreTile;
+    const size_t o_status = W.add<uint64_t>(2 * pre_z + pre_c);
+    const size_t o_small = W.add<uint32_t>(16);
+    const size_t zeroed = W.bytes;
+    const size_t o_geo = W.add<ZoneGeo>(X->nz);
+    const size_t o_zin = W.add<uint4>(X->nz);
+    const size_t o_tiles = W.add<uint4>(two ? n / kTile + nbins + 1 : 0);
+    const size_t o_bin = W.add<uint32_t>(4 * (int64_t)(nbins + 1));
+    const size_t o_bcur = W.add<uint32_t>((int64_t)(nbins + 1) * kCursorStep);
+    const size_t o_zcells = W.add<ZoneCells>(two ? X->nz : 0);
+    const size_t o_czone = W.add<uint32_t>(two ? 2 * cells_cap : 0);
+    const size_t o_cstart = W.add<uint32_t>(cells_cap + 1);
+    const size_t o_cunit = W.add<uint32_t>(cells_cap);
+    const size_t o_unit = W.add<uint4>(units_cap + 1);
+    const size_t o_ucur = W.add<uint32_t>(units_cap * kCursorStep);
     double *d_lon = nullptr, *d_lat = nullptr;
-    uint64_t *keys = nullptr, *tk = nullptr, *pay = nullptr, *tp = nullptr;
-    uint32_t *vals = nullptr, *tv = nullptr;
+    unsigned char* work = nullptr;
+    uint4* tmp = nullptr;
     int32_t* err = nullptr;
-    SortPlan* plan = nullptr;
-    int32_t* lut_cnt = nullptr;
-    int64_t* lut_off = nullptr;
-    LutGap* gaps = nullptr;
-    unsigned long long* n_gaps = nullptr;
-    long long gap_cap = 0;
     int32_t h_err = 0;
 
     auto fail = [&](xm_status code) { st = code; };
     do {
         X->rec = (BRec*)dev_alloc(nn * sizeof(BRec), s);
         X->pos = (double2*)dev_alloc(nn * sizeof(double2), s);
-        X->zone_start = (int64_t*)dev_alloc((X->nz + 1) * sizeof(int64_t), s);
-        X->zones = (ZoneInfo*)dev_alloc(X->nz * sizeof(ZoneInfo), s);
         X->zhot = (ZoneHot*)dev_alloc(X->nz * sizeof(ZoneHot), s);
-        if (!X->rec || !X->pos || !X->zone_start || !X->zones || !X->zhot) { fail(set_error(XM_ENOMEM, "index arrays")); break; }
-        X->bytes = nn * (sizeof(BRec) + sizeof(double2)) + (X->nz + 1) * sizeof(int64_t) +
-                   X->nz * (sizeof(ZoneInfo) + sizeof(ZoneHot));
+        if (!X->rec || !X->pos || !X->zhot) { fail(set_error(XM_ENOMEM, "index arrays")); break; }
+        X->bytes = nn * (sizeof(BRec) + sizeof(double2)) + X->nz * sizeof(ZoneHot);
         if (fp64) {
             X->px = (double*)dev_alloc(3 * nn * sizeof(double), s);
             if (!X->px) { fail(set_error(XM_ENOMEM, "index unit vectors")); break; }
@@ -435,64 +1263,115 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
             lon = d_lon;
             lat = d_lat;
         }
-        keys = (uint64_t*)dev_alloc(2 * nn * sizeof(uint64_t), s);
-        vals = (uint32_t*)dev_alloc(2 * nn * sizeof(uint32_t), s);
-        pay = (uint64_t*)dev_alloc(2 * nn * sizeof(uint64_t), s);
+        work = (unsigned char*)dev_alloc(W.bytes, s);
+        tmp = (uint4*)dev_alloc(nn * sizeof(uint4), s);
         err = (int32_t*)dev_alloc(sizeof(int32_t), s);
-        plan = (SortPlan*)dev_alloc(sizeof(SortPlan), s);
-        lut_cnt = (int32_t*)dev_alloc(X->nz * sizeof(int32_t), s);
-        lut_off = (int64_t*)dev_alloc(X->nz * sizeof(int64_t), s);
-        // bucket tables: a zone of m rows has at most max(2, 2m) + 1 entries
-        X->lut_n = 2 * n + 3 * (int64_t)X->nz + 16;
+        // bucket tables: see k_place_b
+        X->lut_n = 2 * n + 3 * (int64_t)X->nz + 2 * cells_cap + 16;
         X->lut = (uint32_t*)dev_alloc(X->lut_n * sizeof(uint32_t), s);
-        // runs of more than kGapInline entries: at most one per kGapInline + 1
-        // entries, plus one per zone for its last run
-        gap_cap = X->lut_n / (kGapInline + 1) + 2 * (int64_t)X->nz + 16;
-        gaps = (LutGap*)dev_alloc(gap_cap * sizeof(LutGap) + 16, s);
-        n_gaps = gaps ? (unsigned long long*)(gaps + gap_cap) : nullptr;
-        if (!keys || !vals || !pay || !err || !plan || !lut_cnt || !lut_off || !X->lut || !gaps) {
+        if (!work || !tmp || !err || !X->lut) {
             fail(set_error(XM_ENOMEM, "index build buffers"));
             break;
         }
         X->bytes += X->lut_n * sizeof(uint32_t);
-        tk = keys + nn;
-        tv = vals + nn;
-        tp = pay + nn;
         e = cudaMemsetAsync(err, 0, sizeof(int32_t), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(n_gaps, 0, sizeof(unsigned long long), s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(work, 0, zeroed, s);
         if (e != cudaSuccess) { fail(cuda_fail(e, "memset")); break; }
 
         auto body = [&]() -> xm_status {
             const IndexGeom G = X->geom();
-            const unsigned gz = (unsigned)((X->nz + kBlock) / kBlock);
-            xm_status rg = zone_geometry(X->nz, X->zones, s);
-            if (rg != XM_OK) return rg;
-            xm_status r = sort_plan_init(plan, s);
+            const int32_t nz = X->nz;
+            const Lookback lb = lookback_settings();
+            auto at32 = [&](size_t o) { return (uint32_t*)(work + o); };
+            uint32_t* const zcnt = at32(o_zcnt);
+            uint64_t* const status = (uint64_t*)(work + o_status);
+            // [0..2] tile counters, [4] cells, [5] units,
+            // [6..7] range of the RA keys
+            uint32_t* const small = at32(o_small);
+            KeyRange* const range = (KeyRange*)(small + 6);
+            uint32_t* const cstart = at32(o_cstart);
+            uint32_t* const cunit = at32(o_cunit);
+            uint4* const unit = (uint4*)(work + o_unit);
+            uint32_t* const ucur = at32(o_ucur);
+            uint4* const zin = (uint4*)(work + o_zin);
+            uint4* const tile_list = (uint4*)(work + o_tiles);
+            uint32_t* const bin_start = at32(o_bin);
+            uint32_t* const bin_zone = bin_start + nbins + 1;
+            uint32_t* const bin_tile = bin_zone + nbins + 1;
+            uint32_t* const bin_chunk = bin_tile + nbins + 1;
+            ZoneCells* const zcells = two ? (ZoneCells*)(work + o_zcells) : nullptr;
+            uint32_t* const czone = two ? at32(o_czone) : nullptr;
+            uint32_t* const csplit = two ? czone + cells_cap : nullptr;
+            uint32_t* const ccnt = two ? at32(o_ccnt) : zcnt;
+            prepare_build();
+            const ZoneGeo* geo = nullptr;
+            xm_status r = zone_geometry(nz, (ZoneGeo*)(work + o_geo), &geo, s);
             if (r != XM_OK) return r;
-            if (n > 0) {
-                const unsigned g = (unsigned)((n + kBlock - 1) / kBlock);
-                XM_LAUNCH("k_ingest_b", g, kBlock, 0, s, k_ingest_b, lon, lat, n, X->nz, G.h_f,
-                          X->zones, keys, vals, pay, X->pos, X->px, X->py, X->pz, plan, err);
+
+            // (counters in shared memory are worth their set-up from about 1e5 sources)
+            const size_t wide1 = (size_t)nz * 4, wide2 = ((size_t)nz + 1) / 2 * 4;
+            if (n >= (1 << 17) && wide1 <= kCountSmem) {
+                XM_LAUNCH("k_zone_count", 152, 1024, wide1, s, k_zone_count<1>, lat, n, nz, zcnt);
+            } else if (n >= (1 << 17) && wide2 <= kCountSmem) {
+                XM_LAUNCH("k_zone_count", 152, 1024, wide2, s, k_zone_count<2>, lat, n, nz, zcnt);
+            } else if (n > 0) {
+                const int64_t g = (n + 1023) / 1024;
+                XM_LAUNCH("k_zone_count", (unsigned)(g < 8 * 152 ? g : 8 * 152), 1024, 0, s,
+                          k_zone_count<0>, lat, n, nz, zcnt);
             }
-            // the virtual key: zone offset above the RA bits that vary
-            const int max_passes = (bits_for(X->nz - 1) + 32 - kIndexSortBeginBit + 7) / 8;
-            r = index_sort(keys, vals, pay, tk, tv, tp, n, plan, max_passes, err, s);
-            if (r != XM_OK) return r;
-            const Sorted S{keys, vals, pay, tk, tv, tp, plan};
-            XM_LAUNCH("k_zone_start", gz, kBlock, 0, s, k_zone_start, S, n, X->nz, X->zone_start);
-            XM_LAUNCH("k_zone_rows", gz, kBlock, 0, s, k_zone_rows, X->nz, X->zone_start, S,
-                      X->zones, lut_cnt);
-            r = exclusive_scan_i32(lut_cnt, lut_off, X->nz, nullptr, err, s);
-            if (r != XM_OK) return r;
-            XM_LAUNCH("k_zone_lut", gz, kBlock, 0, s, k_zone_lut, X->nz, lut_off, X->zones, X->zhot,
-                      X->lut);
-            if (n > 0) {
-                const unsigned g = (unsigned)((n + kBlock - 1) / kBlock);
-                XM_LAUNCH("k_gather_b", g, kBlock, 0, s, k_gather_b, S, n, X->zones, X->lut,
-                          X->rec, gaps, n_gaps, gap_cap, err);
-                XM_LAUNCH("k_gap_fill", 4 * 152, kBlock, 0, s, k_gap_fill, gaps, n_gaps, gap_cap,
-                          X->lut);
+            const int64_t tiles = (n + kTile - 1) / kTile;
+            if (!two) {
+                XM_LAUNCH("k_cell_units", (unsigned)pre_c, kBlock, 0, s, k_cell_units, zcnt,
+                          (uint32_t)nz, (const uint32_t*)nullptr, (const uint32_t*)nullptr,
+                          (const uint32_t*)nullptr, n, geo, zin, cstart, cunit, unit, ucur,
+                          (uint32_t)units_cap, small + 5, status, small, lb, err);
+                // (few sources: smaller tiles, so that more blocks share them)
+                auto ingest = [&](auto kernel, size_t smem, int64_t rows) -> xm_status {
+                    XM_LAUNCH("k_ingest_b", (unsigned)((n + rows - 1) / rows), kSplitThreads, smem, s,
+                              kernel, lon, lat, n, nz, G.h_f, zin, (int)units_cap, ucur, tmp,
+                              X->pos, X->px, X->py, X->pz, range, err);
+                    return XM_OK;
+                };
+                if (n > 0 && n <= 152 * 2048)
+                    r = ingest(k_ingest_b<2, false, kMaxUnits>, sizeof(SplitSmem<2, kMaxUnits>),
+                               kSplitThreads * 2);
+                else if (n > 0)
+                    r = ingest(k_ingest_b<4, false, kMaxUnits>, sizeof(SplitSmem<4, kMaxUnits>),
+                               kSplitThreads * 4);
+                if (r != XM_OK) return r;
+            } else {
+                // (the records go to the index's own array and back: the last
+                // step writes it from `tmp`)
+                uint4* const rec0 = (uint4*)X->rec;
+                XM_LAUNCH("k_zone_bins", (unsigned)pre_z, kBlock, 0, s, k_zone_bins, zcnt, nz, n, kb,
+                          geo, zin, bin_start, bin_zone, at32(o_bcur), nbins, status, small, lb,
+                          err);
+                if (n > 0)
+                    XM_LAUNCH("k_ingest_b", (unsigned)tiles, kSplitThreads,
+                              sizeof(SplitSmem<kTileItems, kMaxBins>), s,
+                              (k_ingest_b<kTileItems, true, kMaxBins>), lon, lat, n, nz, G.h_f, zin,
+                              nbins, at32(o_bcur), rec0, X->pos, X->px, X->py, X->pz,
+                              range, err);
+                XM_LAUNCH("k_zone_parts", (unsigned)pre_z + 1, kBlock, 0, s, k_zone_parts, zcnt, nz,
+                          range, zcells, czone, csplit, (uint32_t)cells_cap, small + 4, bin_start,
+                          nbins, bin_tile, bin_chunk, status + pre_z, small + 1, lb, err);
+                if (n > 0)
+                    XM_LAUNCH("k_cell_count", (unsigned)(tiles / kCountChunk + nbins + 1),
+                              kSplitThreads, 0, s, k_cell_count, rec0, bin_start, bin_chunk, nbins,
+                              bin_zone, zcells, small + 4, ccnt, bin_tile, tile_list, err);
+                XM_LAUNCH("k_cell_units", (unsigned)pre_c, kBlock, 0, s, k_cell_units, ccnt, 0u,
+                          small + 4, czone, csplit, n, geo, (uint4*)nullptr, cstart, cunit, unit, ucur,
+                          (uint32_t)units_cap, small + 5, status + 2 * pre_z, small + 2, lb, err);
+                if (n > 0)
+                    XM_LAUNCH("k_split", (unsigned)(tiles + nbins), kSplitThreads,
+                              sizeof(SplitSmem<kTileItems, kMaxDigits>), s, k_split, rec0, tile_list,
+                              bin_tile + nbins, nbins, bin_zone, zcells, cunit, small + 5, n, ucur, tmp,
+                              err);
             }
+            const PlaceArgs P{tmp, unit, small + 5, cstart, czone, zcells, range, geo, nz, n,
+                              X->rec, X->lut, X->zhot, err};
+            XM_LAUNCH("k_place_b", (unsigned)(units_cap < kPlaceBlocks * 152 ? units_cap : kPlaceBlocks * 152),
+                      kPlaceThreads, sizeof(PlaceSmem), s, k_place_b, P);
             return XM_OK;
         };
         st = body();
@@ -510,14 +1389,9 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
     } while (0);
 
     dev_free(d_lon, s);
-    dev_free(keys, s);
-    dev_free(vals, s);
-    dev_free(pay, s);
+    dev_free(work, s);
+    dev_free(tmp, s);
     dev_free(err, s);
-    dev_free(plan, s);
-    dev_free(lut_cnt, s);
-    dev_free(lut_off, s);
-    dev_free(gaps, s);
     if (st != XM_OK) {
         xm_index_free(X);
         return st;
@@ -528,8 +1402,7 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
 
 xm_status xm::index_build_status(int32_t bits) {
     if (bits & kErrCoord) return set_error(XM_EINVAL, "B: NaN/inf or |lat| > 90");
-    if (bits & kErrTimeout) return set_error(XM_ETIMEOUT, "index sort: look-back timed out");
-    if (bits & kErrOverflow) return set_error(XM_ECUDA, "index bucket tables: run list overflow");
+    if (bits & kErrTimeout) return set_error(XM_ETIMEOUT, "index build: look-back timed out");
     return XM_OK;
 }
 
@@ -542,8 +1415,6 @@ extern "C" xm_status xm_index_free(xm_index* X) {
     dev_free(X->pos, s);
     dev_free(X->px, s);
     dev_free(X->id, s);
-    dev_free(X->zone_start, s);
-    dev_free(X->zones, s);
     dev_free(X->zhot, s);
     dev_free(X->lut, s);
     dev_free(X->build_err, s);

@@ -61,39 +61,26 @@ enum : int32_t {
     kErrOverflow = 8,   // a fixed-capacity buffer would overflow
 };
 
-// One declination zone. Its B sources are rows [start, end) of the index,
-// sorted by ra_key. The RA bucket table spans the zone's own key range
-// [lut_kmin, last key]: lut[lut_base + k], k = (ra_key - lut_kmin) >>
-// lut_shift (k < lut_nb), holds the first row (relative to start) whose key
-// reaches bucket k, and lut[lut_base + lut_nb] the zone's row count; a window
-// bound is two table reads and a short search.
-struct __align__(16) ZoneInfo {
-    double dec_c;          // zone centre latitude (rad)
-    double sin_c, cos_c;   // of dec_c, float64
-    double binw;           // RA cell width (rad)
-    int64_t start, end;    // index rows of the zone
-    // the four fields the B ingest reads for every source, in one 32-byte
-    // sector (across two sectors its pass took 2.62 ms instead of 2.00 on
-    // the all-sky index)
-    float sin_cf, cos_cf;  // of dec_c, float32
-    float binw_f;          // RA cell width (rad), float32
+// Float32 geometry of one declination zone (16 bytes, one load).
+struct __align__(16) ZoneGeo {
+    float sin_cf, cos_cf;  // of the zone centre latitude
+    float binw_f;          // RA cell width (rad)
     uint32_t nbins;        // RA cells
-    int64_t lut_base;      // first bucket entry of the zone
-    uint32_t lut_shift;    // key bits per bucket
-    uint32_t lut_kmin;     // smallest ra_key of the zone
-    uint32_t lut_nb;       // buckets (a power of two)
 };
 
-// The fields of a zone the candidate scan reads, packed into one 32-byte
-// sector (the table of all zones stays in L2). Catalogues hold fewer than
-// 2^31 rows, so the zone's first row fits 32 bits; the bucket table of a zone
-// of m rows has at most 2m + 1 entries (2 when empty), so its first entry lies
-// within [start + z, 2 start + 2z] and is kept relative to 2 start.
+// One zone of the index, as the candidate scan reads it: one 32-byte sector
+// (the table of all zones stays in L2). A zone's B sources are consecutive
+// rows of the index, in the order of its RA buckets: bucket k holds the keys
+// with (ra_key - lut_kmin) >> shift = k, and entry k of the zone's bucket table
+// is its first index row (entry last + 1: the row after the zone). The table
+// lies at lut[2 * start + lut_rel] (catalogues hold fewer than 2^31 rows, so
+// the zone's first row fits 32 bits; tables take about two entries a row, so
+// their place fits 32 bits relative to it).
 struct __align__(32) ZoneHot {
     uint32_t start;     // first index row of the zone
     int32_t lut_rel;    // first bucket entry of the zone, minus 2 * start
-    uint32_t lut_kmin;  // smallest ra_key of the zone
-    uint32_t shift_lg;  // key bits per bucket | log2(buckets) << 8
+    uint32_t lut_kmin;  // no key of the zone lies below it
+    uint32_t shift_last;  // key bits per bucket | last bucket << 8
     uint32_t nbins;     // RA cells
     float sin_cf, cos_cf;  // of the zone centre latitude
     float binw_f;          // RA cell width (rad)
@@ -106,7 +93,7 @@ __device__ __forceinline__ ZoneHot load_zone_hot(const ZoneHot* p) {
     z.start = u.x;
     z.lut_rel = (int32_t)u.y;
     z.lut_kmin = u.z;
-    z.shift_lg = u.w;
+    z.shift_last = u.w;
     z.nbins = v.x;
     z.sin_cf = __uint_as_float(v.y);
     z.cos_cf = __uint_as_float(v.z);
@@ -158,8 +145,7 @@ struct IndexGeom {
     const double* px;    // float64 unit vectors by B row (nullable)
     const double* py;
     const double* pz;
-    const ZoneInfo* zones;  // [nz]
-    const ZoneHot* zhot;    // [nz] the scan's part of each zone
+    const ZoneHot* zhot;    // [nz]
     const uint32_t* lut;    // RA bucket tables of all zones
     int32_t nz;
     double h;        // zone height (rad)
@@ -215,13 +201,17 @@ struct PosKey {
     float zfrac;     // zone coordinate minus zone centre line, in zones
 };
 
-// High 64 bits of the 128-bit product (host and device).
-__host__ __device__ __forceinline__ uint64_t mulhi64(uint64_t a, uint64_t b) {
-#ifdef __CUDA_ARCH__
-    return __umul64hi(a, b);
-#else
-    return (uint64_t)(((unsigned __int128)a * b) >> 64);
-#endif
+// floor(t / 45) and the remainder, for t < 45 * 2^32, in 32-bit arithmetic:
+// the quotient of t's bits above 6, times 64/45 (rounded down twice, so short
+// by less than 154 / 45), then that of what is left. (A 64-bit division by the
+// constant takes twice the instructions; a B source needs four of these.)
+__host__ __device__ __forceinline__ uint32_t div45(uint64_t t, uint32_t* rem) {
+    const uint32_t h = (uint32_t)(t >> 6);
+    const uint32_t q = h + (uint32_t)(((uint64_t)h * 0x6C16C16Cu) >> 32);  // 2^32 * 19/45
+    const uint32_t r = (uint32_t)t - 45u * q;
+    const uint32_t k = (r * 1457u) >> 16;  // floor(r / 45) for r < 2000
+    *rem = r - 45u * k;
+    return q + k;
 }
 
 // floor(m * 2^s / 45) for m < 2^53 and s <= 18, exactly, in integer
@@ -240,12 +230,21 @@ __host__ __device__ __forceinline__ uint64_t fx_div45(uint64_t m, int s, bool* e
     }
     const uint64_t lo = m << s;
     const uint64_t hi = s ? (m >> (64 - s)) : 0;  // N = hi * 2^64 + lo < 45 * 2^64
-    const uint64_t t1 = (hi << 32) | (lo >> 32);
-    const uint64_t q1 = t1 / 45u;
-    const uint64_t t0 = ((t1 - q1 * 45u) << 32) | (lo & 0xFFFFFFFFull);
-    const uint64_t q0 = t0 / 45u;
-    *exact = q0 * 45u == t0;
-    return (q1 << 32) + q0;
+    uint32_t rem;
+    const uint32_t q1 = div45((hi << 32) | (lo >> 32), &rem);
+    const uint32_t q0 = div45(((uint64_t)rem << 32) | (lo & 0xFFFFFFFFull), &rem);
+    *exact = rem == 0;
+    return ((uint64_t)q1 << 32) | q0;
+}
+
+// The product of a 64-bit fraction (of 2^64) and a count, in counts: integer
+// part, and the top 24 bits of the fraction as a float.
+__host__ __device__ __forceinline__ uint32_t mul_frac(uint64_t f, uint32_t n, float* frac) {
+    const uint64_t p = (f >> 32) * n + (((f & 0xFFFFFFFFull) * n) >> 32);
+    // (the fraction converts through 32 bits: a 64-bit integer conversion
+    // would take the float64 pipe)
+    *frac = (float)((uint32_t)p >> 8) * 5.9604644775390625e-08f;  // 2^-24
+    return (uint32_t)(p >> 32);
 }
 
 // Significand and exponent of |x| (x finite): |x| = m * 2^(e - 52).
@@ -269,6 +268,26 @@ __host__ __device__ __forceinline__ void split_double(double x, uint64_t* m, int
 // key is floor(lon / 360 * 2^64) and the latitude key floor((lat + 90) / 180
 // * 2^64) (clamped below 2^64), both exact; the zone is the top part of the
 // latitude key times the zone count and the zone fraction its low part.
+__host__ __device__ __forceinline__ uint64_t lat_key64(double lat) {
+    uint64_t m;
+    int e;
+    bool exact;
+    // |lat| * 2^64 / 180 = m * 2^(e + 10) / 45
+    split_double(lat, &m, &e);
+    const uint64_t u = fx_div45(m, e + 10, &exact);
+    const uint64_t half = 1ull << 63;
+    uint64_t lat_bits;
+    memcpy(&lat_bits, &lat, sizeof(lat_bits));
+    if ((lat_bits >> 63) == 0) return u >= half ? ~0ull : half + u;
+    return half - (u + (exact ? 0 : 1));
+}
+
+// Zone of a latitude (the z of pos_key).
+__host__ __device__ __forceinline__ int32_t zone_of_lat(double lat, int32_t nz) {
+    const uint64_t lk = lat_key64(lat);
+    return (int32_t)(((lk >> 32) * (uint32_t)nz + (((lk & 0xFFFFFFFFull) * (uint32_t)nz) >> 32)) >> 32);
+}
+
 __host__ __device__ __forceinline__ PosKey pos_key(double lon, double lat, int32_t nz) {
     PosKey k;
     uint64_t m;
@@ -277,17 +296,9 @@ __host__ __device__ __forceinline__ PosKey pos_key(double lon, double lat, int32
     // lon * 2^64 / 360 = m * 2^(e + 9) / 45
     split_double(lon, &m, &e);
     k.key64 = fx_div45(m, e + 9, &exact);
-    // |lat| * 2^64 / 180 = m * 2^(e + 10) / 45
-    split_double(lat, &m, &e);
-    const uint64_t u = fx_div45(m, e + 10, &exact);
-    const uint64_t half = 1ull << 63;
-    uint64_t lk;
-    uint64_t lat_bits;
-    memcpy(&lat_bits, &lat, sizeof(lat_bits));
-    if ((lat_bits >> 63) == 0) lk = u >= half ? ~0ull : half + u;
-    else lk = half - (u + (exact ? 0 : 1));
-    k.z = (int32_t)mulhi64(lk, (uint64_t)nz);
-    k.zfrac = (float)(uint32_t)((lk * (uint64_t)nz) >> 40) * 5.9604644775390625e-08f - 0.5f;  // 2^-24
+    float frac;
+    k.z = (int32_t)mul_frac(lat_key64(lat), (uint32_t)nz, &frac);
+    k.zfrac = frac - 0.5f;
     return k;
 }
 
@@ -299,12 +310,9 @@ __device__ __forceinline__ uint32_t bin_of(uint32_t ra_key, uint32_t nbins) {
 // nbins cells, in cells: key64 * nbins / 2^64 - bin - 1/2, from the exact
 // 128-bit product.
 __device__ __forceinline__ float cells_from_centre(uint64_t key64, uint32_t nbins, uint32_t bin) {
-    const uint64_t hi = __umul64hi(key64, (uint64_t)nbins);
-    const uint64_t lo = key64 * (uint64_t)nbins;
-    // (the 24-bit fraction converts through 32 bits: a 64-bit integer
-    // conversion would take the float64 pipe)
-    const float frac = (float)(uint32_t)(lo >> 40) * 5.9604644775390625e-08f;  // 2^-24
-    return (float)(int32_t)((uint32_t)hi - bin) + (frac - 0.5f);
+    float frac;
+    const uint32_t cell = mul_frac(key64, nbins, &frac);
+    return (float)(int32_t)(cell - bin) + (frac - 0.5f);
 }
 
 // sin(x) and 1 - cos(x) = 2 sin^2(x/2) in float32. Below |x| = 1/16 they are
@@ -560,43 +568,16 @@ xm_status radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* tk, uint32_t*
 // before capturing a stream that sorts).
 void radix_sort_prepare();
 
-// The index sort's plan, decided on the device from the keys themselves:
-// the keys (zone << 32 | RA key) are sorted on the virtual key
-// ((zone - zmin) << rb) | (RA key >> 8 & (2^rb - 1)), where the RA bits
-// above rb are the same in every key, so its order is the key order and it
-// needs only `active` 8-bit passes (trailing passes are skipped).
-struct SortPlan {
-    uint32_t zmin, zmax;      // zone range (atomicMin / atomicMax)
-    uint32_t ra_and, ra_or;   // AND / OR of the 24-bit RA fields
-    uint32_t rb, active;      // RA bits kept, passes needed
-};
-
-// Sets a plan to the empty ranges the key kernel narrows.
-xm_status sort_plan_init(SortPlan* plan, cudaStream_t s);
-
-// Sorts (keys, vals, pay) of an index build by the plan's virtual key with up
-// to `max_passes` launches (each does nothing past plan->active); pay (a
-// 64-bit payload per key, with scratch tp) may be NULL. The sorted data ends
-// in (keys, vals, pay) when plan->active is even, else in (tk, tv, tp);
-// sorted_in_scratch() tells which on the device.
-xm_status index_sort(uint64_t* keys, uint32_t* vals, uint64_t* pay, uint64_t* tk, uint32_t* tv,
-                     uint64_t* tp, int64_t n, SortPlan* plan, int max_passes, int32_t* err,
-                     cudaStream_t s);
-
-__device__ __forceinline__ bool sorted_in_scratch(const SortPlan* plan) { return plan->active & 1; }
-
 // Sort keys file sources by zone, then by RA to 2^-24 of a turn (0.08
 // arcsec): the low 8 bits of the RA key are dropped, so the sort starts at
 // bit 8. Search windows are widened by one such quantum.
 constexpr uint32_t kRaKeyMask = 0xFFFFFF00u;
 constexpr int kSortBeginBit = 8;
-// The index is ordered by zone and the top 16 bits of the RA key (2^-16 of a
-// turn, 20 arcsec): its RA bucket tables never use finer buckets, and the
-// scan compares every record's own (24-bit) key with the search window, so
-// the order within one such bucket does not matter. A 16-bit RA field saves
-// a counting pass over an all-sky index.
-constexpr uint32_t kIndexRaMask = 0xFFFF0000u;
-constexpr int kIndexSortBeginBit = 16;
+// The index files sources by zone and the top 16 bits of the RA key (2^-16
+// of a turn, 20 arcsec): its RA buckets are never finer, and the scan
+// compares every record's own (24-bit) key with the search window, so the
+// order within a bucket does not matter.
+constexpr int kIndexRaShift = 16;
 // out[i] = sum of in[0..i) (int64); *total (device) = sum of all. One
 // launch (single-pass, decoupled look-back); a look-back that timed out sets
 // kErrTimeout in *err (device), which the caller reads at its next
@@ -635,8 +616,6 @@ struct xm_index {
     double2* pos;
     double *px, *py, *pz;
     int64_t* id;
-    int64_t* zone_start;
-    xm::ZoneInfo* zones;
     xm::ZoneHot* zhot;
     uint32_t* lut;
     int64_t lut_n;
@@ -644,7 +623,7 @@ struct xm_index {
     int32_t* build_err;  // error bits of a build whose check was deferred (else NULL)
     cudaStream_t stream;  // the stream it was built on (its memory is freed in its order)
     xm::IndexGeom geom() const {
-        return xm::IndexGeom{rec, pos, px, py, pz, zones, zhot, lut, nz, h, (float)h};
+        return xm::IndexGeom{rec, pos, px, py, pz, zhot, lut, nz, h, (float)h};
     }
 };
 

@@ -358,18 +358,17 @@ __device__ __forceinline__ Window a_window(const APrep& A, const IndexGeom& G) {
 // slower: its dependent loads cost more than the extra candidate rounds.)
 __device__ __forceinline__ void bucket_bounds(const IndexGeom& G, const ZoneHot& Z, uint32_t klo,
                                               uint32_t khi, int64_t* lo_out, int64_t* hi_out) {
-    const int64_t start = Z.start;
     if (khi < Z.lut_kmin) {  // the whole window lies before the zone's first key
-        *lo_out = *hi_out = start;
+        *lo_out = *hi_out = 0;
         return;
     }
-    const uint32_t shift = Z.shift_lg & 0xFFu;
-    const uint32_t last = (1u << (Z.shift_lg >> 8)) - 1u;
-    const uint32_t* L = G.lut + (2 * start + Z.lut_rel);
+    const uint32_t shift = Z.shift_last & 0xFFu;
+    const uint32_t last = Z.shift_last >> 8;
+    const uint32_t* L = G.lut + (2 * (int64_t)Z.start + Z.lut_rel);
     const uint32_t bl = klo <= Z.lut_kmin ? 0u : min((klo - Z.lut_kmin) >> shift, last);
     const uint32_t bh = min((khi - Z.lut_kmin) >> shift, last);
-    *lo_out = start + __ldg(&L[bl]);
-    *hi_out = start + __ldg(&L[bh + 1]);
+    *lo_out = __ldg(&L[bl]);
+    *hi_out = __ldg(&L[bh + 1]);
 }
 
 // Float64 unit vector of B row `row` (exact positions are kept by row).
@@ -412,8 +411,9 @@ __device__ __forceinline__ ItemTerms item_terms(const APrep& A, const ZoneHot& Z
     t.cosc = Z.cos_cf;
     t.binw = Z.binw_f;
     t.nbins = Z.nbins;
-    t.binA = (uint32_t)__umul64hi(A.key64, (uint64_t)Z.nbins);
-    t.ufrac = (float)(uint32_t)((A.key64 * (uint64_t)Z.nbins) >> 40) * 5.9604644775390625e-08f - 0.5f;
+    float frac;
+    t.binA = mul_frac(A.key64, Z.nbins, &frac);
+    t.ufrac = frac - 0.5f;
     return t;
 }
 

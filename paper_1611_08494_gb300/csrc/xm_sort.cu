@@ -1,9 +1,8 @@
 // xm_sort.cu -- device radix sort and prefix sums.
 //
-// The sky partition of paper §2.3 assigns every source of the second
-// catalogue to a cell; here the assignment is realised by sorting sources on
-// a (zone, RA) key. The sort is a stable least-significant-digit radix sort
-// with 8-bit digits: one kernel counts the digits of every pass at once
+// The sort orders catalogue A on its (zone, RA) keys when asked to, the
+// sources of a batch, and the key columns of the Exact Value case. It is a
+// stable least-significant-digit radix sort with 8-bit digits: one kernel counts the digits of every pass at once
 // (they do not depend on the order of the keys) and turns the counts into
 // output offsets, then one kernel per pass in the single-kernel Onesweep
 // form: tiles of 4096 keys take ids in launch order, rank their keys stably
@@ -16,7 +15,7 @@
 #include <atomic>
 #include <mutex>
 
-#include "xm_internal.cuh"
+#include "xm_lookback.cuh"
 
 namespace xm {
 
@@ -28,22 +27,14 @@ constexpr int kSortTile = kSortThreads * kSortItems;  // 4096 keys
 constexpr int kWarps = kSortThreads / 32;
 constexpr int kRadix = 256;
 
-// The virtual key of an index key under a plan.
-__device__ __forceinline__ uint64_t plan_key(const SortPlan& P, uint64_t key) {
-    const uint32_t z = (uint32_t)(key >> 32);
-    const uint32_t ra = (uint32_t)key >> kIndexSortBeginBit;
-    const uint32_t rmask = P.rb >= 32 ? 0xFFFFFFFFu : ((1u << P.rb) - 1u);
-    return ((uint64_t)(z - P.zmin) << P.rb) | (ra & rmask);
-}
-
 // Digit histograms of every pass at once (they do not depend on the order of
-// the keys): hist[p * 256 + d] counts keys whose digit p is d; the digits are
-// those of key >> begin_bit, or of the plan's virtual key. The last block to
-// finish turns every pass's counts into exclusive offsets (the first output
-// slot of each digit), so the passes need not scan them.
+// the keys): hist[p * 256 + d] counts keys whose digit p (of key >> begin_bit)
+// is d. The last block to finish turns every pass's counts into exclusive
+// offsets (the first output slot of each digit), so the passes need not scan
+// them.
 __global__ void __launch_bounds__(kSortThreads) k_digit_hist(const uint64_t* __restrict__ keys,
                                                              int64_t n, int begin_bit,
-                                                             const SortPlan* plan, int passes,
+                                                             int passes,
                                                              unsigned long long* hist,
                                                              unsigned int* done) {
     pdl_wait();
@@ -51,14 +42,10 @@ __global__ void __launch_bounds__(kSortThreads) k_digit_hist(const uint64_t* __r
     __shared__ bool last;
     for (int i = threadIdx.x; i < 8 * kRadix; i += kSortThreads) (&h[0][0])[i] = 0;
     __syncthreads();
-    SortPlan P{};
-    if (plan) P = *plan;
-    // (passes a plan leaves out are not counted: all their digits are 0)
-    const int counted = plan ? min(passes, (int)P.active) : passes;
     for (int64_t i = (int64_t)blockIdx.x * kSortThreads + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * kSortThreads) {
-        const uint64_t k = plan ? plan_key(P, keys[i]) : keys[i] >> begin_bit;
-        for (int p = 0; p < counted; p++) atomicAdd(&h[p][(k >> (8 * p)) & 0xFF], 1u);
+        const uint64_t k = keys[i] >> begin_bit;
+        for (int p = 0; p < passes; p++) atomicAdd(&h[p][(k >> (8 * p)) & 0xFF], 1u);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < passes * kRadix; i += kSortThreads) {
@@ -89,50 +76,9 @@ __global__ void __launch_bounds__(kSortThreads) k_digit_hist(const uint64_t* __r
     }
 }
 
-__global__ void k_plan_init(SortPlan* plan) {
-    pdl_wait();
-    *plan = SortPlan{0xFFFFFFFFu, 0u, 0xFFFFFFFFu, 0u, 0u, 0u};
-}
-
-// The plan from the accumulated ranges: bits of the zone offset and of the
-// varying RA bits, passes needed (none for no keys).
-__global__ void k_plan_finish(SortPlan* plan) {
-    pdl_wait();
-    SortPlan P = *plan;
-    if (P.zmin > P.zmax) {
-        P.rb = 0;
-        P.active = 0;
-        *plan = P;
-        return;
-    }
-    const uint32_t ra_diff = P.ra_and ^ P.ra_or;
-    P.rb = ra_diff ? 32 - __clz(ra_diff) : 0;
-    const uint32_t zd = P.zmax - P.zmin;
-    const uint32_t zb = zd ? 32 - __clz(zd) : 0;
-    P.active = (P.rb + zb + 7) / 8;
-    *plan = P;
-}
-
-// Look-back status word of one (tile, digit): flag in the top two bits,
-// count (or inclusive prefix) below.
-constexpr uint64_t kStAgg = 1ull << 62;   // tile's own count is available
-constexpr uint64_t kStInc = 2ull << 62;   // inclusive prefix is available
-constexpr uint64_t kStMask = (1ull << 62) - 1;
-constexpr int kSpinLimit = 1 << 22;      // polls before a look-back gives up (~1-2 s)
 constexpr int kLookWindow = 8;           // status words loaded per look-back step
 
-__device__ __forceinline__ uint64_t ld_relaxed(const uint64_t* p) {
-    uint64_t v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void st_relaxed(uint64_t* p, uint64_t v) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-// A pass's shared memory; a pass that carries a 64-bit payload per key has
-// kSortTile more words of it after the struct.
+// A pass's shared memory.
 struct OnesweepSmem {
     uint64_t keys[kSortTile];
     uint32_t vals[kSortTile];
@@ -157,37 +103,20 @@ struct OnesweepSmem {
 // lowers it); silent_tile (-1 = none) is a tile that publishes nothing, so
 // the look-backs after it wait on words nobody writes -- the test form of a
 // stalled predecessor, which must end in XM_ETIMEOUT and never in a hang.
-//
-// PAY: every key also carries a 64-bit payload (pay_in -> pay_out), moved
-// with its row.
-template <bool PAY>
 __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(
     const uint64_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
-    const uint64_t* __restrict__ pay_in, int64_t n, int shift,
+    int64_t n, int shift,
     const unsigned long long* __restrict__ offs, uint64_t* status, unsigned int* tile_counter,
     uint64_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out,
-    uint64_t* __restrict__ pay_out, int32_t* err, const SortPlan* plan, int pass,
-    unsigned long long* stats, int spin_limit, int silent_tile) {
+    int32_t* err, unsigned long long* stats, int spin_limit, int silent_tile) {
     pdl_wait();
-    // with a plan: the digit of pass `pass` of the virtual key, and nothing
-    // to do past the passes the plan needs (uniform over the grid)
-    SortPlan P{};
-    const bool planned = plan != nullptr;
-    if (planned) {
-        P = *plan;
-        if (pass >= (int)P.active) return;
-    }
     extern __shared__ __align__(16) unsigned char smem_raw[];
     OnesweepSmem& S = *reinterpret_cast<OnesweepSmem*>(smem_raw);
-    uint64_t* S_pay = reinterpret_cast<uint64_t*>(smem_raw + sizeof(OnesweepSmem));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __shared__ int given_up;
     if (threadIdx.x == 0) {
         S.tile = (int)atomicAdd(tile_counter, 1u);
-        if (S.tile == 0 && stats) {  // keys this pass (and with a payload)
-            atomicAdd(&stats[5], (unsigned long long)n);
-            if (PAY) atomicAdd(&stats[6], (unsigned long long)n);
-        }
+        if (S.tile == 0 && stats) atomicAdd(&stats[5], (unsigned long long)n);  // keys this pass
         given_up = (*(volatile int32_t*)err & kErrTimeout) != 0;
     }
     for (int i = threadIdx.x; i < kWarps * kRadix; i += kSortThreads) (&S.wcount[0][0])[i] = 0;
@@ -213,7 +142,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(
     int32_t rank[kSortItems];
     // warp-striped: item k of lane l is element warp_base + 32 k + l, so the
     // (k, lane) order is the input order and ranks are stable. All key loads
-    // are issued before the ranking so they overlap; the rows (and payloads)
+    // are issued before the ranking so they overlap; the rows
     // are read only when placed (fewer live registers: reading them with the
     // keys measured slower).
 #pragma unroll
@@ -227,7 +156,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(
     uint32_t dpack[kSortItems / 4] = {};
 #pragma unroll
     for (int k = 0; k < kSortItems; k++) {
-        const uint32_t d = (uint32_t)((planned ? plan_key(P, key[k]) : key[k]) >> shift) & 0xFF;
+        const uint32_t d = (uint32_t)(key[k] >> shift) & 0xFF;
         dpack[k >> 2] |= d << (8 * (k & 3));
         if (warp_base + 32 * k + lane < n) atomicAdd(&S.hist[d], 1);
     }
@@ -332,7 +261,6 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(
             const int32_t p = S.dstart[d] + S.wcount[warp][d] + (rank[k] & 0xFFFF);
             S.keys[p] = key[k];
             S.vals[p] = vals_in[warp_base + 32 * k + lane];
-            if (PAY) S_pay[p] = pay_in[warp_base + 32 * k + lane];
             S.dig[p] = (uint8_t)d;
         }
     }
@@ -347,7 +275,6 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(
             if ((uint64_t)g < (uint64_t)n) {  // (always, unless a look-back gave up)
                 keys_out[g] = S.keys[p];
                 vals_out[g] = S.vals[p];
-                if (PAY) pay_out[g] = S_pay[p];
             }
         }
     }
@@ -503,40 +430,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_chained(
         if (w < warp) woff += warp_tot[w];
         all += warp_tot[w];
     }
-    if (warp == 0) {  // publish, then look back 32 tiles per step
-        uint64_t* my = status + tile;
-        int64_t prefix = 0;
-        if (tile == 0) {
-            if (lane == 0) st_relaxed(my, kStInc | (uint64_t)all);
-        } else {
-            if (lane == 0) st_relaxed(my, kStAgg | (uint64_t)all);
-            int64_t top = tile - 1;  // lane j reads tile top - j (before tile 0: an inclusive 0)
-            int spins = 0;
-            while (true) {
-                const int64_t j = top - lane;
-                const uint64_t w = j >= 0 ? ld_relaxed(status + j) : kStInc;
-                const uint64_t flag = w & ~kStMask;
-                const uint32_t inc = __ballot_sync(0xffffffffu, flag == kStInc);
-                const uint32_t unready = __ballot_sync(0xffffffffu, flag == 0);
-                const int first = inc ? __ffs(inc) - 1 : 31;  // words needed: lanes 0..first
-                const uint32_t need = first == 31 ? 0xffffffffu : ((1u << (first + 1)) - 1u);
-                if (unready & need) {
-                    if (++spins > kSpinLimit) {
-                        if (lane == 0) atomicOr(err, kErrTimeout);
-                        break;
-                    }
-                    __nanosleep(64);
-                    continue;
-                }
-                int64_t v = lane <= first ? (int64_t)(w & kStMask) : 0;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                prefix += v;
-                if (inc) break;
-                top -= 32;
-            }
-            if (lane == 0) st_relaxed(my, kStInc | (uint64_t)(prefix + all));
-        }
+    if (warp == 0) {
+        const int64_t prefix = lookback_warp(status, tile, all, kSpinLimit, false, err);
         if (lane == 0) {
             tile_prefix = prefix;
             if (total && (tile + 1) * kScanTile >= n) *total = prefix + all;
@@ -626,10 +521,6 @@ xm_status exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t
     return scan_impl<int64_t>(in, out, n, total, err, s);
 }
 
-size_t onesweep_smem(bool pay) {
-    return sizeof(OnesweepSmem) + (pay ? kSortTile * sizeof(uint64_t) : 0);
-}
-
 void radix_sort_prepare() {
     static std::mutex mu;
     static bool done[64] = {};
@@ -637,91 +528,34 @@ void radix_sort_prepare() {
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> g(mu);
     if (dev < 0 || dev >= 64 || done[dev]) return;
-    cudaFuncSetAttribute(k_onesweep<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)onesweep_smem(false));
-    cudaFuncSetAttribute(k_onesweep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)onesweep_smem(true));
+    cudaFuncSetAttribute(k_onesweep, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(OnesweepSmem));
     done[dev] = true;
 }
 
-// Test settings of the look-back (xm_debug_lookback): poll budget and the
-// tile that withholds its status words.
+// Test settings of the look-backs (xm_debug_lookback).
 std::atomic<int> g_spin_limit{kSpinLimit};
 std::atomic<int> g_silent_tile{-1};
+
+Lookback lookback_settings() { return Lookback{g_spin_limit.load(), g_silent_tile.load()}; }
 
 // One pass: two tiles of 512 threads x 8 keys per SM (64 registers, no
 // spills). Tiles of 256 x 16, 256 x 8, 384 x 12 and 512 x 12 keys, two to
 // four per SM with the rows read with the keys, measured from 3 % faster to
 // 29 % slower on the all-sky index.
-void onesweep_pass(int64_t ntiles, cudaStream_t s, const uint64_t* ki, const uint32_t* vi,
-                   const uint64_t* pi, int64_t n, int shift, const unsigned long long* offs,
-                   uint64_t* status, unsigned int* counter, uint64_t* ko, uint32_t* vo,
-                   uint64_t* po, int32_t* err, const SortPlan* plan, int pass) {
-    if (pi)
-        launch_pdl(k_onesweep<true>, dim3((unsigned)ntiles), dim3(kSortThreads), onesweep_smem(true),
-                   s, ki, vi, pi, n, shift, offs, status, counter, ko, vo, po, err, plan, pass,
-                   device_stats(), g_spin_limit.load(), g_silent_tile.load());
-    else
-        launch_pdl(k_onesweep<false>, dim3((unsigned)ntiles), dim3(kSortThreads), onesweep_smem(false),
-                   s, ki, vi, pi, n, shift, offs, status, counter, ko, vo, po, err, plan, pass,
-                   device_stats(), g_spin_limit.load(), g_silent_tile.load());
+void onesweep_pass(int64_t ntiles, cudaStream_t s, const uint64_t* ki, const uint32_t* vi, int64_t n,
+                   int shift, const unsigned long long* offs, uint64_t* status,
+                   unsigned int* counter, uint64_t* ko, uint32_t* vo, int32_t* err) {
+    const Lookback lb = lookback_settings();
+    launch_pdl(k_onesweep, dim3((unsigned)ntiles), dim3(kSortThreads), sizeof(OnesweepSmem), s, ki, vi,
+               n, shift, offs, status, counter, ko, vo, err, device_stats(), lb.spin_limit,
+               lb.silent_tile);
 }
 
 xm_status sort_guard(const int32_t* err, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1,
                      int64_t n, cudaStream_t s) {
     XM_LAUNCH("k_sort_guard", 2 * 152, 256, 0, s, k_sort_guard, err, k0, v0, k1, v1, n);
     return XM_OK;
-}
-
-xm_status sort_plan_init(SortPlan* plan, cudaStream_t s) {
-    XM_LAUNCH("k_plan_init", 1, 1, 0, s, k_plan_init, plan);
-    return XM_OK;
-}
-
-xm_status index_sort(uint64_t* keys, uint32_t* vals, uint64_t* pay, uint64_t* tk, uint32_t* tv,
-                     uint64_t* tp, int64_t n, SortPlan* plan, int max_passes, int32_t* err,
-                     cudaStream_t s) {
-    if (max_passes < 1 || max_passes > 8) return set_error(XM_EINVAL, "index sort: passes");
-    XM_LAUNCH("k_plan_finish", 1, 1, 0, s, k_plan_finish, plan);
-    if (n <= 1) return XM_OK;  // (one key: the plan needs no pass)
-    const int passes = max_passes;
-    const int64_t ntiles = (n + kSortTile - 1) / kSortTile;
-    const size_t st_words = (size_t)ntiles * kRadix;
-    const size_t bytes = passes * (kRadix * sizeof(unsigned long long) + st_words * sizeof(uint64_t) +
-                                   sizeof(uint64_t)) + 16;
-    unsigned char* work = (unsigned char*)dev_alloc(bytes, s);
-    if (!work) return set_error(XM_ENOMEM, "index sort of %lld keys", (long long)n);
-    unsigned long long* hist = (unsigned long long*)work;
-    uint64_t* status = (uint64_t*)(hist + passes * kRadix);
-    unsigned int* counters = (unsigned int*)(status + passes * st_words);
-    radix_sort_prepare();
-    xm_status st = XM_OK;
-    cudaError_t e = cudaMemsetAsync(work, 0, bytes, s);
-    if (e != cudaSuccess) st = cuda_fail(e, "index sort memset");
-    if (st == XM_OK) {
-        const unsigned hg = (unsigned)(ntiles < 4 * 152 ? ntiles : 4 * 152);
-        launch_begin("k_digit_hist", s);
-        // (counters + passes: a spare word of the zeroed work area)
-        launch_pdl(k_digit_hist, dim3(hg), dim3(kSortThreads), 0, s, keys, n, 0, plan, passes, hist,
-                   counters + passes);
-        e = launch_end("k_digit_hist", s);
-        if (e != cudaSuccess) st = cuda_fail(e, "k_digit_hist");
-    }
-    uint64_t *ki = keys, *ko = tk, *pi = pay, *po = tp;
-    uint32_t *vi = vals, *vo = tv;
-    for (int p = 0; p < passes && st == XM_OK; p++) {
-        launch_begin("k_onesweep", s);
-        onesweep_pass(ntiles, s, ki, vi, pi, n, 8 * p, hist + p * kRadix, status + p * st_words,
-                      counters + p, ko, vo, po, err, plan, p);
-        e = launch_end("k_onesweep", s);
-        if (e != cudaSuccess) { st = cuda_fail(e, "k_onesweep"); break; }
-        uint64_t* t = ki; ki = ko; ko = t;
-        uint32_t* u = vi; vi = vo; vo = u;
-        t = pi; pi = po; po = t;
-    }
-    if (st == XM_OK) st = sort_guard(err, keys, vals, tk, tv, n, s);
-    dev_free(work, s);
-    return st;
 }
 
 xm_status radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* tk, uint32_t* tv, int64_t n,
@@ -749,15 +583,15 @@ xm_status radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* tk, uint32_t*
     if (st == XM_OK) {
         const unsigned hg = (unsigned)(ntiles < 4 * 152 ? ntiles : 4 * 152);
         launch_begin("k_digit_hist", s);
-        launch_pdl(k_digit_hist, dim3(hg), dim3(kSortThreads), 0, s, keys, n, begin_bit,
-                   (const SortPlan*)nullptr, passes, hist, counters + passes);
+        launch_pdl(k_digit_hist, dim3(hg), dim3(kSortThreads), 0, s, keys, n, begin_bit, passes, hist,
+                   counters + passes);
         e = launch_end("k_digit_hist", s);
         if (e != cudaSuccess) st = cuda_fail(e, "k_digit_hist");
     }
     for (int p = 0; p < passes && st == XM_OK; p++) {
         launch_begin("k_onesweep", s);
-        onesweep_pass(ntiles, s, ki, vi, nullptr, n, begin_bit + 8 * p, hist + p * kRadix,
-                      status + p * st_words, counters + p, ko, vo, nullptr, err, nullptr, p);
+        onesweep_pass(ntiles, s, ki, vi, n, begin_bit + 8 * p, hist + p * kRadix,
+                      status + p * st_words, counters + p, ko, vo, err);
         e = launch_end("k_onesweep", s);
         if (e != cudaSuccess) { st = cuda_fail(e, "k_onesweep"); break; }
         uint64_t* t = ki; ki = ko; ko = t;
