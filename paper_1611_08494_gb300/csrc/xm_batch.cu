@@ -126,8 +126,13 @@ __global__ void k_batch_prep(BatchConst C, const uint32_t* __restrict__ vals,
     const double a = col_or(R.a_col, i, R.a);
     const double b = R.shape == XM_CIRCLE ? a : col_or(R.b_col, i, R.b);
     const double pa = col_or(R.pa_col, i, R.pa);
+    APrep P;
+    ACold C64;
     make_aprep(lon, lat, gamma, ok, a, b, pa, R.shape, R.pa_dir, R.size_k, R.pa_zero, C.nz, C.h_f,
-               (int32_t)g, &out[s], &cold[s]);
+               (int32_t)g, &P, &C64);
+    if (R.rotate) P.shape |= kRotated;
+    out[s] = P;
+    cold[s] = C64;
     lrow[g] = (int32_t)i;
 }
 

@@ -14,6 +14,7 @@
 //   k_ingest_b     validity, fixed-point position, the record (float32
 //                  offsets in its cell, RA key, row), exact position kept by
 //                  row; records leave grouped by bin
+//   k_unit_b       float64 unit vectors by row, for a float64 index
 //   k_zone_parts   (large catalogues) zones of many sources cut into RA parts
 //   k_cell_count   (large catalogues) sources of each cell: zone or part
 //   k_cell_units   first row of each cell; units of consecutive cells that
@@ -554,8 +555,7 @@ template <int ITEMS, bool WIDE, int DIGITS>
 __global__ void __launch_bounds__(kSplitThreads, 3) k_ingest_b(
     const double* __restrict__ lon, const double* __restrict__ lat, int64_t n, int32_t nz,
     float h_f, const uint4* __restrict__ zin, int nd, uint32_t* cursors, uint4* __restrict__ out,
-    double2* __restrict__ pos, double* __restrict__ px, double* __restrict__ py,
-    double* __restrict__ pz, KeyRange* range, int32_t* err) {
+    double2* __restrict__ pos, KeyRange* range, int32_t* err) {
     pdl_wait();
     if (build_failed(err)) return;
     extern __shared__ __align__(16) unsigned char split_smem[];
@@ -597,7 +597,6 @@ __global__ void __launch_bounds__(kSplitThreads, 3) k_ingest_b(
             Z.binw_f = __uint_as_float(zu.z);
             Z.nbins = zu.w & ((1u << kDigitShift) - 1u);
             __stcs(&pos[i], make_double2(lon_k, lat_k));
-            if (px) unit64_deg(lon_k, lat_k, &px[i], &py[i], &pz[i]);
             const uint32_t ra = (uint32_t)(key.key64 >> 32) & kRaKeyMask;
             if (WIDE) {
                 not_min = max(not_min, 65535u - (ra >> kIndexRaShift));
@@ -620,6 +619,22 @@ __global__ void __launch_bounds__(kSplitThreads, 3) k_ingest_b(
         }
     }
     split_tile<ITEMS, DIGITS>(S, r, dr, nd, cursors, n, out);
+}
+
+// Float64 unit vectors of B, by row, from the positions the ingest kept. (In
+// the ingest the evaluation's registers would cost it warps; here the pass is
+// bound by its integer instructions, 0.4 of the bandwidth by its 48 bytes a
+// source.)
+__global__ void __launch_bounds__(kBlock) k_unit_b(const double2* __restrict__ pos, int64_t n,
+                                                   double2* __restrict__ p64, const int32_t* err) {
+    pdl_wait();
+    const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
+    if (i >= n || build_failed(err)) return;
+    const double2 q = __ldcs(pos + i);
+    double x, y, z;
+    unit64_turn(lon_turn(q.x), lat_turn(q.y), &x, &y, &z);
+    __stcs(&p64[2 * i], make_double2(x, y));
+    __stcs(&p64[2 * i + 1], make_double2(z, 0.0));
 }
 
 // Chunk t of the bins' chunks: its bin (the last whose first chunk is <= t).
@@ -1234,11 +1249,9 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
         if (!X->rec || !X->pos || !X->zhot) { fail(set_error(XM_ENOMEM, "index arrays")); break; }
         X->bytes = nn * (sizeof(BRec) + sizeof(double2)) + X->nz * sizeof(ZoneHot);
         if (fp64) {
-            X->px = (double*)dev_alloc(3 * nn * sizeof(double), s);
-            if (!X->px) { fail(set_error(XM_ENOMEM, "index unit vectors")); break; }
-            X->py = X->px + nn;
-            X->pz = X->py + nn;
-            X->bytes += 3 * nn * sizeof(double);
+            X->p64 = (double2*)dev_alloc(2 * nn * sizeof(double2), s);
+            if (!X->p64) { fail(set_error(XM_ENOMEM, "index unit vectors")); break; }
+            X->bytes += 2 * nn * sizeof(double2);
         }
         if (B->id) {
             X->id = (int64_t*)dev_alloc(nn * sizeof(int64_t), s);
@@ -1329,7 +1342,7 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
                 auto ingest = [&](auto kernel, size_t smem, int64_t rows) -> xm_status {
                     XM_LAUNCH("k_ingest_b", (unsigned)((n + rows - 1) / rows), kSplitThreads, smem, s,
                               kernel, lon, lat, n, nz, G.h_f, zin, (int)units_cap, ucur, tmp,
-                              X->pos, X->px, X->py, X->pz, range, err);
+                              X->pos, range, err);
                     return XM_OK;
                 };
                 if (n > 0 && n <= 152 * 2048)
@@ -1350,7 +1363,7 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
                     XM_LAUNCH("k_ingest_b", (unsigned)tiles, kSplitThreads,
                               sizeof(SplitSmem<kTileItems, kMaxBins>), s,
                               (k_ingest_b<kTileItems, true, kMaxBins>), lon, lat, n, nz, G.h_f, zin,
-                              nbins, at32(o_bcur), rec0, X->pos, X->px, X->py, X->pz,
+                              nbins, at32(o_bcur), rec0, X->pos,
                               range, err);
                 XM_LAUNCH("k_zone_parts", (unsigned)pre_z + 1, kBlock, 0, s, k_zone_parts, zcnt, nz,
                           range, zcells, czone, csplit, (uint32_t)cells_cap, small + 4, bin_start,
@@ -1368,6 +1381,9 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
                               bin_tile + nbins, nbins, bin_zone, zcells, cunit, small + 5, n, ucur, tmp,
                               err);
             }
+            if (X->p64 && n > 0)
+                XM_LAUNCH("k_unit_b", (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, k_unit_b,
+                          X->pos, n, X->p64, err);
             const PlaceArgs P{tmp, unit, small + 5, cstart, czone, zcells, range, geo, nz, n,
                               X->rec, X->lut, X->zhot, err};
             XM_LAUNCH("k_place_b", (unsigned)(units_cap < kPlaceBlocks * 152 ? units_cap : kPlaceBlocks * 152),
@@ -1413,7 +1429,7 @@ extern "C" xm_status xm_index_free(xm_index* X) {
     cudaStream_t s = X->stream;
     dev_free(X->rec, s);
     dev_free(X->pos, s);
-    dev_free(X->px, s);
+    dev_free(X->p64, s);
     dev_free(X->id, s);
     dev_free(X->zhot, s);
     dev_free(X->lut, s);

@@ -126,9 +126,13 @@ struct __align__(16) APrep {
     float R;              // bounding radius (rad); 0 = empty region
     int32_t row;          // A row: in the caller's catalogue, or batch-wide
     float m00, m01, m10, m11;  // float32 map (x, y) -> (X/a, Y/b)
-    int32_t shape;        // xm_shape of the source's region
+    int32_t shape;        // xm_shape of the source's region, and kRotated
     float g;              // guard band of the float32 test (see make_aprep)
 };
+
+// (APrep::shape) the position was rotated into the index frame, its degrees
+// formed by a division by kDeg.
+constexpr int32_t kRotated = 4;
 
 // The float64 description of an A source, read only by float64 tests
 // (kept apart so the scan's per-source load stays at 48 bytes).
@@ -142,9 +146,7 @@ struct ACold {
 struct IndexGeom {
     const BRec* rec;
     const double2* pos;  // (lon, lat) in degrees, index frame, by B row
-    const double* px;    // float64 unit vectors by B row (nullable)
-    const double* py;
-    const double* pz;
+    const double2* p64;  // float64 unit vectors by B row, (x, y) (z, 0) (nullable)
     const ZoneHot* zhot;    // [nz]
     const uint32_t* lut;    // RA bucket tables of all zones
     int32_t nz;
@@ -352,6 +354,123 @@ __device__ __forceinline__ float zeta_of(float xi, float eta) {
     return -r2 / (1.0f + sqrtf(fmaxf(0.0f, 1.0f - r2)));
 }
 
+// ----------------------------------------- float64 unit vectors, by integers
+//
+// A float64 operation costs 64 float32 ones on this GPU, so the sines and
+// cosines of positions, which are known exactly as 64-bit fractions of a
+// turn, are evaluated in 64-bit fixed point: Taylor series on an eighth of a
+// turn, correct to a few 2^-63, rounded to float64 once. (With the library's
+// float64 functions the ingest of a float64 index of 2e7 sources took 1.97 ms
+// and its scan 1.62 ms for 5e6 sources.)
+
+// The high 64 bits of a * b, short by at most 2.
+__host__ __device__ __forceinline__ uint64_t mulhi_short(uint64_t a, uint64_t b) {
+    const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
+    return (uint64_t)ah * bh + (uint32_t)(((uint64_t)ah * bl) >> 32) + (uint32_t)(((uint64_t)al * bh) >> 32);
+}
+
+__host__ __device__ __forceinline__ uint32_t mulhi32(uint32_t a, uint32_t b) {
+    return (uint32_t)(((uint64_t)a * b) >> 32);
+}
+
+// Magnitudes (units of 2^-64, 1 saturated) and signs of the sine and cosine of
+// f / 2^64 of a turn.
+struct SinCosFx {
+    uint64_t s, c;
+    bool sneg, cneg;
+};
+
+__host__ __device__ __forceinline__ SinCosFx sincos_turn(uint64_t f) {
+    // nearest quarter q, and the rest: an angle of at most an eighth of a turn
+    const uint32_t q = (uint32_t)((f + (1ull << 61)) >> 62) & 3u;
+    const int64_t r = (int64_t)(f - ((uint64_t)q << 62));
+    const bool neg = r < 0;
+    uint64_t u = neg ? 0ull - (uint64_t)r : (uint64_t)r;
+    if (u >= 1ull << 61) u = (1ull << 61) - 1;
+    const uint64_t t = mulhi_short(u << 3, 0xC90FDAA22168C234ull);  // angle; pi / 4
+    const uint64_t z = mulhi_short(t, t);
+    const uint32_t zh = (uint32_t)(z >> 32);
+    // sin t = t - t z (1/3! - z (1/5! - ...)), 1 - cos t = z (1/2! - z (1/4! -
+    // ...)), coefficients in units of 2^-64; the last ones fit 32 bits, and so
+    // do their products
+    uint32_t a = 0xCA96u - mulhi32(zh, 0x98u);         // 1/17!, 1/19!
+    a = 0xD73F9Fu - mulhi32(zh, a);                    // 1/15!
+    a = 0xB092309Du - mulhi32(zh, a);                  // 1/13!
+    uint64_t p = 0x6B99159FD5ull - mulhi32(zh, a);     // 1/11!
+    p = 0x2E3BC74AAD8Eull - mulhi_short(z, p);         // 1/9!
+    p = 0xD00D00D00D00Dull - mulhi_short(z, p);        // 1/7!
+    p = 0x222222222222222ull - mulhi_short(z, p);      // 1/5!
+    p = 0x2AAAAAAAAAAAAAABull - mulhi_short(z, p);     // 1/3!
+    const uint64_t sn = t - mulhi_short(t, mulhi_short(z, p));
+    uint32_t b = 0xD73FAu - mulhi32(zh, 0xB41u);       // 1/16!, 1/18!
+    b = 0xC9CBA54u - mulhi32(zh, b);                   // 1/14!
+    uint64_t w = 0x8F76C77FCull - mulhi32(zh, b);      // 1/12!
+    w = 0x49F93EDDE28ull - mulhi_short(z, w);          // 1/10!
+    w = 0x1A01A01A01A02ull - mulhi_short(z, w);        // 1/8!
+    w = 0x5B05B05B05B05Bull - mulhi_short(z, w);       // 1/6!
+    w = 0xAAAAAAAAAAAAAABull - mulhi_short(z, w);      // 1/4!
+    w = mulhi_short(z, 0x8000000000000000ull - mulhi_short(z, w));  // 1/2!
+    const uint64_t cs = w ? 0ull - w : ~0ull;
+    // quarter q: (s, c), (c, -s), (-s, -c), (-c, s)
+    SinCosFx o;
+    o.s = (q & 1u) ? cs : sn;
+    o.c = (q & 1u) ? sn : cs;
+    o.sneg = (q & 1u) ? q == 3u : neg != (q == 2u);
+    o.cneg = (q & 1u) ? neg != (q == 1u) : q == 2u;
+    return o;
+}
+
+// m / 2^64 as a float64, rounded to nearest (m = 2^64 - 1 is 1), with a sign.
+__host__ __device__ __forceinline__ double from_fx(uint64_t m, bool neg) {
+#ifdef __CUDA_ARCH__
+    const int lz = __clzll((long long)m);
+#else
+    const int lz = m ? __builtin_clzll(m) : 64;
+#endif
+    const uint64_t n = m << (lz & 63);  // top bit set, unless m = 0
+    uint64_t bits = ((uint64_t)(1021 - lz) << 52) + (n >> 11) + ((n >> 10) & 1u);
+    if (m == 0) bits = 0;
+    bits |= (uint64_t)neg << 63;
+    double x;
+#ifdef __CUDA_ARCH__
+    x = __longlong_as_double((long long)bits);
+#else
+    memcpy(&x, &bits, sizeof(x));
+#endif
+    return x;
+}
+
+// Fractions of a turn of a longitude in [0, 360) and a latitude, in degrees.
+__host__ __device__ __forceinline__ uint64_t lon_turn(double lon) {
+    uint64_t m;
+    int e;
+    bool exact;
+    split_double(lon, &m, &e);
+    return fx_div45(m, e + 9, &exact);
+}
+
+__host__ __device__ __forceinline__ uint64_t lat_turn(double lat) {
+    uint64_t m, b;
+    int e;
+    bool exact;
+    split_double(lat, &m, &e);
+    const uint64_t u = fx_div45(m, e + 9, &exact);
+    memcpy(&b, &lat, sizeof(b));
+    return (b >> 63) ? 0ull - u : u;
+}
+
+// Unit vector of a position given as fractions of a turn.
+__host__ __device__ __forceinline__ void unit64_turn(uint64_t lon, uint64_t lat, double* px,
+                                                     double* py, double* pz) {
+    const SinCosFx A = sincos_turn(lon), D = sincos_turn(lat);
+    // (a factor of 1 is 2^64 - 1: the product keeps the other)
+    const uint64_t x = A.c == ~0ull ? D.c : D.c == ~0ull ? A.c : mulhi_short(D.c, A.c);
+    const uint64_t y = A.s == ~0ull ? D.c : D.c == ~0ull ? A.s : mulhi_short(D.c, A.s);
+    *px = from_fx(x, D.cneg != A.cneg);
+    *py = from_fx(y, D.cneg != A.sneg);
+    *pz = from_fx(D.s, D.sneg);
+}
+
 // Float64 basis of an A source (east/north of the index frame).
 struct A64 {
     double sa, ca, sd, cd;  // sin/cos of RA and Dec
@@ -359,11 +478,28 @@ struct A64 {
     double a, b;
 };
 
-__device__ __forceinline__ A64 make_a64(const ACold& A) {
+// A rotated position's degrees are its angle divided by kDeg, which is short of
+// pi / 180 by 1.7e-17 of itself: with `rotated` the turns are scaled back by as
+// much (at 360 degrees it is 2e-11 arcsec, as much as all the rest of a
+// separation's error).
+__device__ __forceinline__ A64 make_a64(const ACold& A, bool rotated) {
     A64 r;
-    sincos(A.lon * kDeg, &r.sa, &r.ca);
-    sincos(A.lat * kDeg, &r.sd, &r.cd);
-    sincos(A.theta, &r.st, &r.ct);
+    uint64_t fl = lon_turn(A.lon), fb = lat_turn(A.lat);
+    if (rotated) {
+        constexpr uint32_t kShort = 312;  // 2^64 * (1 - kDeg * 180 / pi)
+        fl -= (fl >> 32) * kShort >> 32;
+        const int64_t sb = (int64_t)fb;
+        fb -= (uint64_t)((sb >> 32) * (int64_t)kShort >> 32);
+    }
+    const SinCosFx L = sincos_turn(fl), D = sincos_turn(fb);
+    r.sa = from_fx(L.s, L.sneg);
+    r.ca = from_fx(L.c, L.cneg);
+    r.sd = from_fx(D.s, D.sneg);
+    r.cd = from_fx(D.c, D.cneg);
+    // (no angle -- a circle -- needs no evaluation)
+    r.st = 0.0;
+    r.ct = 1.0;
+    if (((uint64_t)__double_as_longlong(A.theta) << 1) != 0) sincos(A.theta, &r.st, &r.ct);
     r.a = A.a;
     r.b = A.b;
     return r;
@@ -437,15 +573,25 @@ __device__ __forceinline__ double norm64(const A64& A, int shape, double px, dou
     return k * fmax(fabs(X) / A.a, fabs(Y) / A.b);
 }
 
-// Float64 unit vector of a position given in degrees.
-__device__ __forceinline__ void unit64_deg(double lon, double lat, double* px, double* py,
+// Float64 unit vector of a position given in degrees (out of line: many
+// registers, and rare except where float64 unit vectors are stored).
+static __device__ __noinline__ void unit64_deg(double lon, double lat, double* px, double* py,
                                            double* pz) {
-    double sa, ca, sd, cd;
-    sincos(lon * kDeg, &sa, &ca);
-    sincos(lat * kDeg, &sd, &cd);
-    *px = cd * ca;
-    *py = cd * sa;
-    *pz = sd;
+    unit64_turn(lon_turn(lon), lat_turn(lat), px, py, pz);
+}
+
+// Float64 unit vector of B row `row` (exact positions are kept by row).
+__device__ __forceinline__ void load_p64(const IndexGeom& G, int32_t row, double* x, double* y,
+                                         double* z) {
+    if (G.p64) {  // one 32-byte sector
+        const double2 xy = __ldg(G.p64 + 2 * (int64_t)row);
+        *x = xy.x;
+        *y = xy.y;
+        *z = __ldg(G.p64 + 2 * (int64_t)row + 1).x;
+    } else {
+        const double2 p = G.pos[row];
+        unit64_deg(p.x, p.y, x, y, z);
+    }
 }
 
 // ---------------------------------------------------------------- host side
@@ -614,7 +760,7 @@ struct xm_index {
     int32_t nz;
     xm::BRec* rec;
     double2* pos;
-    double *px, *py, *pz;
+    double2* p64;
     int64_t* id;
     xm::ZoneHot* zhot;
     uint32_t* lut;
@@ -623,7 +769,7 @@ struct xm_index {
     int32_t* build_err;  // error bits of a build whose check was deferred (else NULL)
     cudaStream_t stream;  // the stream it was built on (its memory is freed in its order)
     xm::IndexGeom geom() const {
-        return xm::IndexGeom{rec, pos, px, py, pz, zhot, lut, nz, h, (float)h};
+        return xm::IndexGeom{rec, pos, p64, zhot, lut, nz, h, (float)h};
     }
 };
 

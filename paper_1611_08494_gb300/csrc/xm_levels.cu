@@ -72,7 +72,9 @@ __global__ void k_lvl_a64(const ACold* __restrict__ acold, int64_t n, const int3
     LvA L;
     L.lon = C.lon;
     L.lat = C.lat;
-    sincospi(C.lat * (1.0 / 180.0), &L.sd, &L.cd);  // degrees reduced exactly
+    const SinCosFx sc = sincos_turn(lat_turn(C.lat));
+    L.sd = from_fx(sc.s, sc.sneg);
+    L.cd = from_fx(sc.c, sc.cneg);
     sincos(C.theta, &L.st, &L.ct);
     L.a = C.a;
     L.b = C.b;
@@ -145,7 +147,9 @@ __global__ void k_lvl_pair(IndexGeom G, const LvA* __restrict__ a64,
     }
     if (!near) {  // from B's unit vector and A's full basis
         A64 A;
-        sincospi(L.lon * (1.0 / 180.0), &A.sa, &A.ca);
+        const SinCosFx sc = sincos_turn(lon_turn(L.lon));
+        A.sa = from_fx(sc.s, sc.sneg);
+        A.ca = from_fx(sc.c, sc.cneg);
         A.sd = L.sd;
         A.cd = L.cd;
         A.st = L.st;
@@ -153,18 +157,7 @@ __global__ void k_lvl_pair(IndexGeom G, const LvA* __restrict__ a64,
         A.a = L.a;
         A.b = L.b;
         double px, py, pz;
-        if (G.px) {
-            px = G.px[row];
-            py = G.py[row];
-            pz = G.pz[row];
-        } else {
-            double sl, cl, sb, cb;
-            sincospi(q.x * (1.0 / 180.0), &sl, &cl);
-            sincospi(q.y * (1.0 / 180.0), &sb, &cb);
-            px = cb * cl;
-            py = cb * sl;
-            pz = sb;
-        }
+        load_p64(G, row, &px, &py, &pz);
         d = norm64(A, shape, px, py, pz);
     }
     dist[p] = d;

@@ -54,18 +54,11 @@ __global__ void k_pick_cont(const int64_t* __restrict__ pb, const double* __rest
 __device__ __forceinline__ double sep64_of(const IndexGeom& G, const ACold* __restrict__ acold,
                                            const int32_t* __restrict__ a_slot, int64_t a,
                                            int64_t b) {
-    const ACold& C = acold[a_slot ? a_slot[a] : a];
-    const A64 A = make_a64(C);
+    ACold C = acold[a_slot ? a_slot[a] : a];
+    C.theta = 0.0;  // (the separation does not depend on the orientation)
+    const A64 A = make_a64(C, false);
     double px, py, pz, rho;
-    const int32_t row = (int32_t)b;
-    if (G.px) {
-        px = G.px[row];
-        py = G.py[row];
-        pz = G.pz[row];
-    } else {
-        const double2 q = G.pos[row];
-        unit64_deg(q.x, q.y, &px, &py, &pz);
-    }
+    load_p64(G, (int32_t)b, &px, &py, &pz);
     test64(A, XM_CIRCLE, px, py, pz, &rho);
     return rho * kRadToArcsec;
 }

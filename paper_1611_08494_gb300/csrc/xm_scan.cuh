@@ -223,6 +223,7 @@ __device__ __forceinline__ void prep_at(const AIn& I, int64_t i, double lon0, do
     }
     make_aprep(lon, lat, gamma, ok, a, b, pa, I.shape, I.pa_dir, I.size_k, I.pa_zero, I.nz, I.h_f,
                (int32_t)i, P, C);
+    if (I.rotate) P->shape |= kRotated;
 }
 
 __device__ __forceinline__ void prep_one(const AIn& I, int64_t i, int32_t* err, APrep* P,
@@ -369,19 +370,6 @@ __device__ __forceinline__ void bucket_bounds(const IndexGeom& G, const ZoneHot&
     const uint32_t bh = min((khi - Z.lut_kmin) >> shift, last);
     *lo_out = __ldg(&L[bl]);
     *hi_out = __ldg(&L[bh + 1]);
-}
-
-// Float64 unit vector of B row `row` (exact positions are kept by row).
-__device__ __forceinline__ void load_p64(const IndexGeom& G, int32_t row, double* x, double* y,
-                                         double* z) {
-    if (G.px) {
-        *x = G.px[row];
-        *y = G.py[row];
-        *z = G.pz[row];
-    } else {
-        const double2 p = G.pos[row];
-        unit64_deg(p.x, p.y, x, y, z);
-    }
 }
 
 __device__ __forceinline__ void warp_add(unsigned long long* dst, uint32_t v) {
@@ -625,7 +613,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan(ScanArgs P) {
         const bool s64 = PREC == kPrecFP64 || MODE == kModeResolve ||
                          W.esep[lane] * 206264.8f > 9e-5f;
         W.sep64[lane] = s64;
-        if (s64 && A.R > 0.0f) W.ac[lane].a64 = make_a64(FUSED ? C : P.Ac[s_me]);
+        if (s64 && A.R > 0.0f) W.ac[lane].a64 = make_a64(FUSED ? C : P.Ac[s_me], A.shape & kRotated);
         else if (FUSED) W.ac[lane].cold = C;
         W.m1[lane] = kKeyInf;
         W.m2[lane] = kKeyInf;
@@ -748,7 +736,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan(ScanArgs P) {
                 bool maybe = true, band = false, in32 = false;
                 if (PREC == kPrecFP32) {
                     // q <= 1 - g: inside; q > 1 + g: outside; between: float64
-                    const float q = q32(A, A.shape, get_t(W.it_t, k), b, &x, &y);
+                    const float q = q32(A, A.shape & ~kRotated, get_t(W.it_t, k), b, &x, &y);
                     const float g = W.g[al];
                     maybe = q <= 1.0f + g;
                     if (maybe) {
@@ -764,14 +752,15 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan(ScanArgs P) {
                     const A64* a64 = &W.ac[al].a64;
                     if (!s64) {  // band recheck of a float32-path source
                         if (a_own_for != al) {
-                            a_own = make_a64(FUSED ? W.ac[al].cold : P.Ac[W.sidx[al]]);
+                            a_own = make_a64(FUSED ? W.ac[al].cold : P.Ac[W.sidx[al]],
+                                             A.shape & kRotated);
                             a_own_for = al;
                         }
                         a64 = &a_own;
                     }
                     double px, py, pz, rho;
                     load_p64(G, b.row, &px, &py, &pz);
-                    const bool in = test64(*a64, A.shape, px, py, pz, &rho);
+                    const bool in = test64(*a64, A.shape & ~kRotated, px, py, pz, &rho);
                     n_flip += band && in != in32;
                     is_mem = in;
                     exact = rho * kRadToArcsec;
@@ -972,19 +961,11 @@ constexpr size_t kSrcSmem = sizeof(SrcWarpSmem) * kScanWarps;
 
 // The float64 decision of a candidate in the guard band (rare), out of line
 // so its registers are not held across the record loop.
-__device__ __noinline__ bool recheck64(const ACold* C, int shape, const double2* pos,
-                                       const double* ux, const double* uy, const double* uz,
+__device__ __noinline__ bool recheck64(const ACold* C, int shape, bool rotated, const IndexGeom* G,
                                        int32_t row) {
-    const A64 a64 = make_a64(*C);
+    const A64 a64 = make_a64(*C, rotated);
     double px, py, pz, rho;
-    if (ux) {
-        px = ux[row];
-        py = uy[row];
-        pz = uz[row];
-    } else {
-        const double2 p = pos[row];
-        unit64_deg(p.x, p.y, &px, &py, &pz);
-    }
+    load_p64(*G, row, &px, &py, &pz);
     return test64(a64, shape, px, py, pz, &rho);
 }
 
@@ -1155,11 +1136,11 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_
                     }
                     n_cand++;
                     float x, y;
-                    const float q = q32(A, A.shape, T, b, &x, &y);
+                    const float q = q32(A, I.shape, T, b, &x, &y);
                     if (q <= 1.0f + A.g) {
                         bool in = true;
                         if (q >= 1.0f - A.g) {  // the guard band: decided in float64
-                            in = recheck64(&W.cold[lane], A.shape, G.pos, G.px, G.py, G.pz, b.row);
+                            in = recheck64(&W.cold[lane], I.shape, I.rotate, &G, b.row);
                             atomicAdd(&P.stats[1], 1ull);
                             if (in != (q <= 1.0f)) atomicAdd(&P.stats[2], 1ull);
                         }
