@@ -282,7 +282,10 @@ xm_status xm_pending::begin() {
     R->n_b = X->n;
     // per-A outputs
     R->count = (int32_t*)dev_alloc(nn * sizeof(int32_t), s);
-    R->pair_off = (int64_t*)dev_alloc(nn * sizeof(int64_t), s);
+    // (the tiles' sums of a large count follow the offsets)
+    const int64_t sum_words = count_scan_words(nA);
+    R->pair_off = (int64_t*)dev_alloc((nn + sum_words) * sizeof(int64_t), s);
+    R->zeros = R->pair_off && sum_words ? R->pair_off + nn : nullptr;
     if (sel & XM_SEL_BEST) {
         R->best_b = (int64_t*)dev_alloc(nn * (sizeof(int64_t) + sizeof(double)), s);
         R->best_sep = R->best_b ? (double*)(R->best_b + nn) : nullptr;
@@ -431,7 +434,8 @@ xm_status xm_pending::begin() {
         r = launch_scan_any(prec, cq, kModeCount, nA, s);
     }
     if (r != XM_OK) return r;
-    r = exclusive_scan_i32(R->count, R->pair_off, nA, total, err, s);
+    r = R->zeros ? count_scan(R->count, R->pair_off, nA, total, R->zeros, s)
+                 : exclusive_scan_i32(R->count, R->pair_off, nA, total, err, s);
     if (r != XM_OK) return r;
 
     // the counts go to the host first; the side stream (float64 best pairs)

@@ -386,21 +386,25 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_scan(const T* __restrict_
 // Elements move between global memory and the threads through shared memory
 // (padded by one word per thread's run), so every global load and store is
 // warp-contiguous while each thread scans kScanItems consecutive elements.
+// CHAIN false: the sums of the tiles before are known (tile_offs).
 __device__ __forceinline__ int scan_pad(int e) { return e + (e >> 4); }
 
-template <typename T>
+template <typename T, bool CHAIN>
 __global__ void __launch_bounds__(kScanThreads) k_scan_chained(
     const T* __restrict__ in, int64_t n, int64_t* __restrict__ out, int64_t* __restrict__ total,
-    uint64_t* status, unsigned int* tile_counter, int32_t* err) {
+    const int64_t* __restrict__ tile_offs, uint64_t* status, unsigned int* tile_counter,
+    int32_t* err) {
     pdl_wait();
     static_assert(kScanItems == 16, "one pad word per 16 elements");
     __shared__ int64_t xs[kScanTile + kScanTile / 16];
     __shared__ int64_t warp_tot[kScanThreads / 32];
     __shared__ int64_t tile_prefix;
     __shared__ unsigned int tile_s;
-    if (threadIdx.x == 0) tile_s = atomicAdd(tile_counter, 1u);
-    __syncthreads();
-    const int64_t tile = tile_s;
+    if (CHAIN) {
+        if (threadIdx.x == 0) tile_s = atomicAdd(tile_counter, 1u);
+        __syncthreads();
+    }
+    const int64_t tile = CHAIN ? tile_s : blockIdx.x;
     const int64_t tbase = tile * kScanTile;
 #pragma unroll
     for (int k = 0; k < kScanItems; k++) {
@@ -431,7 +435,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_chained(
         all += warp_tot[w];
     }
     if (warp == 0) {
-        const int64_t prefix = lookback_warp(status, tile, all, kSpinLimit, false, err);
+        const int64_t prefix =
+            CHAIN ? lookback_warp(status, tile, all, kSpinLimit, false, err) : tile_offs[tile];
         if (lane == 0) {
             tile_prefix = prefix;
             if (total && (tile + 1) * kScanTile >= n) *total = prefix + all;
@@ -450,6 +455,79 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_chained(
         const int e = k * kScanThreads + threadIdx.x;
         if (tbase + e < n) out[tbase + e] = xs[scan_pad(e)];
     }
+}
+
+// Sums of tiles of kScanTile counts, and the zeros of each kCountTile of them
+// (the unmatched sources of a join's tile).
+constexpr int kZeroTiles = kScanTile / kCountTile;
+__global__ void __launch_bounds__(kScanThreads) k_count_sums(const int32_t* __restrict__ in, int64_t n,
+                                                             int64_t* __restrict__ sums,
+                                                             int64_t* __restrict__ zeros) {
+    pdl_wait();
+    __shared__ uint32_t z[kZeroTiles];
+    if (threadIdx.x < kZeroTiles) z[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * kScanTile;
+    int64_t v = 0;
+    uint32_t nz[kZeroTiles] = {};
+#pragma unroll
+    for (int k = 0; k < kScanItems; k++) {
+        const int64_t i = base + (int64_t)k * kScanThreads + threadIdx.x;
+        const int32_t c = i < n ? in[i] : -1;
+        if (c > 0) v += c;
+        nz[k / (kScanItems / kZeroTiles)] += c == 0;
+    }
+#pragma unroll
+    for (int h = 0; h < kZeroTiles; h++) {
+        const uint32_t s = __reduce_add_sync(0xffffffffu, nz[h]);
+        if ((threadIdx.x & 31) == 0 && s) atomicAdd(&z[h], s);
+    }
+    const int64_t t = block_sum<int64_t>(v);  // (its barrier covers z)
+    if (threadIdx.x == 0) sums[blockIdx.x] = t;
+    if (threadIdx.x < kZeroTiles) zeros[(int64_t)blockIdx.x * kZeroTiles + threadIdx.x] = z[threadIdx.x];
+}
+
+// Exclusive prefix sums of two arrays in place, a block each.
+__global__ void __launch_bounds__(1024) k_scan_sums(int64_t* a, int64_t na, int64_t* b, int64_t nb,
+                                                    int64_t* total) {
+    pdl_wait();
+    __shared__ int64_t warp_tot[32];
+    int64_t* const v = blockIdx.x ? b : a;
+    const int64_t n = blockIdx.x ? nb : na;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int64_t run = 0;
+    constexpr int kItems = 8;
+    for (int64_t i0 = 0; i0 < n; i0 += kItems * 1024) {
+        int64_t x[kItems], sum = 0;
+        const int64_t i = i0 + kItems * threadIdx.x;
+#pragma unroll
+        for (int k = 0; k < kItems; k++) {
+            x[k] = i + k < n ? v[i + k] : 0;
+            sum += x[k];
+        }
+        int64_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) warp_tot[warp] = incl;
+        __syncthreads();
+        int64_t before = 0, all = 0;
+        for (int w = 0; w < 32; w++) {
+            if (w < warp) before += warp_tot[w];
+            all += warp_tot[w];
+        }
+        int64_t at = run + before + incl - sum;
+#pragma unroll
+        for (int k = 0; k < kItems; k++) {
+            if (i + k < n) v[i + k] = at;
+            at += x[k];
+        }
+        run += all;
+        __syncthreads();
+    }
+    if (total && blockIdx.x == 0 && threadIdx.x == 0) *total = run;
 }
 
 template <typename T>
@@ -477,8 +555,8 @@ xm_status scan_impl(const T* in, int64_t* out, int64_t n, int64_t* total, int32_
     if (e != cudaSuccess) st = cuda_fail(e, "scan memset");
     if (st == XM_OK) {
         launch_begin("k_scan_chained", s);
-        launch_pdl(k_scan_chained<T>, dim3((unsigned)ntiles), dim3(kScanThreads), 0, s, in, n, out,
-                   total, status, counter, err);
+        launch_pdl(k_scan_chained<T, true>, dim3((unsigned)ntiles), dim3(kScanThreads), 0, s, in, n,
+                   out, total, (const int64_t*)nullptr, status, counter, err);
         e = launch_end("k_scan_chained", s);
         if (e != cudaSuccess) st = cuda_fail(e, "k_scan_chained");
     }
@@ -514,6 +592,22 @@ xm_status exclusive_scan_i32_ws(const int32_t* in, int64_t* out, int64_t n, int6
 xm_status exclusive_scan_i32(const int32_t* in, int64_t* out, int64_t n, int64_t* total,
                              int32_t* err, cudaStream_t s) {
     return scan_impl<int32_t>(in, out, n, total, err, s);
+}
+
+int64_t count_scan_words(int64_t n) {
+    return n >= kCountScanMin ? (1 + kZeroTiles) * ((n + kScanTile - 1) / kScanTile) : 0;
+}
+
+xm_status count_scan(const int32_t* count, int64_t* out, int64_t n, int64_t* total, int64_t* zeros,
+                     cudaStream_t s) {
+    const int64_t ntiles = (n + kScanTile - 1) / kScanTile;
+    int64_t* const sums = zeros + kZeroTiles * ntiles;
+    XM_LAUNCH("k_count_sums", (unsigned)ntiles, kScanThreads, 0, s, k_count_sums, count, n, sums, zeros);
+    XM_LAUNCH("k_scan_sums", 2, 1024, 0, s, k_scan_sums, sums, ntiles, zeros, kZeroTiles * ntiles, total);
+    XM_LAUNCH("k_scan_chained", (unsigned)ntiles, kScanThreads, 0, s, (k_scan_chained<int32_t, false>),
+              count, n, out, (int64_t*)nullptr, sums, (uint64_t*)nullptr, (unsigned int*)nullptr,
+              (int32_t*)nullptr);
+    return XM_OK;
 }
 
 xm_status exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* total,

@@ -295,7 +295,9 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
     const int64_t na1 = n_a > 0 ? n_a : 1, nb1 = n_b > 0 ? n_b : 1;
     const bool want_best = (selection & XM_SEL_BEST) != 0;
     R->count = (int32_t*)dev_alloc(na1 * sizeof(int32_t), s);
-    R->pair_off = (int64_t*)dev_alloc(na1 * sizeof(int64_t), s);
+    const int64_t sum_words = count_scan_words(n_a);
+    R->pair_off = (int64_t*)dev_alloc((na1 + sum_words) * sizeof(int64_t), s);
+    R->zeros = R->pair_off && sum_words ? R->pair_off + na1 : nullptr;
     if (want_best) {
         R->best_b = (int64_t*)dev_alloc(na1 * (sizeof(int64_t) + sizeof(double)), s);
         R->best_sep = R->best_b ? (double*)(R->best_b + na1) : nullptr;
@@ -382,7 +384,9 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
         else if (n_a > 0)
             XM_LAUNCH("k_val_probe", grid_of(n_a), kBlock, 0, s, k_val_probe, ak, n_a, key_type,
                       codes, rows, n_b, V, R->count, first, R->best_b, R->best_sep);
-        xm_status r = exclusive_scan_i32(R->count, R->pair_off, n_a, (int64_t*)(small + 2), err, s);
+        xm_status r = R->zeros ? count_scan(R->count, R->pair_off, n_a, (int64_t*)(small + 2), R->zeros, s)
+                               : exclusive_scan_i32(R->count, R->pair_off, n_a, (int64_t*)(small + 2),
+                                                    err, s);
         if (r != XM_OK) return r;
         unsigned long long h[2] = {0, 0};
         e = cudaMemcpyAsync(h, small + 2, sizeof(h), cudaMemcpyDeviceToHost, s);
