@@ -588,7 +588,7 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
             if (e2 != cudaSuccess) return cuda_fail(e2, "batch memset");
             r = launch_persistent_any(prec, kModeEmit, b, pblocks, s);
             if (r != XM_OK) return r;
-            XM_LAUNCH("k_sort_small", grid_for(total), kBlock, 0, s, k_sort_small, B.count,
+            XM_LAUNCH("k_sort_small", grid_for(total), kBlock, 0, s, k_sort_small<1>, B.count,
                       B.pair_off, total, pair_cap, B.pb, B.ps, (const int32_t*)nullptr);
             XM_LAUNCH("k_sort_warp", (unsigned)(8 * sms), 32 * kWarpSortWarps, 0, s, k_sort_warp,
                       B.count, B.pair_off, total, pair_cap, B.pb, B.ps, (const int32_t*)nullptr);
