@@ -70,8 +70,8 @@ xm_status launch_scan_fused(int prec, const ScanArgs& a, int mode, int64_t n_uni
 // and a region of fixed size whose bounding radius is under 0.4 zone heights,
 // so a source meets at most two zones (sources with more items are left to
 // k_scan by the pass itself).
-bool sparse_scan(int prec, bool sorted_a, const xm_region* region, const xm_index* X) {
-    if (prec != XM_PREC_FP32_RECHECK || sorted_a || region->a_col || region->b_col) return false;
+bool sparse_scan(bool sorted_a, const xm_region* region, const xm_index* X) {
+    if (sorted_a || region->a_col || region->b_col) return false;
     const double k = region->size_scale * region->size_unit_arcsec * kArcsec;
     const double a = fabs(region->a) * k, b = fabs(region->b) * k;
     const double R = region->shape == XM_RECT     ? hypot(a, b)
@@ -80,7 +80,7 @@ bool sparse_scan(int prec, bool sorted_a, const xm_region* region, const xm_inde
     return R < 0.4 * X->h;
 }
 
-xm_status launch_scan_src(const ScanArgs& a, int32_t* defer, int32_t* n_defer, cudaStream_t s) {
+xm_status launch_scan_src(int prec, const ScanArgs& a, int32_t* defer, int32_t* n_defer, cudaStream_t s) {
     prepare_kernels();
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) == cudaSuccess)
@@ -88,7 +88,12 @@ xm_status launch_scan_src(const ScanArgs& a, int32_t* defer, int32_t* n_defer, c
     int64_t g = (a.nA + 32 * kScanWarps - 1) / (32 * kScanWarps);
     if (g > 8LL * sms) g = 8LL * sms;
     if (g < 1) g = 1;
-    XM_LAUNCH("k_scan_src", (unsigned)g, kScanThreads, kSrcSmem, s, k_scan_src, a, defer, n_defer);
+    if (prec == XM_PREC_FP32_RECHECK)
+        XM_LAUNCH("k_scan_src", (unsigned)g, kScanThreads, kSrcSmem<kPrecFP32>, s,
+                  k_scan_src<kPrecFP32>, a, defer, n_defer);
+    else
+        XM_LAUNCH("k_scan_src_fp64", (unsigned)g, kScanThreads, kSrcSmem<kPrecFP64>, s,
+                  k_scan_src<kPrecFP64>, a, defer, n_defer);
     return XM_OK;
 }
 
@@ -419,11 +424,11 @@ xm_status xm_pending::begin() {
     ScanArgs cq = a;
     cq.queue = (unsigned int*)(small + 4);
     xm_status r = XM_OK;
-    if (sparse_scan(prec, sorted_a, &region, X)) {
+    if (sparse_scan(sorted_a, &region, X)) {
         // one lane per source where regions are small against the zones,
         // then the warp-cooperative scan over the sources it left (their
         // number read on the device)
-        r = launch_scan_src(cq, lists + 3 * nn, small + 5, s);
+        r = launch_scan_src(prec, cq, lists + 3 * nn, small + 5, s);
         if (r != XM_OK) return r;
         ScanArgs cd = cq;
         cd.list = lists + 3 * nn;

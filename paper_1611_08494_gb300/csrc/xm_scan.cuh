@@ -15,6 +15,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include <mutex>
 #include <new>
 
@@ -928,53 +930,84 @@ constexpr size_t kScanSmem = sizeof(ScanWarpSmem) * kScanWarps;
 // ------------------------------------------------ the sparse count pass
 //
 // The count pass for regions that are small against the zone height, where a
-// source meets one or two zone items and a few records (the all-sky case):
-// one lane per source from its preparation to its results, with the running
-// state in registers instead of the flattened item and candidate rounds of
-// k_scan. A lane finds its items' bucket ranges at once; then the warp steps
-// through the lanes' records together, one record per lane and step (the next
-// one loaded while this one is tested), so the step's members can be staged
-// in shared memory and written to the record arena with one atomic per warp
-// and stage. The best-pair fold and the member indices are the count pass's
-// (sequential per source, the same minimum, second minimum and lowest-row
-// tie). Sources outside this shape -- more than two items, more than
-// kSrcMaxRec records in their ranges, or float64 separations -- are listed
+// source meets one or two zone items and a few records (the all-sky case).
+// A warp takes 32 sources. Each lane prepares its own and finds its items'
+// bucket ranges at once; the records of all of them are then loaded together,
+// 64 per round, flattened over the lanes, and those whose key lies in their
+// item's window -- one in seven of an all-sky match -- are queued as
+// candidates. The queue is tested 32 at a time, a candidate per lane, and its
+// members, which stay in the order of their sources, are folded by the lane of
+// each source and written to the record arena with one atomic per warp.
+// Sources outside this shape -- more than two items, more than kSrcMaxRec
+// records in their ranges, or (float32 path) float64 separations -- are listed
 // (`defer`) and counted by k_scan over the list afterwards, in the same
 // outputs.
+// Bound by the latency of a chunk's dependent loads (position, zone, bucket
+// table, records), which 24 warps an SM overlap; testing every record where it
+// lay, a lane per source, took eight to ten divergent rounds instead of the
+// one. 3.5 ms for 5e7 sources against 2e8 (4.8 before), 0.73 for 1e7 against
+// 1e8 (0.99); float64, 5e6 against 2e7: 0.51 ms and 0.07 for the rest (1.17
+// with k_scan alone). Six blocks an SM with two rounds in flight: the shared
+// memory of seven or eight, or of four rounds, leaves the L1 too small for the
+// zones' records (3.6 to 5.6 ms).
 
 constexpr int kSrcMaxRec = 48;  // records a lane takes on; more go to k_scan
-constexpr int kSrcStage = 64;   // member records staged per warp
+constexpr int kSrcStage = 64;   // members staged
+constexpr int kSrcRounds = 2;   // rounds of 32 records in flight
+constexpr int kSrcQueue = 128;  // candidates queued (a power of two)
+static_assert(kSrcQueue >= 31 + 32 * kSrcRounds, "a round's records fit the queue");
 
-constexpr int kSrcBuf = 128;    // records of a chunk loaded together
-
-struct SrcWarpSmem {
-    BRec buf[kSrcBuf];  // the chunk's records, lane after lane
-    MemberRec rec[kSrcStage];
-    ACold cold[32];  // float64 part of each lane's source
-    int32_t first[33];       // first record of each lane in buf (prefix)
-    int32_t lo0[32], lo1[32], n0[32];  // each lane's rows
-    uint8_t who[kSrcStage];  // lane of each staged record
-    int32_t drop[32];        // a member of the lane's source did not fit the arena
+struct SrcA32 {
+    uint64_t key64[32];
+    int32_t z[32];
+    float zfrac[32], m00[32], m01[32], m10[32], m11[32];
 };
 
-constexpr size_t kSrcSmem = sizeof(SrcWarpSmem) * kScanWarps;
+struct SrcA64 {
+    double sa[32], ca[32], sd[32], cd[32], st[32], ct[32];
+};
+
+template <int PREC>
+struct SrcWarpSmem {
+    BRec rec[kSrcQueue];
+    double lon[32], lat[32], theta[32];  // float64 part of each lane's source
+    // what the tests read of each lane's source
+    typename std::conditional<PREC == kPrecFP64, SrcA64, SrcA32>::type A;
+    typename std::conditional<PREC == kPrecFP64, long long, int32_t>::type key[kSrcStage];
+    int32_t row[kSrcStage];     // B row of each staged member
+    int32_t first[33];          // first record of each lane in the flattened order
+    int32_t lo0[32], lo1[32], n0[32], z[2][32];  // each lane's rows and zones
+    uint32_t klo[2][32], khi[2][32];             // and windows
+    int32_t mcnt[32];           // members staged for each lane
+    int32_t mk[32];             // index of a lane's first staged member, less its place
+    uint32_t drop;              // lanes of sources with a member that did not fit the arena
+    uint8_t own[kSrcQueue];     // candidate: lane of its source, + 32 for item 1
+    uint8_t who[kSrcStage];     // member: lane of its source
+};
+
+template <int PREC>
+constexpr size_t kSrcSmem = sizeof(SrcWarpSmem<PREC>) * kScanWarps;
 
 // The float64 decision of a candidate in the guard band (rare), out of line
 // so its registers are not held across the record loop.
-__device__ __noinline__ bool recheck64(const ACold* C, int shape, bool rotated, const IndexGeom* G,
-                                       int32_t row) {
-    const A64 a64 = make_a64(*C, rotated);
+__device__ __noinline__ bool recheck64(double lon, double lat, double theta, double a, double b,
+                                       int shape, bool rotated, const IndexGeom* G, int32_t row) {
+    const ACold C{lon, lat, theta, a, b};
+    const A64 a64 = make_a64(C, rotated);
     double px, py, pz, rho;
     load_p64(*G, row, &px, &py, &pz);
     return test64(a64, shape, px, py, pz, &rho);
 }
 
+template <int PREC>
 __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_t* defer,
                                                               int32_t* n_defer) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char src_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    SrcWarpSmem& W = reinterpret_cast<SrcWarpSmem*>(src_smem)[warp];
+    SrcWarpSmem<PREC>& W = reinterpret_cast<SrcWarpSmem<PREC>*>(src_smem)[warp];
+    using Key = typename std::conditional<PREC == kPrecFP64, long long, int32_t>::type;
+    constexpr Key kInf = PREC == kPrecFP64 ? (Key)kKeyInf : (Key)0x7F800000;
     const IndexGeom& G = P.G;
     const uint32_t lt_mask = (1u << lane) - 1u;
     uint32_t n_cand = 0, n_mem = 0;
@@ -987,6 +1020,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_
     const bool same_region = !I.rotate || I.shape == XM_CIRCLE;
     __shared__ APrep s_at;
     __shared__ ACold s_ct;
+    __shared__ double s_st, s_cos;
     if (threadIdx.x == 0) {
         const double b = I.shape == XM_CIRCLE ? I.a : I.b;
         APrep at;
@@ -995,32 +1029,40 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_
                    I.h_f, 0, &at, &ct);
         s_at = at;
         s_ct = ct;
+        if (PREC == kPrecFP64) {
+            const A64 t = make_a64(ct, false);
+            s_st = t.st;
+            s_cos = t.ct;
+        }
         if (blockIdx.x == 0 && P.nA > 0 && !size_ok(I.a, b, I.pa)) atomicOr(P.err, kErrSize);
     }
+    W.mcnt[lane] = 0;
     __syncthreads();
-    // chunks from the queue, the next one claimed while this one runs
+    // chunks from the queue, the next one claimed while this one runs, and
+    // its positions loaded
     unsigned int next = 0;
     if (lane == 0) next = atomicAdd(P.queue, 1u);
-    for (;;) {
-        const int64_t this_first = (int64_t)__shfl_sync(0xffffffffu, next, 0) * 32;
-        if (this_first >= P.nA) break;  // whole warp
+    int64_t this_first = (int64_t)__shfl_sync(0xffffffffu, next, 0) * 32;
+    double lon0 = 0.0, lat0 = 0.0;
+    if (this_first + lane < P.nA) {
+        lon0 = I.lon[this_first + lane];
+        lat0 = I.lat[this_first + lane];
+    }
+    while (this_first < P.nA) {  // whole warp
         if (lane == 0) next = atomicAdd(P.queue, 1u);
-        W.drop[lane] = 0;
+        if (lane == 0) W.drop = 0;
 
         // ---- preparation, window and bucket ranges (lane = source)
-        APrep A;
         bool mine = false;  // this lane's source is counted here
         int n0 = 0, nrec = 0;  // records of item 0, of both items
-        int32_t lo0 = 0, lo1 = 0;  // first rows (rows fit 31 bits)
-        uint32_t klo0 = 0, khi0 = 0, klo1 = 0, khi1 = 0;
-        int32_t z0 = 0, z1 = 0;
         if (this_first + lane < P.nA) {
             const int64_t s = this_first + lane;
+            APrep A;
             ACold C;
             if (same_region) {
                 double lon, lat, gamma;
                 bool ok;
-                a_position_of(I.lon[s], I.lat[s], I.rotate, I.rot, &lon, &lat, &gamma, &ok);
+                a_position_of(lon0, lat0, I.rotate, I.rot, &lon, &lat, &gamma, &ok);
                 if (!ok) atomicOr(P.err, kErrCoord);
                 const PosKey k = pos_key(lon, lat, I.nz);
                 A = s_at;
@@ -1033,14 +1075,26 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_
                     A.g = 0.0f;
                     A.m00 = A.m01 = A.m10 = A.m11 = 0.0f;
                 }
-                C = s_ct;
                 C.lon = lon;
                 C.lat = lat;
+                C.theta = s_ct.theta;
             } else {
-                prep_one(I, s, P.err, &A, &C);
+                prep_at(I, s, lon0, lat0, P.err, &A, &C);
             }
-            W.cold[lane] = C;
-            mine = 16.0f * kEps32 * (A.R + 2.0f * G.h_f) * 206264.8f <= 9e-5f;  // float32 separations
+            if constexpr (PREC != kPrecFP64) {
+                W.A.key64[lane] = A.key64;
+                W.A.z[lane] = A.z;
+                W.A.zfrac[lane] = A.zfrac;
+                W.A.m00[lane] = A.m00;
+                W.A.m01[lane] = A.m01;
+                W.A.m10[lane] = A.m10;
+                W.A.m11[lane] = A.m11;
+            }
+            W.lon[lane] = C.lon;
+            W.lat[lane] = C.lat;
+            W.theta[lane] = C.theta;
+            // (float32 separations, on that path)
+            mine = PREC == kPrecFP64 || 16.0f * kEps32 * (A.R + 2.0f * G.h_f) * 206264.8f <= 9e-5f;
             if (mine && A.R > 0.0f) {
                 const Window w = a_window(A, G);
                 const int items = (w.z1 - w.z0 + 1) * w.nseg;
@@ -1049,159 +1103,243 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_
                 } else {
                     // item 0: (z0, segment 0); item 1: the next zone, or the
                     // second segment of the same zone
-                    z0 = w.z0;
-                    z1 = w.nseg == 2 ? w.z0 : w.z0 + 1;
-                    klo0 = w.lo[0];
-                    khi0 = w.hi[0];
-                    klo1 = w.lo[w.nseg - 1];
-                    khi1 = w.hi[w.nseg - 1];
+                    const int32_t z1 = w.nseg == 2 ? w.z0 : w.z0 + 1;
+                    const uint32_t klo1 = w.lo[w.nseg - 1], khi1 = w.hi[w.nseg - 1];
+                    W.z[0][lane] = w.z0;
+                    W.z[1][lane] = z1;
+                    W.klo[0][lane] = w.lo[0];
+                    W.khi[0][lane] = w.hi[0];
+                    W.klo[1][lane] = klo1;
+                    W.khi[1][lane] = khi1;
                     int64_t l0, h0, l1 = 0, h1 = 0;
                     if (items == 2) bucket_bounds(G, load_zone_hot(G.zhot + z1), klo1, khi1, &l1, &h1);
-                    bucket_bounds(G, load_zone_hot(G.zhot + z0), klo0, khi0, &l0, &h0);
+                    bucket_bounds(G, load_zone_hot(G.zhot + w.z0), w.lo[0], w.hi[0], &l0, &h0);
                     if ((h0 - l0) + (h1 - l1) > kSrcMaxRec) {
                         mine = false;
                     } else {
-                        lo0 = (int32_t)l0;
-                        lo1 = (int32_t)l1;
                         n0 = (int)(h0 - l0);
                         nrec = n0 + (int)(h1 - l1);
+                        W.lo0[lane] = (int32_t)l0;  // (rows fit 31 bits)
+                        W.lo1[lane] = (int32_t)l1;
                     }
                 }
             }
             if (!mine) defer[atomicAdd(n_defer, 1)] = (int32_t)s;
         }
+        const int64_t next_first = (int64_t)__shfl_sync(0xffffffffu, next, 0) * 32;
+        if (next_first + lane < P.nA) {
+            lon0 = I.lon[next_first + lane];
+            lat0 = I.lat[next_first + lane];
+        }
 
-        // ---- records: the warp loads the chunk's records together (32 per
-        // round, flattened over the lanes, so their loads are in flight at
-        // once) into shared memory, kSrcBuf at most; then every lane tests
-        // its own, a step per record (records past the buffer are read from
-        // memory). Keys are the bit patterns of the float32 separations
-        // (non-negative, so ordered as integers).
-        if (!mine) nrec = 0;
         int incl = nrec;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int t = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += t;
         }
-        const int my_first = incl - nrec;
         const int total = __shfl_sync(0xffffffffu, incl, 31);
-        W.first[lane] = my_first;
+        W.first[lane] = incl - nrec;
         if (lane == 31) W.first[32] = total;
-        W.lo0[lane] = lo0;
-        W.lo1[lane] = lo1;
         W.n0[lane] = n0;
-        __syncwarp();
-        const int nbuf = min(total, kSrcBuf);
-        for (int c = lane; c < nbuf; c += 32) {
-            int ol = 0;  // last lane whose first record is <= c
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1)
-                if (W.first[ol + step] <= c) ol += step;
-            const int jj = c - W.first[ol];
-            const int32_t row = jj < W.n0[ol] ? W.lo0[ol] + jj : W.lo1[ol] + (jj - W.n0[ol]);
-            W.buf[c] = load_brec(G.rec + row);
+        if constexpr (PREC == kPrecFP64) if (nrec > 0) {
+            const ACold C{W.lon[lane], W.lat[lane], same_region ? 0.0 : W.theta[lane], 0.0, 0.0};
+            const A64 t = make_a64(C, I.rotate);
+            W.A.sa[lane] = t.sa;
+            W.A.ca[lane] = t.ca;
+            W.A.sd[lane] = t.sd;
+            W.A.cd[lane] = t.cd;
+            W.A.st[lane] = same_region ? s_st : t.st;
+            W.A.ct[lane] = same_region ? s_cos : t.ct;
         }
         __syncwarp();
+
+        // Keys are the bit patterns of the separations (non-negative, so
+        // ordered as integers): float32 radians, or float64 arcseconds.
         int cnt = 0;
-        int32_t m1 = 0x7F800000, m2 = 0x7F800000;  // smallest and second smallest key
+        Key m1 = kInf, m2 = kInf;  // smallest and second smallest
         int32_t b1 = 0x7fffffff;
-        int j = 0, cur = -1;
-        ItemTerms T;
-        int staged = 0;  // (warp-uniform)
-        auto flush = [&]() {
-            __syncwarp();
-            unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(P.arena_n, (unsigned long long)staged);
-            base = __shfl_sync(0xffffffffu, base, 0);
-            for (int i = lane; i < staged; i += 32) {
-                if ((long long)(base + i) < P.arena_cap) P.arena[base + i] = W.rec[i];
-                else W.drop[W.who[i]] = 1;
-            }
-            staged = 0;
-            __syncwarp();
-        };
-        while (__any_sync(0xffffffffu, j < nrec)) {
-            int32_t key = -1, brow = 0;  // key >= 0: the record is a member
-            if (j < nrec) {
-                const int it = j < n0 ? 0 : 1;
-                const BRec b = my_first + j < kSrcBuf ? W.buf[my_first + j]
-                                                      : load_brec(G.rec + (it ? lo1 + (j - n0) : lo0 + j));
-                j++;
-                if (b.ra_key >= (it ? klo1 : klo0) && b.ra_key <= (it ? khi1 : khi0)) {
-                    if (it != cur) {
-                        cur = it;
-                        const int32_t z = it ? z1 : z0;
-                        T = item_terms(A, load_zone_hot(G.zhot + z), z, G.h_f);
+        int c0 = 0, head = 0, tail = 0, nm = 0;  // (warp-uniform)
+        while (c0 < total || tail > head) {
+            // ---- records, their keys against their windows (lane = record)
+            if (c0 < total && tail - head < 32) {
+                BRec b[kSrcRounds];
+                int ol[kSrcRounds];
+#pragma unroll
+                for (int k = 0; k < kSrcRounds; k++) {
+                    const int c = c0 + 32 * k + lane;
+                    ol[k] = 0;  // last lane whose first record is <= c, + 32 for item 1
+                    if (c < total) {
+                        int l = 0;
+#pragma unroll
+                        for (int step = 16; step > 0; step >>= 1)
+                            if (W.first[l + step] <= c) l += step;
+                        const int jj = c - W.first[l], n = W.n0[l];
+                        const int it = jj >= n;
+                        b[k] = load_brec(G.rec + (it ? W.lo1[l] + (jj - n) : W.lo0[l] + jj));
+                        ol[k] = l + 32 * it;
                     }
-                    n_cand++;
+                }
+#pragma unroll
+                for (int k = 0; k < kSrcRounds; k++) {
+                    const bool in = c0 + 32 * k + lane < total &&
+                                    b[k].ra_key >= (&W.klo[0][0])[ol[k]] &&
+                                    b[k].ra_key <= (&W.khi[0][0])[ol[k]];
+                    const uint32_t mm = __ballot_sync(0xffffffffu, in);
+                    if (in) {
+                        const int q = (tail + __popc(mm & lt_mask)) & (kSrcQueue - 1);
+                        W.rec[q] = b[k];
+                        W.own[q] = (uint8_t)ol[k];
+                        n_cand++;
+                    }
+                    tail += __popc(mm);
+                }
+                c0 += 32 * kSrcRounds;
+                __syncwarp();
+                if (c0 < total && tail - head < 32) continue;
+            }
+            // ---- candidates (lane = candidate)
+            const int n = min(32, tail - head);
+            Key key = -1;  // >= 0: the record is a member
+            int32_t brow = 0;
+            int l = 0;
+            if (lane < n) {
+                const int q = (head + lane) & (kSrcQueue - 1);
+                const BRec b = W.rec[q];
+                const int own = W.own[q];
+                l = own & 31;
+                brow = b.row;
+                if constexpr (PREC == kPrecFP64) {
+                    A64 a64;
+                    a64.sa = W.A.sa[l];
+                    a64.ca = W.A.ca[l];
+                    a64.sd = W.A.sd[l];
+                    a64.cd = W.A.cd[l];
+                    a64.st = W.A.st[l];
+                    a64.ct = W.A.ct[l];
+                    a64.a = s_ct.a;
+                    a64.b = s_ct.b;
+                    double px, py, pz, rho;
+                    load_p64(G, brow, &px, &py, &pz);
+                    if (test64(a64, I.shape, px, py, pz, &rho))
+                        key = (Key)__double_as_longlong(rho * kRadToArcsec);
+                } else {
+                    APrep A;
+                    A.key64 = W.A.key64[l];
+                    A.z = W.A.z[l];
+                    A.zfrac = W.A.zfrac[l];
+                    A.m00 = W.A.m00[l];
+                    A.m01 = W.A.m01[l];
+                    A.m10 = W.A.m10[l];
+                    A.m11 = W.A.m11[l];
+                    A.g = s_at.g;  // (of every valid source: one size)
+                    const int32_t z = (&W.z[0][0])[own];
+                    const ItemTerms T = item_terms(A, load_zone_hot(G.zhot + z), z, G.h_f);
                     float x, y;
-                    const float q = q32(A, I.shape, T, b, &x, &y);
-                    if (q <= 1.0f + A.g) {
+                    const float q32v = q32(A, I.shape, T, b, &x, &y);
+                    if (q32v <= 1.0f + A.g) {
                         bool in = true;
-                        if (q >= 1.0f - A.g) {  // the guard band: decided in float64
-                            in = recheck64(&W.cold[lane], I.shape, I.rotate, &G, b.row);
+                        if (q32v >= 1.0f - A.g) {  // the guard band: decided in float64
+                            in = recheck64(W.lon[l], W.lat[l], W.theta[l], s_ct.a, s_ct.b, I.shape,
+                                           I.rotate, &G, b.row);
                             atomicAdd(&P.stats[1], 1ull);
-                            if (in != (q <= 1.0f)) atomicAdd(&P.stats[2], 1ull);
+                            if (in != (q32v <= 1.0f)) atomicAdd(&P.stats[2], 1ull);
                         }
                         if (in) {
                             const float s2 = fmaf(x, x, y * y);
                             const float rho32 = s2 < 1e-6f ? sqrtf(s2) * fmaf(s2, 1.0f / 6.0f, 1.0f)
                                                            : asinf(sqrtf(s2));
-                            key = __float_as_int(rho32);
-                            brow = b.row;
-                            n_mem++;
-                            cnt++;
-                            if (key < m1 || (key == m1 && brow < b1)) {
-                                m2 = m1;
-                                m1 = key;
-                                b1 = brow;
-                            } else {
-                                m2 = min(m2, key);
-                            }
+                            key = (Key)__float_as_int(rho32);
                         }
                     }
                 }
             }
-            if (P.arena) {
-                const uint32_t mm = __ballot_sync(0xffffffffu, key >= 0);
-                if (mm) {
-                    if (staged + __popc(mm) > kSrcStage) flush();
-                    if (key >= 0) {
-                        const int slot = staged + __popc(mm & lt_mask);
-                        MemberRec r;
-                        r.a_row = A.row;
-                        r.k = cnt - 1;
-                        r.b_row = brow;
-                        r.f32 = 1;
-                        r.sep = __longlong_as_double((long long)key);
-                        W.rec[slot] = r;
-                        W.who[slot] = (uint8_t)lane;
-                    }
-                    staged += __popc(mm);
+            head += n;
+            const uint32_t mm = __ballot_sync(0xffffffffu, key >= 0);
+            if (key >= 0) {
+                const int q = nm + __popc(mm & lt_mask);
+                W.key[q] = key;
+                W.row[q] = brow;
+                W.who[q] = (uint8_t)l;
+                atomicAdd(&W.mcnt[l], 1);
+                n_mem++;
+            }
+            nm += __popc(mm);
+            const bool last = c0 >= total && tail == head;
+            if (nm == 0 || !(last || nm > kSrcStage - 32)) continue;
+            // ---- members: to the arena, and each lane's folded
+            __syncwarp();
+            unsigned long long base = 0;
+            if (P.arena && lane == 0) base = atomicAdd(P.arena_n, (unsigned long long)nm);
+            const int mine_n = W.mcnt[lane];
+            int at = mine_n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, at, o);
+                if (lane >= o) at += t;
+            }
+            at -= mine_n;
+            W.mk[lane] = cnt - at;
+            W.mcnt[lane] = 0;
+            for (int j = at; j < at + mine_n; j++) {
+                const Key k = W.key[j];
+                const int32_t r = W.row[j];
+                if (k < m1 || (k == m1 && r < b1)) {
+                    m2 = m1;
+                    m1 = k;
+                    b1 = r;
+                } else {
+                    m2 = min(m2, k);
                 }
             }
+            cnt += mine_n;
+            __syncwarp();
+            if (P.arena) {
+                base = __shfl_sync(0xffffffffu, base, 0);
+                for (int j = lane; j < nm; j += 32) {
+                    const int w = W.who[j];
+                    if ((long long)(base + j) < P.arena_cap) {
+                        MemberRec r;
+                        r.a_row = (int32_t)this_first + w;
+                        r.k = W.mk[w] + j;
+                        r.b_row = W.row[j];
+                        r.f32 = PREC != kPrecFP64;
+                        r.sep = __longlong_as_double((long long)W.key[j]);
+                        P.arena[base + j] = r;
+                    } else {
+                        atomicOr(&W.drop, 1u << w);
+                    }
+                }
+            }
+            nm = 0;
+            __syncwarp();
         }
-        if (P.arena && staged > 0) flush();
-        __syncwarp();
 
         // ---- results (lane = source)
         if (mine) {
-            P.count[A.row] = cnt;
+            const int64_t s = this_first + lane;
+            P.count[s] = cnt;
             max_cnt = max(max_cnt, cnt);
-            if (P.acold_out && cnt > 0) P.acold_out[A.row] = W.cold[lane];
+            if (P.acold_out && cnt > 0)
+                P.acold_out[s] = ACold{W.lon[lane], W.lat[lane], W.theta[lane], s_ct.a, s_ct.b};
             if (P.want_best) {
-                P.best_b[A.row] = cnt ? (int64_t)b1 : -1;
-                P.best_sep[A.row] = cnt ? (double)__int_as_float(m1) * kRadToArcsec : NAN;
+                P.best_b[s] = cnt ? (int64_t)b1 : -1;
+                P.best_sep[s] = cnt == 0 ? NAN
+                                : PREC == kPrecFP64
+                                    ? __longlong_as_double((long long)m1)
+                                    : (double)__int_as_float((int)m1) * kRadToArcsec;
                 // float32 separations within twice their error bound of the
                 // smallest: the best pair is decided in float64
-                const float esep = 16.0f * kEps32 * (A.R + 2.0f * G.h_f);
-                if (cnt > 1 && __int_as_float(m2) - __int_as_float(m1) <= 2.0f * esep)
-                    P.tie_list[atomicAdd(&P.list_n[1], 1)] = A.row;
+                if (PREC != kPrecFP64 && cnt > 1) {
+                    const float esep = 16.0f * kEps32 * (s_at.R + 2.0f * G.h_f);
+                    if (__int_as_float((int)m2) - __int_as_float((int)m1) <= 2.0f * esep)
+                        P.tie_list[atomicAdd(&P.list_n[1], 1)] = (int32_t)s;
+                }
             }
-            if (W.drop[lane]) P.ovf_list[atomicAdd(&P.list_n[0], 1)] = A.row;
+            if ((W.drop >> lane) & 1u) P.ovf_list[atomicAdd(&P.list_n[0], 1)] = (int32_t)s;
         }
         __syncwarp();
+        this_first = next_first;
     }
     warp_add(&P.stats[0], n_cand);
     warp_add(&P.stats[3], n_mem);
@@ -1488,7 +1626,10 @@ void prepare_kernels() {
     cudaFuncSetAttribute(k_scan<kPrecFP32, kModeResolve, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     cudaFuncSetAttribute(k_scan<kPrecFP64, kModeCount, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     cudaFuncSetAttribute(k_scan<kPrecFP64, kModeEmit, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    cudaFuncSetAttribute(k_scan_src, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSrcSmem);
+    cudaFuncSetAttribute(k_scan_src<kPrecFP32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)kSrcSmem<kPrecFP32>);
+    cudaFuncSetAttribute(k_scan_src<kPrecFP64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)kSrcSmem<kPrecFP64>);
     radix_sort_prepare();
     done[dev] = true;
 }

@@ -157,3 +157,42 @@ def test_sparse_count_pass_rotated_frames(xm, shape):
     np.testing.assert_array_equal(_host(res.b_row), ref["b_row"])
     assert np.max(np.abs(_host(res.sep) - ref["sep"])) <= SEP_TOL
     np.testing.assert_array_equal(_host(res.best_b), bb["best_b"])
+
+
+@pytest.mark.parametrize("n_a,members", [(1, 1), (31, 3), (32, 45), (33, 3), (97, 12), (1000, 30), (5003, 1)])
+@pytest.mark.parametrize("frame", [0, 1])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_sparse_count_pass_equals_the_general_scan(xm, n_a, members, frame, prec):
+    """At the edges of a chunk of sources, of a round of records and of the
+    member stage: sources with `members` catalogue sources around each (so a
+    chunk has up to 32 times as many), a third of them in no region, in either
+    precision, both frames and every shape, against the warp-cooperative scan
+    (sources in sorted order). Rows and counts must be the same; separations
+    to the error of the path (float64: rounding of a few operations at 1e-5
+    rad, 1e-9 arcsec)."""
+    g = np.random.Generator(np.random.Philox(key=n_a + members))
+    lon, lat = g.uniform(0.0, 360.0, n_a), np.degrees(np.arcsin(g.uniform(-0.98, 0.98, n_a)))
+    lon[: n_a // 8] = np.mod(g.normal(0.0, 2.0 / 3600.0, n_a // 8), 360.0)  # windows on the seam
+    k = np.repeat(np.arange(n_a), members)
+    d = g.normal(0.0, 1.0 / 3600.0, (2, k.size)) + (k % 3 == 0) * 5.0 / 3600.0
+    b_lat = lat[k] + d[1]
+    b_lon = np.mod(lon[k] + d[0] / np.cos(np.radians(b_lat)), 360.0)
+    if frame:
+        lon, lat = oracle.from_equatorial(lon, lat, oracle.GAL)
+    idx = xm.Index(_cuda(b_lon), _cuda(b_lat), zone_height_arcsec=ZONE_H, build_fp64=prec == xm.PREC_FP64)
+    name = "k_scan_src" if prec == xm.PREC_FP32 else "k_scan_src_fp64"
+    for region in (dict(shape=0, a=2.0), dict(shape=1, a=3.0, b=1.5, pa=30.0),
+                   dict(shape=2, a=2.5, b=1.0, pa=110.0)):
+        xm.prof_enable(True)
+        try:
+            got, ref = (xm.Result(idx, _cuda(lon), _cuda(lat), frame=frame, precision=prec,
+                                  a_order=order, **region)
+                        for order in (xm.A_ORDER_INPUT, xm.A_ORDER_SORTED))
+            assert xm.prof_all()[name][1] == 1
+        finally:
+            xm.prof_enable(False)
+        tol = SEP_TOL if prec == xm.PREC_FP32 else 1e-9
+        for f in ("a_row", "b_row", "count", "best_b"):
+            np.testing.assert_array_equal(_host(getattr(got, f)), _host(getattr(ref, f)), err_msg=f)
+        for f in ("sep", "best_sep"):
+            np.testing.assert_allclose(_host(getattr(got, f)), _host(getattr(ref, f)), rtol=0, atol=tol)
