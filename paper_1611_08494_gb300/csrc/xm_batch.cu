@@ -104,15 +104,15 @@ __global__ void k_batch_ingest(BatchConst C, uint64_t* __restrict__ keys,
         atomicOr(err, kErrSize);
         atomicMin(bad_req, r);
     }
-    if (!keys) return;  // validation only (input order)
     const PosKey k = pos_key(lon, lat, C.nz);
     keys[g] = ((uint64_t)k.z << 32) | ((uint32_t)(k.key64 >> 32) & kRaKeyMask);
     vals[g] = (uint32_t)g;
 }
 
+// err, bad_req: also validates (input order, which needs no sort keys).
 __global__ void k_batch_prep(BatchConst C, const uint32_t* __restrict__ vals,
                              APrep* __restrict__ out, ACold* __restrict__ cold,
-                             int32_t* __restrict__ lrow) {
+                             int32_t* __restrict__ lrow, int32_t* err, int32_t* bad_req) {
     pdl_wait();
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= C.total) return;
@@ -126,6 +126,11 @@ __global__ void k_batch_prep(BatchConst C, const uint32_t* __restrict__ vals,
     const double a = col_or(R.a_col, i, R.a);
     const double b = R.shape == XM_CIRCLE ? a : col_or(R.b_col, i, R.b);
     const double pa = col_or(R.pa_col, i, R.pa);
+    if (err) {
+        if (!ok) atomicOr(err, kErrCoord);
+        if (!size_ok(a, b, pa)) atomicOr(err, kErrSize);
+        if (!ok || !size_ok(a, b, pa)) atomicMin(bad_req, r);
+    }
     APrep P;
     ACold C64;
     make_aprep(lon, lat, gamma, ok, a, b, pa, R.shape, R.pa_dir, R.size_k, R.pa_zero, C.nz, C.h_f,
@@ -146,26 +151,49 @@ __device__ __forceinline__ bool jt_un_b(int t) {
     return t == XM_JOIN_OR || t == XM_JOIN_ALL2 || t == XM_JOIN_NOT2_1 || t == XM_JOIN_XOR;
 }
 
+constexpr int kRowsBlock = 8;  // sources per thread of k_batch_rows_a
+
 // A-side rows of each batch row's join, and unmatched A sources per request.
 __global__ void k_batch_rows_a(BatchConst C, const int32_t* __restrict__ count,
                                int32_t* __restrict__ rows, unsigned long long* __restrict__ req_un_a) {
     pdl_wait();
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= C.total) return;
-    const int32_t r = find_req(C.off, C.n_req, g);
-    const ReqDev& R = C.req[r];
-    const int32_t c = count[g];
-    int32_t n = 0;
-    if (R.join_type >= 0) {
-        const int32_t sel = R.join_sel == XM_SEL_ALL ? c : (c > 0 ? 1 : 0);
-        n = jt_pairs(R.join_type) ? sel : 0;
-        if (sel == 0 && jt_un_a(R.join_type)) n = 1;
+    // (a block's sources almost always belong to one request: its unmatched
+    // ones are then one atomic; one per warp took 0.65 ms of a batch of 3e7
+    // sources on the few counters)
+    const int64_t first = (int64_t)blockIdx.x * (kRowsBlock * kBlock);
+    const int64_t last = min(first + kRowsBlock * kBlock, C.total) - 1;
+    const int32_t r0 = find_req(C.off, C.n_req, first);
+    const bool one = last < __ldg(&C.off[r0 + 1]);
+    __shared__ uint32_t block_un;
+    if (threadIdx.x == 0) block_un = 0;
+    __syncthreads();
+    uint32_t un = 0;
+#pragma unroll
+    for (int k = 0; k < kRowsBlock; k++) {
+        const int64_t g = first + k * kBlock + threadIdx.x;
+        const int32_t c = g <= last ? count[g] : -1;
+        const int32_t r = one || g > last ? r0 : find_req(C.off, C.n_req, g);
+        const ReqDev& R = C.req[r];
+        int32_t n = 0;
+        if (R.join_type >= 0) {
+            const int32_t sel = R.join_sel == XM_SEL_ALL ? c : (c > 0 ? 1 : 0);
+            n = jt_pairs(R.join_type) ? sel : 0;
+            if (sel == 0 && jt_un_a(R.join_type)) n = 1;
+        }
+        if (g <= last) rows[g] = n;
+        if (one) {
+            un += c == 0;
+        } else {  // one atomic per request and warp
+            const uint32_t peers = __match_any_sync(0xffffffffu, c == 0 ? r : -1);
+            const uint32_t lt = (1u << (threadIdx.x & 31)) - 1u;
+            if (c == 0 && (peers & lt) == 0)
+                atomicAdd(&req_un_a[r], (unsigned long long)__popc(peers));
+        }
     }
-    rows[g] = n;
-    // unmatched A sources per request, one atomic per request and warp
-    const uint32_t peers = __match_any_sync(__activemask(), c == 0 ? r : -1);
-    const uint32_t lt = (1u << (threadIdx.x & 31)) - 1u;
-    if (c == 0 && (peers & lt) == 0) atomicAdd(&req_un_a[r], (unsigned long long)__popc(peers));
+    un = __reduce_add_sync(0xffffffffu, un);
+    if ((threadIdx.x & 31) == 0 && un) atomicAdd(&block_un, un);
+    __syncthreads();
+    if (threadIdx.x == 0 && block_un) atomicAdd(&req_un_a[r0], (unsigned long long)block_un);
 }
 
 __global__ void k_batch_write_a(BatchConst C, const int32_t* __restrict__ count,
@@ -341,8 +369,8 @@ struct BatchBufs {
 };
 
 // small[]: 0 total pairs, 1 total rows, 2 arena records, 3 (int32 x2) error
-// bits and first bad request, 4 (int32 x4) list counts + pad, 6.. per-request
-// counters follow at small + 8: unmatched A [n], matched B [n]
+// bits and first bad request, 4 (int32 x4) list counts + chunk queue, 6 (int32)
+// largest member count, per-request counters follow at small + 8: unmatched A [n], matched B [n]
 constexpr int kSmallWords = 8;
 
 }  // namespace
@@ -442,7 +470,9 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
 
     // ---- buffers
     B.count = (int32_t*)dev_alloc(nn * sizeof(int32_t), s);
-    B.pair_off = (int64_t*)dev_alloc(nn * sizeof(int64_t), s);
+    // (the tiles' sums of a large count follow the offsets)
+    const int64_t sum_words = count_scan_words(total);
+    B.pair_off = (int64_t*)dev_alloc((nn + sum_words) * sizeof(int64_t), s);
     B.best_b = (int64_t*)dev_alloc(nn * (sizeof(int64_t) + sizeof(double)), s);
     B.pa = (int64_t*)dev_alloc((size_t)std::max(pair_cap, 1LL) * (2 * sizeof(int64_t) + sizeof(double)), s);
     if (want_rows)
@@ -466,7 +496,7 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
     B.lists = (int32_t*)dev_alloc(3 * nn * sizeof(int32_t), s);
     B.arena = (MemberRec*)dev_alloc(arena_cap * sizeof(MemberRec), s);
     B.rows = (int32_t*)dev_alloc(nn * sizeof(int32_t), s);
-    B.row_off = (int64_t*)dev_alloc(nn * sizeof(int64_t), s);
+    B.row_off = (int64_t*)dev_alloc((nn + sum_words) * sizeof(int64_t), s);
     if (tsize) B.table = (uint64_t*)dev_alloc(tsize * sizeof(uint64_t), s);
     B.small = (int64_t*)dev_alloc((kSmallWords + 2 * n + 1) * sizeof(int64_t), s);
     B.bounds = (int64_t*)dev_alloc((4 * n + 1) * sizeof(int64_t), s);
@@ -537,13 +567,11 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
                 xm_status r = radix_sort_u64(B.keys, B.vals, B.keys + nn, B.vals + nn, total,
                                              kSortBeginBit, 32 + bits_for(X->nz - 1), err, s);
                 if (r != XM_OK) return r;
-            } else {  // validation only; the scan takes the sources request by request
-                XM_LAUNCH("k_batch_ingest", grid_for(total), kBlock, 0, s, k_batch_ingest, C,
-                          (uint64_t*)nullptr, (uint32_t*)nullptr, err, bad_req);
             }
+            // (input order: the scan takes the sources request by request)
             XM_LAUNCH("k_batch_prep", grid_for(total), kBlock, 0, s, k_batch_prep, C,
                       sorted_a ? (const uint32_t*)B.vals : (const uint32_t*)nullptr, B.prep, B.cold,
-                      B.lrow);
+                      B.lrow, sorted_a ? (int32_t*)nullptr : err, bad_req);
         }
         ScanArgs a{};
         a.G = X->geom();
@@ -562,6 +590,7 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
         a.big_list = B.lists + 2 * nn;
         a.list_n = list_n;
         a.queue = queue;
+        a.max_count = (int32_t*)(B.small + 6);
         a.stats = stats;
         a.err = err;
         a.lrow = B.lrow;
@@ -570,7 +599,8 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
             r = launch_persistent_any(prec, kModeCount, a, pblocks, s);
             if (r != XM_OK) return r;
         }
-        r = exclusive_scan_i32(B.count, B.pair_off, total, B.small + 0, err, s);
+        r = sum_words ? count_scan(B.count, B.pair_off, total, B.small + 0, B.pair_off + nn, s)
+                      : exclusive_scan_i32(B.count, B.pair_off, total, B.small + 0, err, s);
         if (r != XM_OK) return r;
         if (total > 0) {
             XM_LAUNCH("k_place", 4 * sms, 256, 0, s, k_place, B.arena, arena_n, arena_cap,
@@ -588,12 +618,8 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
             if (e2 != cudaSuccess) return cuda_fail(e2, "batch memset");
             r = launch_persistent_any(prec, kModeEmit, b, pblocks, s);
             if (r != XM_OK) return r;
-            XM_LAUNCH("k_sort_small", grid_for(total), kBlock, 0, s, k_sort_small<1>, B.count,
-                      B.pair_off, total, pair_cap, B.pb, B.ps, (const int32_t*)nullptr);
-            XM_LAUNCH("k_sort_warp", (unsigned)(8 * sms), 32 * kWarpSortWarps, 0, s, k_sort_warp,
-                      B.count, B.pair_off, total, pair_cap, B.pb, B.ps, (const int32_t*)nullptr);
-            XM_LAUNCH("k_seg_sort", (unsigned)(2 * sms), 256, 0, s, k_seg_sort, B.count,
-                      B.pair_off, total, pair_cap, B.pb, B.ps, (const int32_t*)nullptr);
+            r = launch_member_sorts(B.count, B.pair_off, total, pair_cap, B.pb, B.ps, a.max_count, s);
+            if (r != XM_OK) return r;
             if (prec == XM_PREC_FP32_RECHECK) {
                 ScanArgs c = a;
                 c.list = B.lists + nn;
@@ -603,11 +629,12 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
                 r = launch_persistent_any(prec, kModeResolve, c, pblocks, s);
                 if (r != XM_OK) return r;
             }
-            XM_LAUNCH("k_batch_rows_a", grid_for(total), kBlock, 0, s, k_batch_rows_a, C,
+            XM_LAUNCH("k_batch_rows_a", grid_for((total + kRowsBlock - 1) / kRowsBlock), kBlock, 0, s, k_batch_rows_a, C,
                       B.count, B.rows, req_un_a);
         }
         if (want_rows) {
-            r = exclusive_scan_i32(B.rows, B.row_off, total, B.small + 1, err, s);
+            r = sum_words ? count_scan(B.rows, B.row_off, total, B.small + 1, B.row_off + nn, s)
+                          : exclusive_scan_i32(B.rows, B.row_off, total, B.small + 1, err, s);
             if (r != XM_OK) return r;
             if (total > 0) {
                 XM_LAUNCH("k_batch_write_a", grid_for(total), kBlock, 0, s, k_batch_write_a, C,

@@ -491,21 +491,8 @@ xm_status xm_pending::place_and_sort(int64_t np, int64_t n_ovf) {
         xm_status rr = launch_scan_any(prec, b, kModeEmit, n_ovf, s);
         if (rr != XM_OK) return rr;
     }
-    const unsigned gsm = grid_for(nA) < 8u * 152u ? grid_for(nA) : 8u * 152u;
-    // (four rows per lane once that leaves every SM its blocks)
-    if (nA >= 8 * 152 * 1024)
-        XM_LAUNCH("k_sort_small", gsm, kBlock, 0, s, k_sort_small<4>, R->count, R->pair_off, nA,
-                  (long long)np, R->b_row, R->sep, max_count);
-    else
-        XM_LAUNCH("k_sort_small", gsm, kBlock, 0, s, k_sort_small<1>, R->count, R->pair_off, nA,
-                  (long long)np, R->b_row, R->sep, max_count);
-    const int64_t gw = (nA + 32 * kWarpSortWarps - 1) / (32 * kWarpSortWarps);
-    XM_LAUNCH("k_sort_warp", (unsigned)(gw < 8 * 152 ? gw : 8 * 152), 32 * kWarpSortWarps, 0, s,
-              k_sort_warp, R->count, R->pair_off, nA, (long long)np, R->b_row, R->sep, max_count);
-    const int64_t gs = (nA + 255) / 256;
-    XM_LAUNCH("k_seg_sort", (unsigned)(gs < 2 * 152 ? gs : 2 * 152), 256, 0, s, k_seg_sort,
-              R->count, R->pair_off, nA, (long long)np, R->b_row, R->sep, max_count);
-    return XM_OK;
+    return launch_member_sorts(R->count, R->pair_off, nA, (long long)np, R->b_row, R->sep, max_count,
+                               s);
 }
 
 bool xm_pending::alloc_pairs(int64_t np) {

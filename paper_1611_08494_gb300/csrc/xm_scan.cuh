@@ -1473,12 +1473,14 @@ __global__ void __launch_bounds__(256) k_sort_small(const int32_t* __restrict__ 
 // Members of A rows with kSmallSort < count <= kWarpSort into ascending B row,
 // one warp per row: every entry's final place is the number of entries with a
 // smaller B row (all distinct within a row), counted against a copy in shared
-// memory. Warps stride over the rows 32 at a time: one coalesced load of 32
+// memory. Warps stride over the rows 32 G at a time: a coalesced load of 32
 // counts and a ballot find the rows of this size class, so rows of other
-// classes cost no dependent load.
+// classes cost no dependent load (G such loads in flight: 3e7 rows of a batch,
+// few of this class, took 0.21 ms with one).
 constexpr int kWarpSort = 512;
 constexpr int kWarpSortWarps = 4;
 
+template <int G>
 __global__ void __launch_bounds__(32 * kWarpSortWarps) k_sort_warp(
     const int32_t* __restrict__ count, const int64_t* __restrict__ pair_off, int64_t nA,
     long long out_cap, int64_t* __restrict__ out_b, double* __restrict__ out_sep,
@@ -1488,40 +1490,52 @@ __global__ void __launch_bounds__(32 * kWarpSortWarps) k_sort_warp(
     __shared__ int64_t sb[kWarpSortWarps][kWarpSort];
     __shared__ double ss[kWarpSortWarps][kWarpSort];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * kWarpSortWarps * 32;
-    for (int64_t base = ((int64_t)blockIdx.x * kWarpSortWarps + w) * 32; base < nA; base += stride) {
-        const int64_t mine = base + lane;
-        const int32_t cm = mine < nA ? count[mine] : 0;
-        unsigned todo = __ballot_sync(0xffffffffu, cm > kSmallSort && cm <= kWarpSort);
-        while (todo) {
-            const int l = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const int64_t row = base + l;
-            const int32_t c = __shfl_sync(0xffffffffu, cm, l);
-            const int64_t o = pair_off[row];
-            if (o + c > out_cap) continue;  // uniform over the warp
-            for (int k = lane; k < c; k += 32) {
-                sb[w][k] = out_b[o + k];
-                ss[w][k] = out_sep[o + k];
+    const int64_t stride = (int64_t)gridDim.x * kWarpSortWarps * (32 * G);
+    for (int64_t base0 = ((int64_t)blockIdx.x * kWarpSortWarps + w) * (32 * G); base0 < nA;
+         base0 += stride) {
+        int32_t cg[G];
+#pragma unroll
+        for (int g = 0; g < G; g++) {
+            const int64_t mine = base0 + 32 * g + lane;
+            cg[g] = mine < nA ? __ldg(count + mine) : 0;
+        }
+        for (int g = 0; g < G; g++) {
+            const int64_t base = base0 + 32 * g;
+            int32_t cm = cg[0];
+#pragma unroll
+            for (int h = 1; h < G; h++) cm = g == h ? cg[h] : cm;
+            unsigned todo = __ballot_sync(0xffffffffu, cm > kSmallSort && cm <= kWarpSort);
+            while (todo) {
+                const int l = __ffs(todo) - 1;
+                todo &= todo - 1;
+                const int64_t row = base + l;
+                const int32_t c = __shfl_sync(0xffffffffu, cm, l);
+                const int64_t o = pair_off[row];
+                if (o + c > out_cap) continue;  // uniform over the warp
+                for (int k = lane; k < c; k += 32) {
+                    sb[w][k] = out_b[o + k];
+                    ss[w][k] = out_sep[o + k];
+                }
+                __syncwarp();
+                for (int k = lane; k < c; k += 32) {
+                    const int64_t key = sb[w][k];
+                    int rank = 0;
+                    for (int j = 0; j < c; j++) rank += sb[w][j] < key;
+                    out_b[o + rank] = key;
+                    out_sep[o + rank] = ss[w][k];
+                }
+                __syncwarp();
             }
-            __syncwarp();
-            for (int k = lane; k < c; k += 32) {
-                const int64_t key = sb[w][k];
-                int rank = 0;
-                for (int j = 0; j < c; j++) rank += sb[w][j] < key;
-                out_b[o + rank] = key;
-                out_sep[o + rank] = ss[w][k];
-            }
-            __syncwarp();
         }
     }
 }
 
 // Members of A rows with kWarpSort < count <= kSegMax into ascending B row:
 // a bitonic network in shared memory, one block per row. Blocks stride over
-// the rows a block's width at a time, each thread checking one count, and sort the rows
-// of this size class found in the chunk (no list, so no host
+// the rows G times a block's width at a time, each thread checking G counts,
+// and sort the rows of this size class found in the chunk (no list, so no host
 // synchronisation is needed to launch it).
+template <int G>
 __global__ void __launch_bounds__(256) k_seg_sort(const int32_t* __restrict__ count,
                                                   const int64_t* __restrict__ pair_off, int64_t nA,
                                                   long long out_cap, int64_t* __restrict__ out_b,
@@ -1531,17 +1545,22 @@ __global__ void __launch_bounds__(256) k_seg_sort(const int32_t* __restrict__ co
     if (max_count && *max_count <= kWarpSort) return;  // no row of this size class
     __shared__ int64_t kb[kSegMax];
     __shared__ double ks[kSegMax];
-    __shared__ int32_t found[256];
+    __shared__ int32_t found[256 * G];
     __shared__ int n_found;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nA;
-         base += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t base = (int64_t)blockIdx.x * (256 * G); base < nA;
+         base += (int64_t)gridDim.x * (256 * G)) {
         if (threadIdx.x == 0) n_found = 0;
         __syncthreads();
-        const int64_t mine = base + threadIdx.x;
-        if (mine < nA) {
-            const int32_t cm = count[mine];
-            if (cm > kWarpSort && cm <= kSegMax) found[atomicAdd(&n_found, 1)] = (int32_t)threadIdx.x;
+        int32_t cg[G];
+#pragma unroll
+        for (int g = 0; g < G; g++) {
+            const int64_t mine = base + 256 * g + threadIdx.x;
+            cg[g] = mine < nA ? __ldg(count + mine) : 0;
         }
+#pragma unroll
+        for (int g = 0; g < G; g++)
+            if (cg[g] > kWarpSort && cg[g] <= kSegMax)
+                found[atomicAdd(&n_found, 1)] = 256 * g + (int32_t)threadIdx.x;
         __syncthreads();
         const int nf = n_found;
         for (int f = 0; f < nf; f++) {
@@ -1583,6 +1602,34 @@ __global__ void __launch_bounds__(256) k_seg_sort(const int32_t* __restrict__ co
         }
         __syncthreads();  // n_found is reset for the next chunk
     }
+}
+
+// The three sorts over a placed pair list of nA rows.
+xm_status launch_member_sorts(const int32_t* count, const int64_t* pair_off, int64_t nA,
+                              long long out_cap, int64_t* out_b, double* out_sep,
+                              const int32_t* max_count, cudaStream_t s) {
+    const int64_t g = (nA + 255) / 256;
+    const int64_t gw = (nA + 32 * kWarpSortWarps - 1) / (32 * kWarpSortWarps);
+    const unsigned small = (unsigned)(g < 8 * 152 ? g : 8 * 152);
+    const unsigned warp = (unsigned)(gw < 8 * 152 ? gw : 8 * 152);
+    const unsigned seg = (unsigned)(g < 2 * 152 ? g : 2 * 152);
+    // (four rows per lane once that leaves every SM its blocks)
+    if (nA >= 8 * 152 * 1024) {
+        XM_LAUNCH("k_sort_small", small, 256, 0, s, k_sort_small<4>, count, pair_off, nA, out_cap,
+                  out_b, out_sep, max_count);
+        XM_LAUNCH("k_sort_warp", warp, 32 * kWarpSortWarps, 0, s, k_sort_warp<4>, count, pair_off,
+                  nA, out_cap, out_b, out_sep, max_count);
+        XM_LAUNCH("k_seg_sort", seg, 256, 0, s, k_seg_sort<4>, count, pair_off, nA, out_cap, out_b,
+                  out_sep, max_count);
+    } else {
+        XM_LAUNCH("k_sort_small", small, 256, 0, s, k_sort_small<1>, count, pair_off, nA, out_cap,
+                  out_b, out_sep, max_count);
+        XM_LAUNCH("k_sort_warp", warp, 32 * kWarpSortWarps, 0, s, k_sort_warp<1>, count, pair_off,
+                  nA, out_cap, out_b, out_sep, max_count);
+        XM_LAUNCH("k_seg_sort", seg, 256, 0, s, k_seg_sort<1>, count, pair_off, nA, out_cap, out_b,
+                  out_sep, max_count);
+    }
+    return XM_OK;
 }
 
 // Long segments: sort (b_row, position) pairs with the radix sort, then
