@@ -704,7 +704,8 @@ xm_status index_build_status(int32_t bits);
 
 // Device primitives (xm_sort.cu).
 // Stable LSD radix sort of (keys, vals) on key bits [begin_bit, end_bit).
-// Sorted data ends in (keys, vals); (tk, tv) are scratch of the same sizes.
+// Sorted data ends in (keys, vals); (tk, tv) are scratch of the same sizes
+// (vals and tv NULL: keys alone).
 // A look-back that timed out sets kErrTimeout in *err (device), which the
 // caller reads at its next synchronisation.
 xm_status radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* tk, uint32_t* tv, int64_t n,

@@ -6,18 +6,20 @@
 //
 //   k_val_key     keys to order-preserving unsigned codes (int64: sign bit
 //                 flipped; float64: IEEE total order with -0 folded into +0;
-//                 NaN -> all ones, above every number, never looked up), row
-//                 payloads, and the AND / OR of all B codes (bits that never
-//                 differ need no sort pass)
-//   radix sort    stable, so equal keys keep ascending B rows (xm_sort.cu):
-//                 on the codes themselves when they differ in at most 32
-//                 bits, else on a 32-bit hash of them (half the passes;
-//                 equal keys still form one run, now shared with the few
-//                 keys whose hash collides, told apart by the codes)
-//   k_val_lut     a bucket table over the sorted codes (one bucket per two
+//                 NaN -> all ones, above every number, never looked up), and
+//                 the AND / OR of all B codes (bits that never differ need no
+//                 sort pass); writes a 32-bit hash of each code and its row,
+//                 packed in 64 bits
+//   k_val_pack    the same with the codes' low bits, when they differ in no
+//                 more than 32
+//   radix sort    stable, so equal keys keep ascending B rows (xm_sort.cu), on
+//                 the high half of the packed words: one array of 8 bytes a
+//                 source. Equal keys form one run, shared under the hash with
+//                 the few keys that collide, which B's keys tell apart
+//   k_val_lut     a bucket table over the sorted words (one bucket per two
 //                 to four keys; long runs of entries by k_val_runs)
-//   k_val_probe   per A: the run of equal B codes, searched inside one
-//                 bucket; count, best B row, first sorted position
+//   k_val_probe   per A: the run of equal words, searched inside one bucket;
+//                 count, best B row, and that row or the first match's place
 //   prefix sum    pair offsets
 //   k_val_emit    the pairs of each A row
 #include <math.h>
@@ -54,11 +56,9 @@ __device__ __forceinline__ uint64_t code_hash(uint64_t x) {
 }
 
 // Grid-stride over B (a few blocks per SM), so the AND / OR of all codes
-// costs one pair of atomics per block. Writes the codes by row and, for the
-// hashed order, their hashes.
+// costs one pair of atomics per block.
 __global__ void k_val_key(const void* __restrict__ keys, int64_t n, int32_t type,
-                          uint64_t* __restrict__ codes, uint64_t* __restrict__ hashes,
-                          uint32_t* __restrict__ rows, unsigned long long* __restrict__ and_or) {
+                          uint64_t* __restrict__ packed, unsigned long long* __restrict__ and_or) {
     pdl_wait();
     __shared__ unsigned long long s_and, s_or;
     if (threadIdx.x == 0) {
@@ -70,9 +70,7 @@ __global__ void k_val_key(const void* __restrict__ keys, int64_t n, int32_t type
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t c = key_code(keys, i, type);
-        codes[i] = c;
-        hashes[i] = code_hash(c);
-        rows[i] = (uint32_t)i;
+        packed[i] = code_hash(c) << 32 | (uint32_t)i;
         c_and &= c;
         c_or |= c;
     }
@@ -91,10 +89,19 @@ __global__ void k_val_key(const void* __restrict__ keys, int64_t n, int32_t type
     }
 }
 
-// Bucket table over the sorted codes: the codes share every bit above
-// end_bit; bucket(c) = low end_bit bits of c >> shift, and lut[k] is the
-// first sorted position whose bucket reaches k (lut[nb] = n). Runs of
-// entries longer than kRunInline go to a list filled by k_val_runs.
+// The low bits of the codes instead of their hashes.
+__global__ void k_val_pack(const void* __restrict__ keys, int64_t n, int32_t type, uint64_t mask,
+                           uint64_t* __restrict__ packed) {
+    pdl_wait();
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) packed[i] = (key_code(keys, i, type) & mask) << 32 | (uint32_t)i;
+}
+
+// Bucket table over the sorted words (word = hash or low code bits, above the
+// row): bucket = word >> shift, and lut[k] is the first sorted position whose
+// bucket reaches k (lut[nb] = n). Codes share every bit outside mask with
+// prefix (unhashed). Runs of entries longer than kRunInline go to a list
+// filled by k_val_runs.
 struct ValLut {
     uint64_t prefix, mask;  // common high bits, mask of the low end_bit bits
     uint32_t shift, nb;     // bucket shift, buckets
@@ -108,8 +115,8 @@ struct ValRun {
 
 constexpr int64_t kRunInline = 32;
 
-__device__ __forceinline__ uint32_t val_bucket(const ValLut& V, uint64_t c) {
-    return (uint32_t)((c & V.mask) >> V.shift);
+__device__ __forceinline__ uint32_t val_bucket(const ValLut& V, uint64_t packed) {
+    return (uint32_t)(packed >> 32) >> V.shift;
 }
 
 __global__ void k_val_lut(const uint64_t* __restrict__ sorted, int64_t n, ValLut V,
@@ -144,116 +151,143 @@ __global__ void k_val_runs(const ValRun* __restrict__ runs, const unsigned long 
     }
 }
 
-// First position in sorted[lo, hi) whose code is >= c (or > c when upper).
+// First position in sorted[lo, hi) whose word is >= w (or > w when upper).
 __device__ __forceinline__ int64_t bound(const uint64_t* __restrict__ sorted, int64_t lo, int64_t hi,
-                                         uint64_t c, bool upper) {
+                                         uint32_t w, bool upper) {
     while (lo < hi) {
         const int64_t mid = lo + ((hi - lo) >> 1);
-        const uint64_t v = __ldg(&sorted[mid]);
-        if (upper ? v <= c : v < c) lo = mid + 1;
+        const uint32_t v = (uint32_t)(__ldg(&sorted[mid]) >> 32);
+        if (upper ? v <= w : v < w) lo = mid + 1;
         else hi = mid;
     }
     return lo;
 }
 
-__global__ void k_val_probe(const void* __restrict__ a_keys, int64_t n_a, int32_t type,
-                            const uint64_t* __restrict__ sorted, const uint32_t* __restrict__ rows,
-                            int64_t n_b, ValLut V, int32_t* __restrict__ count,
-                            int64_t* __restrict__ first, int64_t* __restrict__ best_b,
-                            double* __restrict__ best_sep) {
-    pdl_wait();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_a) return;
-    const uint64_t c = key_code(a_keys, i, type);
-    int64_t lo = 0, hi = 0;
-    // (NaN never matches; the int64 maximum has the same code and does)
-    if (n_b > 0 && !(type == XM_KEY_FLOAT64 && c == kNaNCode) && (c & ~V.mask) == V.prefix) {
-        const uint32_t b = val_bucket(V, c);
-        const int64_t b0 = __ldg(&V.lut[b]), b1 = __ldg(&V.lut[b + 1]);
-        lo = bound(sorted, b0, b1, c, false);
-        hi = lo < b1 && __ldg(&sorted[lo]) == c ? bound(sorted, lo, b1, c, true) : lo;
-    }
-    const int64_t m = hi - lo;
-    count[i] = (int32_t)(m < 2147483647 ? m : 2147483647);
-    first[i] = lo;
-    if (best_b) {
-        best_b[i] = m > 0 ? (int64_t)rows[lo] : -1;
-        best_sep[i] = m > 0 ? 0.0 : NAN;
-    }
-}
+constexpr int kProbeKeys = 4;  // A keys per thread
+constexpr int kProbeRun = 4;   // words of a bucket read at once
 
-// Hashed order: the run of A's hash, then the B rows whose code is A's.
-__global__ void k_val_probe_hashed(const void* __restrict__ a_keys, int64_t n_a, int32_t type,
-                                   const uint64_t* __restrict__ sorted,
-                                   const uint32_t* __restrict__ rows,
-                                   const uint64_t* __restrict__ codes, int64_t n_b, ValLut V,
-                                   int32_t* __restrict__ count, int64_t* __restrict__ first,
-                                   int64_t* __restrict__ best_b, double* __restrict__ best_sep) {
+// Per A key the B rows of equal keys. Bound by the latency of dependent loads
+// (bucket table, bucket, B's key under the hash), kept in flight for four keys
+// at a time. first: the only match's row, or the place of the first of several
+// (k_val_emit then reads no list for most keys: 0.45 ms for 2.5e7 against 0.81
+// when each went through its place to a row). 1.8 ms for 2.5e7 keys among 1e8;
+// 2.0 a key per thread with codes and rows apart from the sorted hashes.
+template <bool HASHED>
+__global__ void __launch_bounds__(kBlock) k_val_probe(
+    const void* __restrict__ a_keys, int64_t n_a, int32_t type, const uint64_t* __restrict__ sorted,
+    const void* __restrict__ b_keys, int64_t n_b, ValLut V, int32_t* __restrict__ count,
+    int64_t* __restrict__ first, int64_t* __restrict__ best_b, double* __restrict__ best_sep) {
     pdl_wait();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_a) return;
-    const uint64_t c = key_code(a_keys, i, type);
-    int64_t lo = 0, m = 0, best = -1;
-    if (n_b > 0 && !(type == XM_KEY_FLOAT64 && c == kNaNCode)) {
-        const uint64_t h = code_hash(c);
-        const uint32_t b = val_bucket(V, h);
-        const int64_t b0 = __ldg(&V.lut[b]), b1 = __ldg(&V.lut[b + 1]);
-        lo = bound(sorted, b0, b1, h, false);
-        for (int64_t p = lo; p < b1 && __ldg(&sorted[p]) == h; p++) {
-            const uint32_t r = __ldg(&rows[p]);
-            if (__ldg(&codes[r]) == c) {
-                if (m == 0) best = r;
-                m++;
+    const int64_t i0 = (int64_t)blockIdx.x * (kProbeKeys * kBlock) + threadIdx.x;
+    uint64_t c[kProbeKeys];
+    uint32_t w[kProbeKeys], lo[kProbeKeys], hi[kProbeKeys];
+    uint64_t e[kProbeKeys][kProbeRun];
+#pragma unroll
+    for (int k = 0; k < kProbeKeys; k++) {
+        const int64_t i = i0 + k * kBlock;
+        c[k] = i < n_a ? key_code(a_keys, i, type) : 0;
+        // (NaN never matches; the int64 maximum has the same code and does)
+        const bool any = i < n_a && n_b > 0 && !(type == XM_KEY_FLOAT64 && c[k] == kNaNCode) &&
+                         (HASHED || (c[k] & ~V.mask) == V.prefix);
+        w[k] = (uint32_t)(HASHED ? code_hash(c[k]) : c[k] & V.mask);
+        const uint32_t b = w[k] >> V.shift;
+        lo[k] = any ? __ldg(&V.lut[b]) : 0;
+        hi[k] = any ? __ldg(&V.lut[b + 1]) : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kProbeKeys; k++) {
+        if (hi[k] - lo[k] > 2 * kProbeRun) lo[k] = (uint32_t)bound(sorted, lo[k], hi[k], w[k], false);
+#pragma unroll
+        for (int j = 0; j < kProbeRun; j++)
+            e[k][j] = lo[k] + j < hi[k] ? __ldg(&sorted[lo[k] + j]) : 0;
+    }
+    int32_t at[kProbeKeys];  // the first word equal to w among those read, or -1
+    bool eq[kProbeKeys];
+#pragma unroll
+    for (int k = 0; k < kProbeKeys; k++) {
+        at[k] = -1;
+        uint32_t row = 0;
+#pragma unroll
+        for (int j = kProbeRun - 1; j >= 0; j--)
+            if (lo[k] + j < hi[k] && (uint32_t)(e[k][j] >> 32) == w[k]) {
+                at[k] = j;
+                row = (uint32_t)e[k][j];
+            }
+        eq[k] = at[k] >= 0 && (!HASHED || key_code(b_keys, row, type) == c[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < kProbeKeys; k++) {
+        const int64_t i = i0 + k * kBlock;
+        if (i >= n_a) break;
+        int64_t m = 0, f = 0, best = -1, p = lo[k];
+        if (at[k] < 0 && hi[k] - lo[k] > kProbeRun && (uint32_t)(e[k][kProbeRun - 1] >> 32) < w[k])
+            p = bound(sorted, lo[k] + kProbeRun, hi[k], w[k], false);
+        else if (at[k] < 0)
+            p = hi[k];
+        else
+            p += at[k];
+        // (p: the first word equal to w, or one past those below it)
+        bool known = at[k] >= 0;
+        for (; p < hi[k]; p++) {
+            const int64_t j = p - lo[k];
+            uint64_t v = 0;
+            if (j < kProbeRun) {
+#pragma unroll
+                for (int q = 0; q < kProbeRun; q++) v = q == j ? e[k][q] : v;
+            } else {
+                v = __ldg(&sorted[p]);
+            }
+            if ((uint32_t)(v >> 32) != w[k]) break;
+            const uint32_t r = (uint32_t)v;
+            const bool match = known ? eq[k] : !HASHED || key_code(b_keys, r, type) == c[k];
+            known = false;
+            if (!match) continue;
+            if (m == 0) {
+                best = r;
+                f = p;
+            }
+            m++;
+            if (!HASHED && p - f >= 2 * kProbeRun) {  // a long run of equal keys
+                m = bound(sorted, p, hi[k], w[k], true) - f;
+                break;
             }
         }
-    }
-    count[i] = (int32_t)(m < 2147483647 ? m : 2147483647);
-    first[i] = lo;
-    if (best_b) {
-        best_b[i] = best;
-        best_sep[i] = m > 0 ? 0.0 : NAN;
+        count[i] = (int32_t)(m < 2147483647 ? m : 2147483647);
+        first[i] = m == 1 ? best : f;
+        if (best_b) {
+            best_b[i] = best;
+            best_sep[i] = m > 0 ? 0.0 : NAN;
+        }
     }
 }
 
-__global__ void k_val_emit_hashed(const void* __restrict__ a_keys, int32_t type,
-                                  const int32_t* __restrict__ count,
-                                  const int64_t* __restrict__ first,
-                                  const int64_t* __restrict__ pair_off,
-                                  const uint32_t* __restrict__ rows,
-                                  const uint64_t* __restrict__ codes, int64_t n_a,
-                                  int64_t* __restrict__ pa, int64_t* __restrict__ pb,
-                                  double* __restrict__ ps) {
+template <bool HASHED>
+__global__ void k_val_emit(const void* __restrict__ a_keys, int32_t type,
+                           const int32_t* __restrict__ count, const int64_t* __restrict__ first,
+                           const int64_t* __restrict__ pair_off, const uint64_t* __restrict__ sorted,
+                           const void* __restrict__ b_keys, int64_t n_a, int64_t* __restrict__ pa,
+                           int64_t* __restrict__ pb, double* __restrict__ ps) {
     pdl_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_a) return;
     const int32_t c = count[i];
     if (c == 0) return;
-    const uint64_t code = key_code(a_keys, i, type);
-    const int64_t o = pair_off[i];
+    const int64_t o = pair_off[i], f = first[i];
+    if (c == 1) {
+        pa[o] = i;
+        pb[o] = f;
+        ps[o] = 0.0;
+        return;
+    }
+    const uint64_t code = HASHED ? key_code(a_keys, i, type) : 0;
     int32_t k = 0;
-    for (int64_t p = first[i]; k < c; p++) {  // (the run holds all c matches)
-        const uint32_t r = rows[p];
-        if (codes[r] != code) continue;
+    for (int64_t p = f; k < c; p++) {  // (the run holds all c matches)
+        const uint32_t r = (uint32_t)sorted[p];
+        if (HASHED && key_code(b_keys, r, type) != code) continue;
         pa[o + k] = i;
         pb[o + k] = r;
         ps[o + k] = 0.0;
         k++;
-    }
-}
-
-__global__ void k_val_emit(const int32_t* __restrict__ count, const int64_t* __restrict__ first,
-                           const int64_t* __restrict__ pair_off, const uint32_t* __restrict__ rows,
-                           int64_t n_a, int64_t* __restrict__ pa, int64_t* __restrict__ pb,
-                           double* __restrict__ ps) {
-    pdl_wait();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_a) return;
-    const int32_t c = count[i];
-    const int64_t o = pair_off[i], f = first[i];
-    for (int32_t k = 0; k < c; k++) {
-        pa[o + k] = i;
-        pb[o + k] = rows[f + k];
-        ps[o + k] = 0.0;
     }
 }
 
@@ -306,16 +340,13 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
     // positions, totals and the error word
     void* d_a = nullptr;
     void* d_b = nullptr;
-    uint64_t* codes = (uint64_t*)dev_alloc(2 * nb1 * sizeof(uint64_t), s);
-    uint64_t* hashes = (uint64_t*)dev_alloc(2 * nb1 * sizeof(uint64_t), s);
-    uint32_t* rows = (uint32_t*)dev_alloc(2 * nb1 * sizeof(uint32_t), s);
+    uint64_t* packed = (uint64_t*)dev_alloc(2 * nb1 * sizeof(uint64_t), s);
     int64_t* first = (int64_t*)dev_alloc(na1 * sizeof(int64_t), s);
     unsigned long long* small = (unsigned long long*)dev_alloc(4 * sizeof(unsigned long long), s);
     uint32_t* lut = nullptr;
     ValRun* runs = nullptr;
     auto body = [&]() -> xm_status {
-        if (!R->count || !R->pair_off || (want_best && !R->best_b) || !codes || !hashes || !rows ||
-            !first || !small)
+        if (!R->count || !R->pair_off || (want_best && !R->best_b) || !packed || !first || !small)
             return set_error(XM_ENOMEM, "xm_match_values: work buffers");
         cudaError_t e;
         const void* ak = a_keys;
@@ -338,8 +369,7 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
         int32_t* err = (int32_t*)(small + 3);
         if (n_b > 0) {
             const unsigned gk = grid_of(n_b) < 8 * 152 ? grid_of(n_b) : 8 * 152;
-            XM_LAUNCH("k_val_key", gk, kBlock, 0, s, k_val_key, bk, n_b, key_type, codes, hashes,
-                      rows, small);
+            XM_LAUNCH("k_val_key", gk, kBlock, 0, s, k_val_key, bk, n_b, key_type, packed, small);
         }
         unsigned long long h_ao[2] = {~0ull, 0ull};
         e = cudaMemcpyAsync(h_ao, small, sizeof(h_ao), cudaMemcpyDeviceToHost, s);
@@ -350,9 +380,12 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
         const int code_bits = top_bit(h_ao[0] ^ h_ao[1]);
         const bool hashed = code_bits > 32;
         const int end_bit = hashed ? 32 : code_bits;
-        uint64_t* sorted = hashed ? hashes : codes;
+        if (n_b > 0 && !hashed)
+            XM_LAUNCH("k_val_pack", grid_of(n_b), kBlock, 0, s, k_val_pack, bk, n_b, key_type,
+                      (1ull << end_bit) - 1, packed);
         if (n_b > 1 && end_bit > 0) {
-            xm_status r = radix_sort_u64(sorted, rows, sorted + nb1, rows + nb1, n_b, 0, end_bit, err, s);
+            xm_status r = radix_sort_u64(packed, nullptr, packed + nb1, nullptr, n_b, 32, 32 + end_bit,
+                                         err, s);
             if (r != XM_OK) return r;
         }
         // bucket table: about one bucket per 2-4 keys over the differing bits
@@ -373,17 +406,17 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
         e = cudaMemsetAsync(n_runs, 0, sizeof(unsigned long long), s);
         if (e != cudaSuccess) return cuda_fail(e, "xm_match_values: memset");
         if (n_b > 0) {
-            XM_LAUNCH("k_val_lut", grid_of(n_b), kBlock, 0, s, k_val_lut, sorted, n_b, V, runs,
+            XM_LAUNCH("k_val_lut", grid_of(n_b), kBlock, 0, s, k_val_lut, packed, n_b, V, runs,
                       n_runs, run_cap, err);
             XM_LAUNCH("k_val_runs", 4 * 152, kBlock, 0, s, k_val_runs, runs, n_runs, run_cap, lut);
         }
+        const unsigned gp = grid_of((n_a + kProbeKeys - 1) / kProbeKeys);
         if (n_a > 0 && hashed)
-            XM_LAUNCH("k_val_probe", grid_of(n_a), kBlock, 0, s, k_val_probe_hashed, ak, n_a,
-                      key_type, sorted, rows, codes, n_b, V, R->count, first, R->best_b,
-                      R->best_sep);
+            XM_LAUNCH("k_val_probe", gp, kBlock, 0, s, k_val_probe<true>, ak, n_a, key_type, packed, bk,
+                      n_b, V, R->count, first, R->best_b, R->best_sep);
         else if (n_a > 0)
-            XM_LAUNCH("k_val_probe", grid_of(n_a), kBlock, 0, s, k_val_probe, ak, n_a, key_type,
-                      codes, rows, n_b, V, R->count, first, R->best_b, R->best_sep);
+            XM_LAUNCH("k_val_probe", gp, kBlock, 0, s, k_val_probe<false>, ak, n_a, key_type, packed, bk,
+                      n_b, V, R->count, first, R->best_b, R->best_sep);
         xm_status r = R->zeros ? count_scan(R->count, R->pair_off, n_a, (int64_t*)(small + 2), R->zeros, s)
                                : exclusive_scan_i32(R->count, R->pair_off, n_a, (int64_t*)(small + 2),
                                                     err, s);
@@ -402,21 +435,18 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
             R->b_row = R->a_row + np;
             R->sep = (double*)(R->b_row + np);
             if (n_a > 0 && hashed)
-                XM_LAUNCH("k_val_emit", grid_of(n_a), kBlock, 0, s, k_val_emit_hashed, ak, key_type,
-                          R->count, first, R->pair_off, rows, codes, n_a, R->a_row, R->b_row,
-                          R->sep);
+                XM_LAUNCH("k_val_emit", grid_of(n_a), kBlock, 0, s, k_val_emit<true>, ak, key_type,
+                          R->count, first, R->pair_off, packed, bk, n_a, R->a_row, R->b_row, R->sep);
             else if (n_a > 0)
-                XM_LAUNCH("k_val_emit", grid_of(n_a), kBlock, 0, s, k_val_emit, R->count, first,
-                          R->pair_off, rows, n_a, R->a_row, R->b_row, R->sep);
+                XM_LAUNCH("k_val_emit", grid_of(n_a), kBlock, 0, s, k_val_emit<false>, ak, key_type,
+                          R->count, first, R->pair_off, packed, bk, n_a, R->a_row, R->b_row, R->sep);
         }
         return XM_OK;
     };
     const xm_status st = body();
     dev_free(d_a, s);
     dev_free(d_b, s);
-    dev_free(codes, s);
-    dev_free(hashes, s);
-    dev_free(rows, s);
+    dev_free(packed, s);
     dev_free(first, s);
     dev_free(small, s);
     dev_free(lut, s);
