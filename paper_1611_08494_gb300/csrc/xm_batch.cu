@@ -4,12 +4,15 @@
 // The A sources of all requests form one batch-wide catalogue: batch row
 // g = off[r] + i for row i of request r. The device pipeline is the one of
 // xm_match run once for the batch:
-//   k_batch_ingest  per batch row: request (binary search of the offsets),
-//                   position in the index frame, validity, (zone, RA) key
-//   radix sort      all requests together, so neighbouring warps share the
-//                   index's B rows in L2 whatever request they serve
+//   k_batch_ingest  (sorted order) per batch row: request (binary search of the
+//                   offsets), position in the index frame, validity, (zone,
+//                   RA) key
+//   radix sort      (sorted order) all requests together, so neighbouring warps
+//                   share the index's B rows in L2 whatever request they serve
 //   k_batch_prep    prepared sources with their request's region and shape
-//   k_scan          persistent: a fixed grid whose warps take 32-source
+//                   (input order: and validity)
+//   k_scan_src      the sources whose regions are small against the zones
+//   k_scan          the rest; persistent: a fixed grid whose warps take 32-source
 //                   chunks from a device work queue until it is empty, so a
 //                   mix of tiny and huge requests keeps every SM busy
 //   placement, segment sorts, float64 best-pair resolution  (as xm_match)
@@ -370,7 +373,8 @@ struct BatchBufs {
 
 // small[]: 0 total pairs, 1 total rows, 2 arena records, 3 (int32 x2) error
 // bits and first bad request, 4 (int32 x4) list counts + chunk queue, 6 (int32)
-// largest member count, per-request counters follow at small + 8: unmatched A [n], matched B [n]
+// largest member count and sources the sparse pass leaves, 7 (int32) the sparse
+// pass's queue, per-request counters follow at small + 8: unmatched A [n], matched B [n]
 constexpr int kSmallWords = 8;
 
 }  // namespace
@@ -493,7 +497,7 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
     B.prep = (APrep*)dev_alloc(nn * sizeof(APrep), s);
     B.cold = (ACold*)dev_alloc(nn * sizeof(ACold), s);
     B.lrow = (int32_t*)dev_alloc(nn * sizeof(int32_t), s);
-    B.lists = (int32_t*)dev_alloc(3 * nn * sizeof(int32_t), s);
+    B.lists = (int32_t*)dev_alloc(4 * nn * sizeof(int32_t), s);
     B.arena = (MemberRec*)dev_alloc(arena_cap * sizeof(MemberRec), s);
     B.rows = (int32_t*)dev_alloc(nn * sizeof(int32_t), s);
     B.row_off = (int64_t*)dev_alloc((nn + sum_words) * sizeof(int64_t), s);
@@ -596,7 +600,22 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
         a.lrow = B.lrow;
         xm_status r = XM_OK;
         if (total > 0) {
-            r = launch_persistent_any(prec, kModeCount, a, pblocks, s);
+            // sources whose regions are small against the zones, then the
+            // rest of them, as in a single match
+            int32_t* const left = (int32_t*)(B.small + 6) + 1;
+            ScanArgs q = a;
+            q.queue = (unsigned int*)(B.small + 7);
+            const unsigned gs = (unsigned)std::min<int64_t>(8LL * sms, (total + 127) / 128);
+            if (prec == XM_PREC_FP32_RECHECK)
+                XM_LAUNCH("k_scan_src", gs, kScanThreads, (kSrcSmem<kPrecFP32, true>), s,
+                          (k_scan_src<kPrecFP32, true>), q, B.lists + 3 * nn, left);
+            else
+                XM_LAUNCH("k_scan_src_fp64", gs, kScanThreads, (kSrcSmem<kPrecFP64, true>), s,
+                          (k_scan_src<kPrecFP64, true>), q, B.lists + 3 * nn, left);
+            q = a;
+            q.list = B.lists + 3 * nn;
+            q.nlist_dev = left;
+            r = launch_persistent_any(prec, kModeCount, q, pblocks, s);
             if (r != XM_OK) return r;
         }
         r = sum_words ? count_scan(B.count, B.pair_off, total, B.small + 0, B.pair_off + nn, s)

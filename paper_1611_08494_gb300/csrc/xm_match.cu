@@ -89,11 +89,11 @@ xm_status launch_scan_src(int prec, const ScanArgs& a, int32_t* defer, int32_t* 
     if (g > 8LL * sms) g = 8LL * sms;
     if (g < 1) g = 1;
     if (prec == XM_PREC_FP32_RECHECK)
-        XM_LAUNCH("k_scan_src", (unsigned)g, kScanThreads, kSrcSmem<kPrecFP32>, s,
-                  k_scan_src<kPrecFP32>, a, defer, n_defer);
+        XM_LAUNCH("k_scan_src", (unsigned)g, kScanThreads, (kSrcSmem<kPrecFP32, false>), s,
+                  (k_scan_src<kPrecFP32, false>), a, defer, n_defer);
     else
-        XM_LAUNCH("k_scan_src_fp64", (unsigned)g, kScanThreads, kSrcSmem<kPrecFP64>, s,
-                  k_scan_src<kPrecFP64>, a, defer, n_defer);
+        XM_LAUNCH("k_scan_src_fp64", (unsigned)g, kScanThreads, (kSrcSmem<kPrecFP64, false>), s,
+                  (k_scan_src<kPrecFP64, false>), a, defer, n_defer);
     return XM_OK;
 }
 

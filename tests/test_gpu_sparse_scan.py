@@ -196,3 +196,42 @@ def test_sparse_count_pass_equals_the_general_scan(xm, n_a, members, frame, prec
             np.testing.assert_array_equal(_host(getattr(got, f)), _host(getattr(ref, f)), err_msg=f)
         for f in ("sep", "best_sep"):
             np.testing.assert_allclose(_host(getattr(got, f)), _host(getattr(ref, f)), rtol=0, atol=tol)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("order", [0, 1])
+def test_sparse_count_pass_of_a_batch(xm, prec, order):
+    """Requests of every shape, with one size and with sizes by source (small
+    and too large for the pass mixed), whose edges lie inside chunks: rows and
+    counts equal those of each request matched alone, separations to the error
+    of the path, and both passes ran."""
+    g = np.random.Generator(np.random.Philox(key=9))
+    lon, lat = g.uniform(20.0, 22.0, 40_000), g.uniform(-1.0, 1.0, 40_000)
+    idx = xm.Index(_cuda(lon), _cuda(lat), zone_height_arcsec=ZONE_H, build_fp64=prec == xm.PREC_FP64)
+    reqs = []
+    for k, n in enumerate((1, 31, 700, 33, 2500, 64, 5)):
+        pick = g.integers(0, lon.size, n)
+        q = dict(lon=_cuda(lon[pick] + g.normal(0.0, 5e-4, n)), lat=_cuda(lat[pick] + g.normal(0.0, 5e-4, n)),
+                 shape=k % 3)
+        if k % 2:
+            q.update(a_col=_cuda(g.uniform(0.5, 20.0, n)), b_col=_cuda(g.uniform(0.5, 8.0, n)),
+                     pa_col=_cuda(g.uniform(0.0, 180.0, n)))
+        else:
+            q.update(a=2.0 + k, b=1.5, pa=35.0)
+        reqs.append(q)
+    xm.prof_enable(True)
+    try:
+        batch = xm.Batch(idx, reqs, precision=prec, a_order=xm.A_ORDER_SORTED if order else xm.A_ORDER_INPUT)
+        got = [batch.view(r) for r in range(batch.n)]
+        prof = xm.prof_all()
+    finally:
+        xm.prof_enable(False)
+    assert prof["k_scan_src" if prec == xm.PREC_FP32 else "k_scan_src_fp64"][1] == 1
+    tol = SEP_TOL if prec == xm.PREC_FP32 else 1e-9
+    for q, v in zip(reqs, got):
+        q = dict(q)
+        ref = xm.Result(idx, q.pop("lon"), q.pop("lat"), precision=prec, a_order=xm.A_ORDER_SORTED, **q)
+        for f in ("a_row", "b_row", "count", "best_b"):
+            np.testing.assert_array_equal(_host(v[f]), _host(getattr(ref, f)), err_msg=f)
+        for f in ("sep", "best_sep"):
+            np.testing.assert_allclose(_host(v[f]), _host(getattr(ref, f)), rtol=0, atol=tol)
