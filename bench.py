@@ -1,7 +1,7 @@
 """Benchmark of the sky cross-match hot path (one JSON line on stdout).
 
 A step is one pass of the whole path over one synthetic workload: build the
-index of catalogue B (ingest, radix sort on (zone, RA), bucket tables, cell
+index of catalogue B (ingest, partition by zone and RA, bucket tables, cell
 offsets), match catalogue A against it with both selections (all pairs and
 best pair), and build the "1 or 2" join rows. The workload is the largest
 single-GPU configuration: the all-sky circle cross-match, A = 5e7 against
@@ -356,6 +356,8 @@ KERNEL_SOURCES = {
     "k_scan_src": ("xm_scan.cuh", "xm_internal.cuh"),
     "k_gather_b": ("xm_index.cu", "xm_internal.cuh"),
     "k_ingest_b": ("xm_index.cu", "xm_internal.cuh"),
+    "k_split": ("xm_index.cu", "xm_internal.cuh"),
+    "k_place_b": ("xm_index.cu", "xm_internal.cuh"),
 }
 
 
@@ -965,7 +967,7 @@ def values_leg(args, xm, torch):
                           sorted(prof.items(), key=lambda kv: -kv[1][0])[:6]}}
     sw = prof.get("k_onesweep")
     if sw:
-        alg = 24.0 * xm.stats()["sort_key_passes"] / sw[1]  # key and row, read and written
+        alg = 16.0 * xm.stats()["sort_key_passes"] / sw[1]  # packed words, read and written
         ach = alg / (sw[0] / sw[1] * 1e-3) / 1e9
         out["roofline"] = {"kernel": "k_onesweep", "bound": "hbm", "algorithmic_bytes": alg,
                            "ms_per_launch": sw[0] / sw[1], "achieved": ach, "peak": peak,
@@ -1200,10 +1202,9 @@ def algorithmic_bytes(kernel, st, steps, launches, n_a, n_b, region):
     """Bytes the method must move per launch of a kernel (averaged over the
     launches, so achieved = all bytes / all kernel time):
     k_onesweep   per key and pass 8 B key + 4 B row, read and written, over
-                 the passes that ran (the library counts keys x passes; an
-                 index sort planned to fewer passes launches the rest empty),
-                 and 8 B more each way for keys that carry a payload (the
-                 index sort carries each record's float32 offsets);
+                 the passes that ran (the library counts keys x passes), and
+                 8 B more each way for keys that carry a payload (none does
+                 now);
     k_scan_fp32_count, k_scan_src (the count pass, warp-cooperative or one
                  lane per source)  per A 16 B position + 8 B per region column given per
                  source + 16 B best pair, per candidate 12 B (offsets + RA
@@ -1211,7 +1212,10 @@ def algorithmic_bytes(kernel, st, steps, launches, n_a, n_b, region):
     k_prep_a     per A 16 B position (+ region columns) read, 88 B of
                  prepared record written;
     k_gather_b   per B 8 B key + 4 B row + 8 B offsets read, 16 B record
-                 written."""
+                 written (no kernel of this library any more);
+    k_ingest_b   per B 16 B position read, 16 B record and 16 B position
+                 written;
+    k_split, k_place_b   per B the 16 B record, read and written."""
     cols = sum(1 for k in ("a_col", "b_col", "pa_col") if region.get(k) is not None)
     if kernel == "k_onesweep":
         return (24.0 * st["sort_key_passes"] + 16.0 * st.get("sort_pay_passes", 0)) / launches
@@ -1221,6 +1225,10 @@ def algorithmic_bytes(kernel, st, steps, launches, n_a, n_b, region):
         return n_a * (16 + 8 * cols + 88) * steps / launches
     if kernel == "k_gather_b":
         return n_b * (8 + 4 + 8 + 16) * steps / launches
+    if kernel == "k_ingest_b":
+        return n_b * (16 + 16 + 16) * steps / launches
+    if kernel in ("k_split", "k_place_b"):
+        return n_b * (16 + 16) * steps / launches
     return None
 
 

@@ -60,7 +60,7 @@ constexpr int kMaxUnits = 2048, kMaxBins = 1024, kMaxDigits = 1536;
 constexpr int kBinZoneBits = 11;
 
 // Three blocks of 384 threads an SM, 3072 records a tile. Bound by latency and
-// instruction issue (all-sky index, 2e8 sources: ingest 3.57 ms, second split
+// instruction issue (all-sky index, 2e8 sources: ingest 2.90 ms, second split
 // 2.20 ms, at 0.4 of the copy bandwidth by their 48 and 32 bytes a source); two
 // blocks of 512 with 4096 records measured within 7 % of it.
 constexpr int kSplitThreads = 384;
