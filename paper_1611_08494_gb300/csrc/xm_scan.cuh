@@ -1717,6 +1717,21 @@ __global__ void k_seg_permute(const uint32_t* __restrict__ vals, int64_t n,
     s_out[i] = s_in[vals[i]];
 }
 
+// k_scan_src's blocks stay for the whole kernel, with the split of an SM's
+// memory between L1 and shared memory that they found: without a preference an
+// SM may keep the one of the kernel before (k_place_b's leaves a small L1), and
+// one all-sky pass in three took 4.8 to 5.0 ms instead of 3.4.
+template <int PREC, bool PREP>
+void prepare_scan_src() {
+    constexpr size_t smem = kSrcSmem<PREC, PREP>;
+    cudaFuncSetAttribute(k_scan_src<PREC, PREP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
+    // six blocks (with the 1 KB each reserves and the static part), of 228 KB
+    constexpr int percent = (int)((6 * (smem + 1536) * 100 + 228 * 1024 - 1) / (228 * 1024));
+    cudaFuncSetAttribute(k_scan_src<PREC, PREP>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                         percent < 100 ? percent : 100);
+}
+
 // Shared-memory limits of this translation unit's scan kernels and of the
 // sort, set once per device (thread-safe; before any capture that scans).
 void prepare_kernels() {
@@ -1737,14 +1752,10 @@ void prepare_kernels() {
     cudaFuncSetAttribute(k_scan<kPrecFP32, kModeResolve, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     cudaFuncSetAttribute(k_scan<kPrecFP64, kModeCount, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     cudaFuncSetAttribute(k_scan<kPrecFP64, kModeEmit, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    cudaFuncSetAttribute(k_scan_src<kPrecFP32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kSrcSmem<kPrecFP32, false>);
-    cudaFuncSetAttribute(k_scan_src<kPrecFP32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kSrcSmem<kPrecFP32, true>);
-    cudaFuncSetAttribute(k_scan_src<kPrecFP64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kSrcSmem<kPrecFP64, false>);
-    cudaFuncSetAttribute(k_scan_src<kPrecFP64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kSrcSmem<kPrecFP64, true>);
+    prepare_scan_src<kPrecFP32, false>();
+    prepare_scan_src<kPrecFP32, true>();
+    prepare_scan_src<kPrecFP64, false>();
+    prepare_scan_src<kPrecFP64, true>();
     radix_sort_prepare();
     done[dev] = true;
 }
