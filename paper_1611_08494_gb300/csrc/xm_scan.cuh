@@ -945,11 +945,11 @@ constexpr size_t kScanSmem = sizeof(ScanWarpSmem) * kScanWarps;
 // Bound by the latency of a chunk's dependent loads (position, zone, bucket
 // table, records), which 24 warps an SM overlap; testing every record where it
 // lay, a lane per source, took eight to ten divergent rounds instead of the
-// one. 3.5 ms for 5e7 sources against 2e8 (4.8 before), 0.73 for 1e7 against
-// 1e8 (0.99); float64, 5e6 against 2e7: 0.51 ms and 0.07 for the rest (1.17
-// with k_scan alone). Six blocks an SM with two rounds in flight: the shared
-// memory of seven or eight, or of four rounds, leaves the L1 too small for the
-// zones' records (3.6 to 5.6 ms).
+// one. 3.4 ms for 5e7 sources against 2e8 (4.8 before), 0.72 for 1e7 against
+// 1e8 (0.99); float64, 5e6 against 2e7: 0.49 ms and 0.07 for the rest (1.17
+// with k_scan alone). Six blocks an SM with two rounds in flight: five take 3.7
+// ms, seven 3.6, eight 5.9 and four rounds 3.8, by the registers spilled or by
+// the L1 that their shared memory leaves to the zones' records.
 
 constexpr int kSrcMaxRec = 48;  // records a lane takes on; more go to k_scan
 constexpr int kSrcStage = 64;   // members staged
