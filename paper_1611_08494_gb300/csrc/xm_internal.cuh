@@ -736,7 +736,7 @@ xm_status exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t
 // Prefix sums of many member counts (n >= kCountScanMin) in three launches
 // that wait on nothing: tile sums, their prefix, the elements. The chained
 // form advances a tile per 27 ns whatever the bandwidth (0.27 ms for 5e7
-// counts, and as long again in the join, which needs the zeros: 0.20 ms here
+// counts, and as long again in the join, which needs the zeros: 0.22 ms here
 // for both), which costs more than two launches from some 3e5 counts on.
 // zeros[t]: the counts of zero before element kCountTile * t (a join's
 // unmatched sources), count_scan_words(n) words (0 below kCountScanMin).
