@@ -22,7 +22,7 @@
 //   k_split        (large catalogues) records of a bin grouped by unit
 //   k_place_b      per unit: RA buckets counted in shared memory, the zones'
 //                  bucket tables and the records in bucket order written
-// Up to about a million sources the bins are the units themselves and the
+// Up to some 4e5 sources the bins are the units themselves and the
 // steps marked "large catalogues" are left out.
 #include <math.h>
 #include <string.h>
@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "xm_lookback.cuh"
+#include "xm_plan.cuh"
 
 namespace xm {
 
@@ -39,25 +40,12 @@ namespace {
 
 constexpr int kBlock = 256;
 
-// Units: consecutive cells whose first rows fall in the same window of
-// 2^kUnitRowBits rows, of zones in the same kUnitZones, form one unit; a part
-// of a zone, and a cell of more rows than a window, begins a unit (which ends
-// with it: the next cell begins in a later window). So a unit of several
-// cells holds fewer than two windows' rows, and only a unit of one cell can
-// hold more than k_place_b stages. Zones of more than kPartMin sources are cut
-// into parts of half of kPartRows to kPartRows on average, so nearly every
-// unit fits the stage. (Unstaged, a block per zone reading its records twice
-// from L2, the placing of 2e8 records took 2.3 ms in zones of 7400 and 4 to 5
-// ms in zones of 22000 and more, whose records no longer stay in L2.)
-constexpr int kUnitRowBits = 9, kUnitZoneBits = 6;
-constexpr int kUnitZones = 1 << kUnitZoneBits;
+// Zones of more than kPartMin sources are cut into parts of half of kPartRows
+// to kPartRows on average, so nearly every unit (xm_plan.cuh) fits the stage.
+// (Unstaged, a block per zone reading its records twice from L2, the placing
+// of 2e8 records took 2.3 ms in zones of 7400 and 4 to 5 ms in zones of 22000
+// and more, whose records no longer stay in L2.)
 constexpr uint32_t kPartMin = 896, kPartRows = 800;
-
-// Digits of a split: the units of a small catalogue, or the bins of the first
-// of two splits, or the units of a bin in the second. A bin covers zones with
-// the same z >> kBinZoneBits (records carry the low bits of their zone).
-constexpr int kMaxUnits = 2048, kMaxBins = 1024, kMaxDigits = 1536;
-constexpr int kBinZoneBits = 11;
 
 // Three blocks of 384 threads an SM, 3072 records a tile. Bound by latency and
 // instruction issue (all-sky index, 2e8 sources: ingest 2.90 ms, second split
@@ -1200,19 +1188,10 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
     const bool deferred = opts && opts->deferred_check;
     const int64_t nn = n > 0 ? n : 1;
 
-    // The bins of one split are the units; past kMaxUnits units there are two
-    // splits, into 384 to 767 bins of 2^kb rows (at least a unit's window, so
-    // that units do not straddle bins) and those into units.
-    int64_t cells_cap = X->nz;
-    int64_t units_cap = 2 * (n >> kUnitRowBits) + (X->nz >> kUnitZoneBits) + 1;
-    const bool two = units_cap > kMaxUnits;
-    int kb = kUnitRowBits;
-    while (two && (n >> (kb + 1)) >= 384) kb++;
-    const int nbins = two ? (int)((n >> kb) + (X->nz >> kBinZoneBits) + 1) : 0;
-    if (two) {  // parts of zones: of half of kPartRows rows or more, of zones past kPartMin
-        cells_cap += n / 200 + 16;
-        units_cap += n / 160 + 16;
-    }
+    const BuildPlan plan = build_plan(n, X->nz);
+    const bool two = plan.two;
+    const int kb = plan.kb, nbins = plan.nbins;
+    const int64_t cells_cap = plan.cells_cap, units_cap = plan.units_cap;
 
     xm_status st = XM_OK;
     // temporaries: one block, the part that starts as zeros first
