@@ -1029,19 +1029,20 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_
     uint32_t n_cand = 0, n_mem = 0;
     int max_cnt = 0;
     // The region has a fixed size: its prepared terms are the same for every
-    // source, except when a frame rotation turns a region that is not a
-    // circle (the position angle then varies with the position). They are
-    // prepared once per block; each source adds its position.
+    // source, except where a region that is not a circle has an angle of its
+    // own (from a column, or a frame rotation, which turns it by position).
+    // They are prepared once per block; each source adds its position.
     const AIn& I = P.in;
-    const bool same_region = !I.rotate || I.shape == XM_CIRCLE;
+    const bool same_region = I.shape == XM_CIRCLE || (!I.rotate && !I.pa_col);
     __shared__ APrep s_at;
     __shared__ ACold s_ct;
     __shared__ double s_st, s_cos;
     if (!PREP && threadIdx.x == 0) {
         const double b = I.shape == XM_CIRCLE ? I.a : I.b;
+        const double pa = I.pa_col ? 0.0 : I.pa;
         APrep at;
         ACold ct;
-        make_aprep(0.0, 0.0, 0.0, true, I.a, b, I.pa, I.shape, I.pa_dir, I.size_k, I.pa_zero, I.nz,
+        make_aprep(0.0, 0.0, 0.0, true, I.a, b, pa, I.shape, I.pa_dir, I.size_k, I.pa_zero, I.nz,
                    I.h_f, 0, &at, &ct);
         s_at = at;
         s_ct = ct;
@@ -1050,7 +1051,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_
             s_st = t.st;
             s_cos = t.ct;
         }
-        if (blockIdx.x == 0 && P.nA > 0 && !size_ok(I.a, b, I.pa)) atomicOr(P.err, kErrSize);
+        if (blockIdx.x == 0 && P.nA > 0 && !size_ok(I.a, b, pa)) atomicOr(P.err, kErrSize);
     }
     W.mcnt[lane] = 0;
     __syncthreads();
@@ -1086,6 +1087,8 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_
                 bool ok;
                 a_position_of(lon0, lat0, I.rotate, I.rot, &lon, &lat, &gamma, &ok);
                 if (!ok) atomicOr(P.err, kErrCoord);
+                // (a circle's angle is checked and not used)
+                if (I.pa_col && !finite_bits(I.pa_col[s])) atomicOr(P.err, kErrSize);
                 const PosKey k = pos_key(lon, lat, I.nz);
                 A = s_at;
                 A.key64 = k.key64;
