@@ -389,6 +389,7 @@ struct xm_batch {
     cudaStream_t stream = nullptr;
     int64_t n_req, total_a, total_pairs, total_rows, n_b;
     int32_t precision;
+    int32_t max_count = 0;             // largest member count of any source
     std::vector<int64_t> off;          // [n_req + 1]
     std::vector<int64_t> bounds;       // 4 per request
     std::vector<int64_t> un_a, un_b;   // per request
@@ -741,6 +742,7 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
             st = set_error(XM_ETIMEOUT, "batch sort: look-back timed out");
         if (st == XM_OK) {
             out->total_pairs = h_small[0];
+            out->max_count = (int32_t)(h_small[6] & 0xffffffff);
             out->total_rows = want_rows ? h_small[1] : 0;
             const int64_t n_big = h_lists[2];
             if (out->total_pairs > pair_cap || out->total_rows > row_cap || (h_err & kErrOverflow))
@@ -958,6 +960,7 @@ extern "C" xm_status xm_batch_join(const xm_batch* X, int64_t r, void* stream, x
     view.device = X->device;
     view.selection = X->sel[r];
     view.precision = X->precision;
+    view.max_count = X->max_count;
     view.n_a = X->off[r + 1] - a0;
     view.n_b = X->n_b;
     view.n_pairs = X->bounds[4 * r + 1] - p0;

@@ -11,7 +11,8 @@
 // the result is deterministic); one pass over the A sources that knows the
 // unmatched ones before each and writes their rows, the best pairs or the
 // pairs (many pairs for each source: a pass of their own, each as many places
-// on as unmatched A rows come before it); one pass over the bitset that counts
+// on as unmatched A rows come before it; many for a few: left to a pass over a
+// list of them); one pass over the bitset that counts
 // the unmatched B rows before each word by a chained prefix sum and writes
 // them. xm_join_noalloc, which learns the row count before it writes, keeps
 // rows per source and per word and their prefix sums in its scratch array.
@@ -139,6 +140,8 @@ constexpr int kRowsA = 4;  // A sources per thread: 128 in a row per warp
 constexpr int kTileA = kRowsA * kBlock;
 static_assert(kTileA == kCountTile, "the match counts unmatched sources per tile");
 constexpr int kRowsThread = 16;  // pairs that a thread writes for its source
+constexpr int kRowsWarp = 512;   // pairs that a warp writes for its 32 sources
+constexpr int kRowsChunk = 4 * kBlock;  // pairs of a listed chunk
 
 // Exclusive prefix of v over the block; *all: the block's sum.
 __device__ __forceinline__ uint32_t block_prefix(uint32_t v, uint32_t* all) {
@@ -167,6 +170,14 @@ struct JoinTile {
     long long prefix;
 };
 
+// Pairs that the A-side pass leaves: [p0, p0 + n) of the 32 sources from i0 on,
+// before which `un` sources are unmatched, and of which those in `mask` are.
+struct __align__(32) PairChunk {
+    int64_t p0, un, i0;
+    uint32_t mask;
+    int32_t n;
+};
+
 // What the A-side pass reads and writes. counts: [0] A-side rows, [2]
 // unmatched A sources.
 struct JoinA {
@@ -182,6 +193,8 @@ struct JoinA {
     const int64_t* zeros;  // unmatched A sources before each tile (NULL: chained)
     int32_t rows;          // this pass writes the "all" selection's pair rows
     int32_t* un_before;    // (nullable) unmatched A sources before each source
+    PairChunk* chunks;     // (nullable: no source has more than kRowsThread pairs)
+    unsigned int* n_chunks;
     int64_t* oa;
     int64_t* ob;
     double* os;
@@ -194,7 +207,8 @@ struct JoinA {
 // of many sources, else they come from a chained prefix sum over tiles in
 // launch order. A thread writes the pairs of its own sources while no source
 // of the warp's 32 has more than kRowsThread, else the warp writes them a
-// pair per lane. Bound by memory: pair rows and unmatched rows share sectors,
+// pair per lane, or lists them for k_join_long where the 32 have more than
+// kRowsWarp. Bound by memory: pair rows and unmatched rows share sectors,
 // so they are written together, and nothing is kept per source between passes.
 // 0.50 ms for 5e7 sources, 3e7 pairs and 5.1e7 rows (2.8 GB, 5.6 TB/s) against
 // 1.3 ms in a pass for the rows of each source, their prefix sum, a pass over
@@ -280,6 +294,19 @@ __global__ void __launch_bounds__(kBlock) k_join_a(JoinA J, uint64_t* status, un
         int64_t p1 = c[k] > 0 ? at[k] + c[k] : 0;
 #pragma unroll
         for (int o = 16; o; o >>= 1) p1 = max(p1, __shfl_xor_sync(0xffffffffu, p1, o));
+        if (p1 - p0 > kRowsWarp) {
+            const int64_t un0 = __shfl_sync(0xffffffffu, un, 0);
+            const uint32_t n = (uint32_t)((p1 - p0 + kRowsChunk - 1) / kRowsChunk);
+            uint32_t base = 0;
+            if (lane == 0) base = atomicAdd(J.n_chunks, n);
+            base = __shfl_sync(0xffffffffu, base, 0);
+            for (uint32_t j = lane; j < n; j += 32) {
+                const int64_t q = p0 + (int64_t)j * kRowsChunk;
+                J.chunks[base + j] = PairChunk{q, un0, i - lane, un_mask[k],
+                                               (int32_t)min((int64_t)kRowsChunk, p1 - q)};
+            }
+            continue;
+        }
         for (int64_t q = p0; q < p1; q += 32) {
             const int64_t p = q + lane;
             int l = 0;  // the last source whose pairs start at p or before
@@ -293,6 +320,39 @@ __global__ void __launch_bounds__(kBlock) k_join_a(JoinA J, uint64_t* status, un
                 J.ob[o] = __ldcs(J.pb + p);
                 J.os[o] = __ldcs(J.ps + p);
             }
+        }
+    }
+}
+
+// The pair rows of the listed chunks, a block each: 12 us for a region of 1e6
+// members among 1e6 small ones, whose join takes 0.088 ms (26 ms with one warp
+// for all the pairs of its 32 sources). Where the longest takes a warp 3 us or
+// less, at kRowsThread members, nothing is launched.
+__global__ void __launch_bounds__(kBlock) k_join_long(JoinA J, const int64_t* __restrict__ pa) {
+    pdl_wait();
+    const unsigned int n = *J.n_chunks;
+    for (unsigned int c = blockIdx.x; c < n; c += gridDim.x) {
+        const PairChunk C = J.chunks[c];
+        int64_t a[4], b[4];
+        double v[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int32_t j = k * kBlock + threadIdx.x;
+            if (j < C.n) {
+                a[k] = __ldcs(pa + C.p0 + j);
+                b[k] = __ldcs(J.pb + C.p0 + j);
+                v[k] = __ldcs(J.ps + C.p0 + j);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int32_t j = k * kBlock + threadIdx.x;
+            if (j >= C.n) break;
+            const uint32_t below = (1u << ((uint32_t)(a[k] - C.i0) & 31u)) - 1u;
+            const int64_t o = C.p0 + j + (J.with_un_a ? C.un + __popc(C.mask & below) : 0);
+            J.oa[o] = a[k] + J.a_off;
+            J.ob[o] = b[k];
+            J.os[o] = v[k];
         }
     }
 }
@@ -614,20 +674,28 @@ static xm_status join_impl(const xm_result* R, int32_t selection, int32_t join_t
     // each, 2e5 sources: 26 us in two passes, 48 to 70 in one).
     const bool pair_rows = sel_all && with_pairs && R->n_pairs > 0 && R->a_row;
     const bool apart = pair_rows && R->n_pairs > 4 * nA;
+    // Where a few sources have very many, their pairs go to a list: room for
+    // two chunks per kRowsChunk pairs, as the listed 32 have more than half.
+    const bool listed = pair_rows && !apart && R->n_pairs > kRowsWarp &&
+                        (R->max_count == 0 || R->max_count > kRowsThread);
+    static_assert(2 * kRowsWarp >= kRowsChunk, "chunks of the listed sources fit their list");
+    const int64_t max_chunks = listed ? R->n_pairs / kRowsWarp : 0;
     // one work block: the chained sums' status words and tile counters and the
     // matched B rows (all of which start as zeros), then the unmatched A
-    // sources before each one, where a pass of its own writes the pair rows
+    // sources before each one, where a pass of its own writes the pair rows, or
+    // the list
     const int64_t tiles_a = (nA + kTileA - 1) / kTileA, tiles_b = (nwords + kBlock - 1) / kBlock;
     auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
-    const size_t o_bits = up((tiles_a + tiles_b + 1) * sizeof(uint64_t));
+    const size_t o_bits = up((tiles_a + tiles_b + 2) * sizeof(uint64_t));
     const size_t zeroed = o_bits + (ext_bits ? 0 : up(nwords * sizeof(uint32_t)));
     unsigned char* work = (unsigned char*)dev_alloc(
-        zeroed + (apart && with_un_a ? nA * sizeof(int32_t) : 0), s);
+        zeroed + (apart && with_un_a ? nA * sizeof(int32_t) : max_chunks * sizeof(PairChunk)), s);
     uint64_t* const status = (uint64_t*)work;
     unsigned int* const counter = work ? (unsigned int*)(status + tiles_a + tiles_b) : nullptr;
     uint32_t* const own_bits = ext_bits || !work ? nullptr : (uint32_t*)(work + o_bits);
     const uint32_t* bits = ext_bits ? ext_bits : own_bits;
     int32_t* const un_before = apart && with_un_a && work ? (int32_t*)(work + zeroed) : nullptr;
+    PairChunk* const chunks = listed && work ? (PairChunk*)(work + zeroed) : nullptr;
     // counts read later by xm_rows_get: [0] A-side rows, [1] unmatched B,
     // [2] unmatched A, [4] error bits
     int64_t* small = (int64_t*)dev_alloc(5 * sizeof(int64_t), s);
@@ -662,9 +730,13 @@ static xm_status join_impl(const xm_result* R, int32_t selection, int32_t join_t
         if (nA > 0) {
             const JoinA P{R->count, R->pair_off, R->b_row, R->sep, R->best_b, R->best_sep, nA,
                           R->n_pairs, sel_all, with_pairs, with_un_a, a_off, R->zeros,
-                          pair_rows && !apart, un_before, J->a_row, J->b_row, J->sep, small};
+                          pair_rows && !apart, un_before, chunks, counter + 2, J->a_row, J->b_row,
+                          J->sep, small};
             XM_LAUNCH("k_join_a", (unsigned)tiles_a, kBlock, 0, s, k_join_a, P, status, counter, lb,
                       err);
+            if (listed)
+                XM_LAUNCH("k_join_long", (unsigned)(max_chunks < 4 * 152 ? max_chunks : 4 * 152),
+                          kBlock, 0, s, k_join_long, P, R->a_row);
         }
         if (apart)
             XM_LAUNCH("k_join_pairs", grid_for((R->n_pairs + 3) / 4), kBlock, 0, s, k_join_pairs,

@@ -514,6 +514,7 @@ xm_status xm_pending::finish() {
     if (h_small[0] & kErrTimeout) return set_error(XM_ETIMEOUT, "A sort: look-back timed out");
     const int64_t n_ovf = h_small[1], n_tie = h_small[2], n_big = h_small[3];
     R->n_pairs = want_all ? h_total[0] : 0;
+    R->max_count = h_small[6];
     xm_status r = XM_OK;
 
     // near ties of the best pair, decided in float64 on the side stream

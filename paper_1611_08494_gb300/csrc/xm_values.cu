@@ -176,7 +176,8 @@ template <bool HASHED>
 __global__ void __launch_bounds__(kBlock) k_val_probe(
     const void* __restrict__ a_keys, int64_t n_a, int32_t type, const uint64_t* __restrict__ sorted,
     const void* __restrict__ b_keys, int64_t n_b, ValLut V, int32_t* __restrict__ count,
-    int64_t* __restrict__ first, int64_t* __restrict__ best_b, double* __restrict__ best_sep) {
+    int64_t* __restrict__ first, int64_t* __restrict__ best_b, double* __restrict__ best_sep,
+    int32_t* max_count) {
     pdl_wait();
     const int64_t i0 = (int64_t)blockIdx.x * (kProbeKeys * kBlock) + threadIdx.x;
     uint64_t c[kProbeKeys];
@@ -252,7 +253,9 @@ __global__ void __launch_bounds__(kBlock) k_val_probe(
                 break;
             }
         }
-        count[i] = (int32_t)(m < 2147483647 ? m : 2147483647);
+        const int32_t c32 = (int32_t)(m < 2147483647 ? m : 2147483647);
+        count[i] = c32;
+        if (c32 > 1 && c32 > *(volatile const int32_t*)max_count) atomicMax(max_count, c32);
         first[i] = m == 1 ? best : f;
         if (best_b) {
             best_b[i] = best;
@@ -342,7 +345,7 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
     void* d_b = nullptr;
     uint64_t* packed = (uint64_t*)dev_alloc(2 * nb1 * sizeof(uint64_t), s);
     int64_t* first = (int64_t*)dev_alloc(na1 * sizeof(int64_t), s);
-    unsigned long long* small = (unsigned long long*)dev_alloc(4 * sizeof(unsigned long long), s);
+    unsigned long long* small = (unsigned long long*)dev_alloc(5 * sizeof(unsigned long long), s);
     uint32_t* lut = nullptr;
     ValRun* runs = nullptr;
     auto body = [&]() -> xm_status {
@@ -362,8 +365,9 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
             ak = d_a;
             bk = d_b;
         }
-        // small: [0] AND of codes, [1] OR, [2] pair total, [3] error bits
-        const unsigned long long init[4] = {~0ull, 0ull, 0ull, 0ull};
+        // small: [0] AND of codes, [1] OR, [2] pair total, [3] error bits, [4]
+        // largest count above 1
+        const unsigned long long init[5] = {~0ull, 0ull, 0ull, 0ull, 0ull};
         e = cudaMemcpyAsync(small, init, sizeof(init), cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return cuda_fail(e, "xm_match_values: init");
         int32_t* err = (int32_t*)(small + 3);
@@ -413,20 +417,21 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
         const unsigned gp = grid_of((n_a + kProbeKeys - 1) / kProbeKeys);
         if (n_a > 0 && hashed)
             XM_LAUNCH("k_val_probe", gp, kBlock, 0, s, k_val_probe<true>, ak, n_a, key_type, packed, bk,
-                      n_b, V, R->count, first, R->best_b, R->best_sep);
+                      n_b, V, R->count, first, R->best_b, R->best_sep, (int32_t*)(small + 4));
         else if (n_a > 0)
             XM_LAUNCH("k_val_probe", gp, kBlock, 0, s, k_val_probe<false>, ak, n_a, key_type, packed, bk,
-                      n_b, V, R->count, first, R->best_b, R->best_sep);
+                      n_b, V, R->count, first, R->best_b, R->best_sep, (int32_t*)(small + 4));
         xm_status r = R->zeros ? count_scan(R->count, R->pair_off, n_a, (int64_t*)(small + 2), R->zeros, s)
                                : exclusive_scan_i32(R->count, R->pair_off, n_a, (int64_t*)(small + 2),
                                                     err, s);
         if (r != XM_OK) return r;
-        unsigned long long h[2] = {0, 0};
+        unsigned long long h[3] = {0, 0, 0};
         e = cudaMemcpyAsync(h, small + 2, sizeof(h), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return cuda_fail(e, "xm_match_values sync");
         if ((int32_t)h[1] & kErrTimeout) return set_error(XM_ETIMEOUT, "xm_match_values: look-back timed out");
         if ((int32_t)h[1] & kErrOverflow) return set_error(XM_ECUDA, "xm_match_values: run list overflow");
+        R->max_count = h[2] ? (int32_t)h[2] : 1;
         R->n_pairs = (selection & XM_SEL_ALL) ? (int64_t)h[0] : 0;
         if (selection & XM_SEL_ALL) {
             const int64_t np = R->n_pairs > 0 ? R->n_pairs : 1;
