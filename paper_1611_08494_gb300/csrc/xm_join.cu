@@ -193,7 +193,7 @@ struct JoinA {
     const int64_t* zeros;  // unmatched A sources before each tile (NULL: chained)
     int32_t rows;          // this pass writes the "all" selection's pair rows
     int32_t* un_before;    // (nullable) unmatched A sources before each source
-    PairChunk* chunks;     // (nullable: no source has more than kRowsThread pairs)
+    PairChunk* chunks;
     unsigned int* n_chunks;
     int64_t* oa;
     int64_t* ob;
@@ -206,13 +206,14 @@ struct JoinA {
 // "all" selection. The unmatched ones before a tile are known from the match
 // of many sources, else they come from a chained prefix sum over tiles in
 // launch order. A thread writes the pairs of its own sources while no source
-// of the warp's 32 has more than kRowsThread, else the warp writes them a
-// pair per lane, or lists them for k_join_long where the 32 have more than
-// kRowsWarp. Bound by memory: pair rows and unmatched rows share sectors,
+// of the warp's 32 has more than kRowsThread, else (MANY: where the match may
+// have counted such a source) the warp writes them a pair per lane, or lists
+// them for k_join_long where the 32 have more than kRowsWarp. Bound by memory: pair rows and unmatched rows share sectors,
 // so they are written together, and nothing is kept per source between passes.
 // 0.50 ms for 5e7 sources, 3e7 pairs and 5.1e7 rows (2.8 GB, 5.6 TB/s) against
 // 1.3 ms in a pass for the rows of each source, their prefix sum, a pass over
 // the pairs and one over the sources.
+template <bool MANY>
 __global__ void __launch_bounds__(kBlock) k_join_a(JoinA J, uint64_t* status, unsigned int* counter,
                                                    Lookback lb, int32_t* err) {
     pdl_wait();
@@ -279,7 +280,7 @@ __global__ void __launch_bounds__(kBlock) k_join_a(JoinA J, uint64_t* status, un
         }
         if (J.un_before && c[k] >= 0) J.un_before[i] = (int32_t)un;
         if (!J.rows) continue;
-        if (__reduce_max_sync(0xffffffffu, c[k]) <= kRowsThread) {
+        if (!MANY || __reduce_max_sync(0xffffffffu, c[k]) <= kRowsThread) {
             const int64_t o = at[k] + (J.with_un_a ? un : 0);
 #pragma unroll 1
             for (int32_t j = 0; j < c[k]; j++) {
@@ -326,8 +327,8 @@ __global__ void __launch_bounds__(kBlock) k_join_a(JoinA J, uint64_t* status, un
 
 // The pair rows of the listed chunks, a block each: 12 us for a region of 1e6
 // members among 1e6 small ones, whose join takes 0.088 ms (26 ms with one warp
-// for all the pairs of its 32 sources). Where the longest takes a warp 3 us or
-// less, at kRowsThread members, nothing is launched.
+// for all the pairs of its 32 sources). Where no source has more than
+// kRowsThread, no 32 of them have more than kRowsWarp: nothing is launched.
 __global__ void __launch_bounds__(kBlock) k_join_long(JoinA J, const int64_t* __restrict__ pa) {
     pdl_wait();
     const unsigned int n = *J.n_chunks;
@@ -676,8 +677,8 @@ static xm_status join_impl(const xm_result* R, int32_t selection, int32_t join_t
     const bool apart = pair_rows && R->n_pairs > 4 * nA;
     // Where a few sources have very many, their pairs go to a list: room for
     // two chunks per kRowsChunk pairs, as the listed 32 have more than half.
-    const bool listed = pair_rows && !apart && R->n_pairs > kRowsWarp &&
-                        (R->max_count == 0 || R->max_count > kRowsThread);
+    const bool many = pair_rows && !apart && (R->max_count == 0 || R->max_count > kRowsThread);
+    const bool listed = many && R->n_pairs > kRowsWarp;
     static_assert(2 * kRowsWarp >= kRowsChunk, "chunks of the listed sources fit their list");
     const int64_t max_chunks = listed ? R->n_pairs / kRowsWarp : 0;
     // one work block: the chained sums' status words and tile counters and the
@@ -732,8 +733,12 @@ static xm_status join_impl(const xm_result* R, int32_t selection, int32_t join_t
                           R->n_pairs, sel_all, with_pairs, with_un_a, a_off, R->zeros,
                           pair_rows && !apart, un_before, chunks, counter + 2, J->a_row, J->b_row,
                           J->sep, small};
-            XM_LAUNCH("k_join_a", (unsigned)tiles_a, kBlock, 0, s, k_join_a, P, status, counter, lb,
-                      err);
+            if (many)
+                XM_LAUNCH("k_join_a", (unsigned)tiles_a, kBlock, 0, s, k_join_a<true>, P, status,
+                          counter, lb, err);
+            else
+                XM_LAUNCH("k_join_a", (unsigned)tiles_a, kBlock, 0, s, k_join_a<false>, P, status,
+                          counter, lb, err);
             if (listed)
                 XM_LAUNCH("k_join_long", (unsigned)(max_chunks < 4 * 152 ? max_chunks : 4 * 152),
                           kBlock, 0, s, k_join_long, P, R->a_row);
