@@ -24,6 +24,7 @@
 //                  bucket tables and the records in bucket order written
 // Up to some 4e5 sources the bins are the units themselves and the
 // steps marked "large catalogues" are left out.
+#include <cooperative_groups.h>
 #include <math.h>
 #include <string.h>
 
@@ -216,6 +217,28 @@ __device__ __forceinline__ int64_t tile_prefix(PreTile& S, int64_t tile, const i
     return S.prefix + mine;
 }
 
+// Calls f(i, lo, a, b, c) for every i of each lane's [lo, hi): a lane its own
+// few, the whole warp those of a lane with many (a zone of thousands of parts
+// kept one thread busy for 0.37 ms; dozens, as a lane each has in a dense
+// catalogue, are faster its own). Called by whole warps.
+template <typename F>
+__device__ __forceinline__ void warp_fill(uint32_t lo, uint32_t hi, uint32_t a, uint32_t b, uint32_t c,
+                                          F&& f) {
+    constexpr uint32_t kFew = 128;
+    const bool many = hi > lo && hi - lo > kFew;
+    if (!many)
+        for (uint32_t i = lo; i < hi; i++) f(i, lo, a, b, c);
+    uint32_t todo = __ballot_sync(0xffffffffu, many);
+    while (todo) {
+        const int l = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const uint32_t l0 = __shfl_sync(0xffffffffu, lo, l), l1 = __shfl_sync(0xffffffffu, hi, l);
+        const uint32_t la = __shfl_sync(0xffffffffu, a, l), lb = __shfl_sync(0xffffffffu, b, l),
+                       lc = __shfl_sync(0xffffffffu, c, l);
+        for (uint32_t i = l0 + (threadIdx.x & 31); i < l1; i += 32) f(i, l0, la, lb, lc);
+    }
+}
+
 // First row of each zone, and the bins of the first split (two splits):
 // zones whose first rows share row >> kb, and whose numbers share
 // z >> kBinZoneBits.
@@ -335,16 +358,17 @@ __global__ void __launch_bounds__(kBlock) k_zone_parts(
 #pragma unroll
     for (int k = 0; k < kPreItems; k++) {
         const int64_t z = z0 + k;
-        if (z >= nz) break;
         const uint32_t first = (uint32_t)(run & 0x7FFFFFFF), split = (uint32_t)(run >> 31);
-        const uint32_t parts = (uint32_t)(v[k] & 0x7FFFFFFF);
-        zcells[z] = ZoneCells{first, parts, parts > 1 ? kmin >> sh[k] : 0, sh[k]};
-        for (uint32_t p = 0; p < parts && first + p < cells_cap; p++) {
-            cell_zone[first + p] = (uint32_t)z;
-            // parts are units of their own: each part (marked in the top
-            // bit), and the zone after them, starts a unit
-            cell_split[first + p] = parts > 1 ? (split + p + 1) | 0x80000000u : split;
-        }
+        const uint32_t parts = (uint32_t)(v[k] & 0x7FFFFFFF);  // (0 past the zones)
+        if (parts) zcells[z] = ZoneCells{first, parts, parts > 1 ? kmin >> sh[k] : 0, sh[k]};
+        warp_fill(first, first + parts, (uint32_t)z, split, parts > 1,
+                  [&](uint32_t c, uint32_t c0, uint32_t zc, uint32_t sp, uint32_t many) {
+                      if (c >= cells_cap) return;
+                      cell_zone[c] = zc;
+                      // parts are units of their own: each part (marked in the
+                      // top bit), and the zone after them, starts a unit
+                      cell_split[c] = many ? (sp + (c - c0) + 1) | 0x80000000u : sp;
+                  });
         run += v[k];
         if (z == nz - 1) *n_cells = min((uint32_t)(run & 0x7FFFFFFF), cells_cap);
     }
@@ -391,18 +415,24 @@ __global__ void __launch_bounds__(kBlock) k_cell_units(
 #pragma unroll
     for (int k = 0; k < kPreItems; k++) {
         const int64_t c = c0 + k;
-        if (c >= n_cells) break;
-        wide += v[k] >> 31;
-        const int64_t u = unit_of(c, start, wide);
-        cell_start[c] = (uint32_t)start;
-        cell_unit[c] = (uint32_t)u;
-        if (zin) write_zone_in(geo, zin, c, (uint32_t)u);
-        const uint32_t z = cell_zone ? cell_zone[c] : (uint32_t)c;
-        for (int64_t i = up + 1; i <= u && i < unit_cap; i++) {  // (ids skipped: empty units)
-            unit[i] = make_uint4((uint32_t)c, z, (uint32_t)start, 0);
-            ucur[i * kCursorStep] = (uint32_t)start;
+        const bool on = c < n_cells;
+        uint32_t z = 0;
+        int64_t u = up;
+        if (on) {
+            wide += v[k] >> 31;
+            u = unit_of(c, start, wide);
+            cell_start[c] = (uint32_t)start;
+            cell_unit[c] = (uint32_t)u;
+            if (zin) write_zone_in(geo, zin, c, (uint32_t)u);
+            z = cell_zone ? cell_zone[c] : (uint32_t)c;
         }
-        if (c == (int64_t)n_cells - 1) {
+        // (ids skipped, after a cell of many rows: empty units)
+        warp_fill((uint32_t)(up + 1), (uint32_t)min(u + 1, (int64_t)unit_cap), (uint32_t)c, z,
+                  (uint32_t)start, [&](uint32_t i, uint32_t, uint32_t uc, uint32_t uz, uint32_t us) {
+                      unit[i] = make_uint4(uc, uz, us, 0);
+                      ucur[(int64_t)i * kCursorStep] = us;
+                  });
+        if (on && c == (int64_t)n_cells - 1) {
             cell_start[n_cells] = (uint32_t)n;
             const int64_t nu = min(u + 1, (int64_t)unit_cap);
             unit[nu] = make_uint4(n_cells, 0, (uint32_t)n, 0);
@@ -533,6 +563,20 @@ __device__ __forceinline__ uint32_t count_digit(uint32_t* cnt, int32_t d) {
         return (uint32_t)d << 16 | (__shfl_sync(0xffffffffu, base, 0) + lane);
     }
     return d < 0 ? kNoRecord : (uint32_t)d << 16 | atomicAdd(&cnt[d], 1u);
+}
+
+// Places for the warp's records in c[step * i], one atomic per distinct i: the
+// first of the lane's run, and the record's rank in it. (2e6 atomics on one
+// counter take 1.3 ms.)
+__device__ __forceinline__ uint32_t claim_places(uint32_t* c, int step, uint32_t i, bool on,
+                                                 uint32_t* rank) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t peers = __match_any_sync(0xffffffffu, on ? i : 0xFFFFFFFFu);
+    const int first = __ffs(peers) - 1;
+    uint32_t base = 0;
+    if (on && lane == first) base = atomicAdd(&c[(int64_t)i * step], (uint32_t)__popc(peers));
+    *rank = (uint32_t)__popc(peers & ((1u << lane) - 1u));
+    return __shfl_sync(0xffffffffu, base, first);
 }
 
 // Ingest of B: validity, longitude mod 360, the exact position kept by row,
@@ -677,8 +721,10 @@ __global__ void __launch_bounds__(kSplitThreads) k_cell_count(
         if (h[i]) atomicAdd(&ccnt[first + i], h[i]);
 }
 
-// The second split: a tile of one bin's records grouped by unit. (A bin of
-// more units than a tile counts claims every record's place by itself.)
+// The second split: a tile of one bin's records grouped by unit. (A bin of more
+// units than a tile counts -- of a zone of about a million rows, or after a cell
+// of as many -- claims the places of a warp's records at a time: in pieces of
+// kMaxDigits units it took as long.)
 __global__ void __launch_bounds__(kSplitThreads, 3) k_split(
     const uint4* __restrict__ rec, const uint4* __restrict__ tiles, const uint32_t* n_tiles, int nbins,
     const uint32_t* __restrict__ bin_zone, const ZoneCells* __restrict__ zcells,
@@ -704,14 +750,14 @@ __global__ void __launch_bounds__(kSplitThreads, 3) k_split(
     const uint32_t u0 = cell_unit[zcells[z0].first];
     const uint32_t z1 = b + 1 < nbins ? bin_zone[b + 1] : 0;
     const uint32_t nd = (z1 > z0 ? cell_unit[zcells[z1].first] : *n_units) - u0;
-    if (nd > kMaxDigits) {  // (rare: every record claims its place by itself)
+    if (nd > kMaxDigits) {
 #pragma unroll
         for (int k = 0; k < kTileItems; k++) {
-            if (lo + tid + k * kSplitThreads >= hi) break;
-            const ZoneCells Z = load_cells(zcells + (zhi + wide_tag(r[k])));
-            const uint32_t u = __ldg(cell_unit + cell_of(Z, r[k].z));
-            const uint32_t g = atomicAdd(&ucur[(int64_t)u * kCursorStep], 1u);
-            if (g < n) out[g] = narrow_record(r[k]);
+            const bool on = lo + tid + k * kSplitThreads < hi;
+            uint32_t u = 0, rank;
+            if (on) u = __ldg(cell_unit + cell_of(load_cells(zcells + (zhi + wide_tag(r[k]))), r[k].z));
+            const uint32_t g = claim_places(ucur, kCursorStep, u, on, &rank) + rank;
+            if (on && g < n) out[g] = narrow_record(r[k]);
         }
         return;
     }
@@ -765,6 +811,10 @@ struct PlaceArgs {
     uint32_t* lut;
     ZoneHot* zhot;
     const int32_t* err;
+    // units of one cell of more than giant_rows rows: a list for k_place_giant
+    uint32_t giant_rows;
+    uint32_t* giants;
+    uint32_t* n_giants;
 };
 
 // Buckets of a zone of m rows whose keys span [kmin, kmax] (top 16 bits in
@@ -811,6 +861,7 @@ __device__ __forceinline__ void write_zone(const PlaceArgs& P, uint32_t z, uint3
 }
 
 // Block-wide exclusive prefix of one value per thread.
+template <int THREADS = kPlaceThreads>
 __device__ __forceinline__ uint32_t block_offset(uint32_t sum, uint32_t* warp_tot) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t incl = sum;
@@ -823,21 +874,21 @@ __device__ __forceinline__ uint32_t block_offset(uint32_t sum, uint32_t* warp_to
     __syncthreads();
     uint32_t run = incl - sum;
 #pragma unroll
-    for (int w = 0; w < kPlaceThreads / 32; w++)
+    for (int w = 0; w < THREADS / 32; w++)
         if (w < warp) run += warp_tot[w];
     return run;
 }
 
 // Inclusive prefix, plus `add`, of n 32-bit counters in place. GLOBAL: they
 // lie in global memory, counted by atomics (read past L1).
-template <bool GLOBAL>
+template <bool GLOBAL, int THREADS>
 __device__ __forceinline__ void scan_counters(uint32_t* c, uint32_t n, uint32_t add,
                                               uint32_t* warp_tot) {
-    const uint32_t per = ((n + kPlaceThreads - 1) / kPlaceThreads) | 1u;
+    const uint32_t per = ((n + THREADS - 1) / THREADS) | 1u;
     const uint32_t lo = min(n, threadIdx.x * per), hi = min(n, lo + per);
     uint32_t sum = 0;
     for (uint32_t i = lo; i < hi; i++) sum += GLOBAL ? __ldcg(c + i) : c[i];
-    uint32_t run = add + block_offset(sum, warp_tot);
+    uint32_t run = add + block_offset<THREADS>(sum, warp_tot);
     for (uint32_t i = lo; i < hi; i++) {
         run += GLOBAL ? __ldcg(c + i) : c[i];
         c[i] = run;
@@ -865,10 +916,73 @@ __device__ __forceinline__ void scan_pairs(uint32_t* c, uint32_t n, uint32_t* wa
 
 __device__ __forceinline__ uint32_t clean(uint32_t key) { return key & kRaKeyMask; }
 
-// Rows [s, e) of one cell, too many to stage (or of too many buckets): counted,
-// then moved one by one. B: the zone's buckets, of which the cell holds
-// [b0, b1); `base` is the table place of b0. Buckets past the counters in
-// shared memory are counted in the table itself.
+// Rows [s, e) of one cell counted by bucket into c, and moved to their buckets'
+// places (c then the row after each bucket, at the end its first row), by the
+// threads `tid` of `step` (whole warps). B: the zone's buckets, of which the
+// cell holds those from b0 on. Cells of so many rows are mostly sources on one
+// spot: a warp's sources in one bucket take one atomic; with FEW buckets, each
+// group of them does (which costs more where they lie apart).
+__device__ __forceinline__ uint32_t clean_bucket(uint32_t key, const Buckets& B, uint32_t b0) {
+    return ((clean(key) - B.kmin) >> B.shift) - b0;
+}
+
+// The lanes with the same b, or the lane alone.
+template <bool FEW>
+__device__ __forceinline__ uint32_t bucket_peers(uint32_t b, uint32_t lane) {
+    if (FEW) return __match_any_sync(0xffffffffu, b);
+    return __all_sync(0xffffffffu, b == __shfl_sync(0xffffffffu, b, 0)) ? 0xffffffffu : 1u << lane;
+}
+
+template <bool FEW>
+__device__ __forceinline__ void count_rows(const PlaceArgs& P, uint32_t s, uint32_t e, uint32_t tid,
+                                           uint32_t step, const Buckets& B, uint32_t b0, uint32_t* c) {
+    const uint32_t lane = tid & 31;
+    for (uint32_t i0 = s + (tid - lane); i0 < e; i0 += step * 4) {
+        uint32_t key[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const uint32_t i = i0 + lane + k * step;
+            key[k] = i < e ? __ldg(&P.rec[i].z) : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const bool on = i0 + lane + k * step < e;
+            const uint32_t b = on ? clean_bucket(key[k], B, b0) : 0xFFFFFFFFu;
+            const uint32_t peers = bucket_peers<FEW>(b, lane);
+            if (on && (peers & ((1u << lane) - 1u)) == 0) atomicAdd(&c[b], (uint32_t)__popc(peers));
+        }
+    }
+}
+
+template <bool FEW>
+__device__ __forceinline__ void move_rows(const PlaceArgs& P, uint32_t s, uint32_t e, uint32_t tid,
+                                          uint32_t step, const Buckets& B, uint32_t b0, uint32_t* c) {
+    const uint32_t lane = tid & 31;
+    for (uint32_t i0 = s + (tid - lane); i0 < e; i0 += step * 4) {
+        uint4 r[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const uint32_t i = i0 + lane + k * step;
+            if (i < e) r[k] = __ldg(&P.rec[i]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const bool on = i0 + lane + k * step < e;
+            const uint32_t b = on ? clean_bucket(r[k].z, B, b0) : 0xFFFFFFFFu;
+            const uint32_t peers = bucket_peers<FEW>(b, lane);
+            const uint32_t below = __popc(peers & ((1u << lane) - 1u));
+            uint32_t at = 0;
+            if (on && below == 0) at = atomicSub(&c[b], (uint32_t)__popc(peers));
+            at = __shfl_sync(0xffffffffu, at, __ffs(peers) - 1);
+            r[k].z = clean(r[k].z);
+            if (on) reinterpret_cast<uint4*>(P.out)[at - 1u - below] = r[k];
+        }
+    }
+}
+
+// Rows [s, e) of one cell, too many to stage (or of too many buckets), by a
+// block. The cell holds buckets [b0, b1); `base` is the table place of b0.
+// Buckets past the counters in shared memory are counted in the table itself.
 __device__ __noinline__ void place_large(const PlaceArgs& P, PlaceSmem& S, uint32_t s, uint32_t e,
                             const Buckets& B, uint32_t b0, uint32_t b1, int64_t base) {
     const uint32_t nb = b1 - b0;
@@ -877,36 +991,36 @@ __device__ __noinline__ void place_large(const PlaceArgs& P, PlaceSmem& S, uint3
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < nb; i += kPlaceThreads) c[i] = 0;
     __syncthreads();
-    for (uint32_t i0 = s + threadIdx.x; i0 < e; i0 += kPlaceThreads * 4) {
-        uint32_t key[4];
-#pragma unroll
-        for (int k = 0; k < 4; k++)
-            key[k] = i0 + k * kPlaceThreads < e ? __ldg(&P.rec[i0 + k * kPlaceThreads].z) : 0;
-#pragma unroll
-        for (int k = 0; k < 4; k++)
-            if (i0 + k * kPlaceThreads < e)
-                atomicAdd(&c[((clean(key[k]) - B.kmin) >> B.shift) - b0], 1u);
-    }
+    count_rows<false>(P, s, e, threadIdx.x, kPlaceThreads, B, b0, c);
     __syncthreads();
-    if (c != L) scan_counters<false>(c, nb, s, S.warp_tot);  // c[b]: the row after bucket b
-    else scan_counters<true>(c, nb, s, S.warp_tot);
-    for (uint32_t i0 = s + threadIdx.x; i0 < e; i0 += kPlaceThreads * 4) {
-        uint4 r[4];
-#pragma unroll
-        for (int k = 0; k < 4; k++)
-            if (i0 + k * kPlaceThreads < e) r[k] = __ldg(&P.rec[i0 + k * kPlaceThreads]);
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            if (i0 + k * kPlaceThreads >= e) break;
-            r[k].z = clean(r[k].z);
-            const uint32_t p = atomicSub(&c[((r[k].z - B.kmin) >> B.shift) - b0], 1u) - 1u;
-            reinterpret_cast<uint4*>(P.out)[p] = r[k];
-        }
-    }
+    if (c != L) scan_counters<false, kPlaceThreads>(c, nb, s, S.warp_tot);  // c[b]: the row after bucket b
+    else scan_counters<true, kPlaceThreads>(c, nb, s, S.warp_tot);
+    move_rows<false>(P, s, e, threadIdx.x, kPlaceThreads, B, b0, c);
     __syncthreads();  // (c[b]: the first row of bucket b)
     if (c != L)
         for (uint32_t i = threadIdx.x; i < nb; i += kPlaceThreads) L[i] = c[i];
     __syncthreads();
+}
+
+// The buckets of part cell c0 of zone z0: nb of them from b0 on, their table
+// from `base` on. `write`: the first part's thread writes the zone, the last
+// one's the entry after the table (row e).
+__device__ __forceinline__ void part_buckets(const PlaceArgs& P, const ZoneCells& Z, uint32_t c0,
+                                             uint32_t z0, uint32_t e, uint32_t rel0, bool write,
+                                             Buckets* B, uint32_t* b0, uint32_t* nb, int64_t* base) {
+    const uint32_t zs = P.cell_start[Z.first];
+    const uint32_t mz = P.cell_start[Z.first + Z.parts] - zs;
+    *B = buckets_of(mz, (65535u - P.range->not_min) << 16, P.range->max << 16, true,
+                    Z.shift + kIndexRaShift);
+    const uint32_t p = c0 - Z.first;
+    const uint32_t at = Z.p0 + p, sh = Z.shift + 16;
+    *b0 = p == 0 ? 0 : ((at << sh) - B->kmin) >> B->shift;
+    *nb = (p + 1 == Z.parts ? B->last + 1 : (((at + 1) << sh) - B->kmin) >> B->shift) - *b0;
+    *base = 2 * (int64_t)zs + rel0 + *b0;
+    if (write) {
+        if (p == 0) write_zone(P, z0, zs, rel0, *B);
+        if (p + 1 == Z.parts) P.lut[*base + *nb] = e;
+    }
 }
 
 // Units, a block each: the records of consecutive zones, or of one part of a
@@ -946,6 +1060,10 @@ __global__ void __launch_bounds__(kPlaceThreads, kPlaceBlocks) k_place_b(PlaceAr
         }
         if (c0 == c1) continue;  // an id without cells
         const uint32_t m = e - s, nzones = c1 - c0;
+        if (m > P.giant_rows) {
+            if (tid == 0) P.giants[atomicAdd(P.n_giants, 1u)] = u;
+            continue;
+        }
         bool large = m > kPlaceCap;
         uint4 r[kPlaceItems];
         if (!large) {
@@ -966,19 +1084,9 @@ __global__ void __launch_bounds__(kPlaceThreads, kPlaceBlocks) k_place_b(PlaceAr
         uint32_t b0 = 0;
         __syncthreads();  // (the last unit's stage and tables are out)
         if (part) {
-            const uint32_t zs = P.cell_start[Z.first];
-            const uint32_t mz = P.cell_start[Z.first + Z.parts] - zs;
-            B = buckets_of(mz, (65535u - P.range->not_min) << 16, P.range->max << 16, true,
-                           Z.shift + kIndexRaShift);
-            const uint32_t p = c0 - Z.first;
-            const uint32_t at = Z.p0 + p, sh = Z.shift + 16;
-            b0 = p == 0 ? 0 : ((at << sh) - B.kmin) >> B.shift;
-            nb = (p + 1 == Z.parts ? B.last + 1 : (((at + 1) << sh) - B.kmin) >> B.shift) - b0;
-            base = 2 * (int64_t)zs + rel0 + b0;
+            part_buckets(P, Z, c0, z0, e, rel0, tid == 0, &B, &b0, &nb, &base);
             large |= nb > kPlaceCtr;
             if (tid == 0) {
-                if (p == 0) write_zone(P, z0, zs, rel0, B);
-                if (p + 1 == Z.parts) P.lut[base + nb] = e;
                 S.zkmin[0] = B.kmin;
                 S.zshift[0] = B.shift;
                 S.zlb[0] = 0u - b0;
@@ -1076,6 +1184,91 @@ __global__ void __launch_bounds__(kPlaceThreads, kPlaceBlocks) k_place_b(PlaceAr
         for (uint32_t i = tid; i < m; i += kPlaceThreads)
             reinterpret_cast<uint4*>(P.out)[s + i] = S.stage[i];
     }
+}
+
+// The units of very many rows, which one block of k_place_b would hold up (a
+// unit of 2e6 rows took it 5.8 ms): a cluster of eight blocks each, counting in
+// the bucket table. Listed from kGiantRows rows on, some 50 us of a block's
+// time, and a 2048th of the catalogue's, so that the list stays short; where
+// one split makes the units, whose zones are not cut into parts and have up to
+// 65536 buckets, from kGiantZone on.
+constexpr uint32_t kGiantRows = 16384, kGiantZone = 4096;
+constexpr int kGiantThreads = 1024, kGiantBlocks = 8;
+
+__global__ void __cluster_dims__(kGiantBlocks, 1, 1) __launch_bounds__(kGiantThreads)
+    k_place_giant(PlaceArgs P) {
+    pdl_wait();
+    const uint32_t n = *P.n_giants;
+    if (n == 0 || build_failed(P.err)) return;  // (the whole cluster)
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const uint32_t rank = cluster.block_rank();
+    constexpr uint32_t kStep = kGiantThreads * kGiantBlocks;
+    const uint32_t tid = rank * kGiantThreads + threadIdx.x;
+    __shared__ uint32_t kmin, kmax, total, warp_tot[kGiantThreads / 32];
+    for (uint32_t g = blockIdx.x / kGiantBlocks; g < n; g += gridDim.x / kGiantBlocks) {
+        const uint32_t u = P.giants[g];
+        const uint4 d = __ldg(P.unit + u);
+        const uint32_t c0 = d.x, z0 = d.y, s = d.z, e = __ldg(P.unit + u + 1).z;
+        ZoneCells Z{c0, 1, 0, 16};
+        if (P.zcells) Z = load_cells(P.zcells + z0);
+        const uint32_t rel0 = P.zcells ? 3 * z0 + 2 * Z.first : 5 * z0;
+        uint32_t b0 = 0, nb = 0;
+        int64_t base = 2 * (int64_t)s + rel0;
+        Buckets B{};
+        if (Z.parts > 1) {
+            part_buckets(P, Z, c0, z0, e, rel0, tid == 0, &B, &b0, &nb, &base);
+        } else {  // one zone
+            if (threadIdx.x == 0) {
+                kmin = 0xFFFFu;
+                kmax = 0;
+            }
+            __syncthreads();
+            uint32_t lo = 0xFFFFu, hi = 0;
+            for (uint32_t i = s + tid; i < e; i += kStep) {
+                const uint32_t key = __ldg(&P.rec[i].z) >> 16;
+                lo = min(lo, key);
+                hi = max(hi, key);
+            }
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if ((threadIdx.x & 31) == 0) {
+                atomicMin(&kmin, lo);
+                atomicMax(&kmax, hi);
+            }
+            cluster.sync();
+            for (int k = 0; k < kGiantBlocks; k++) {
+                lo = min(lo, *cluster.map_shared_rank(&kmin, k));
+                hi = max(hi, *cluster.map_shared_rank(&kmax, k));
+            }
+            B = buckets_of(e - s, lo << 16, hi << 16, false, 32);
+            nb = B.last + 1;
+            if (tid == 0) {
+                write_zone(P, z0, s, rel0, B);
+                P.lut[base + nb] = e;
+            }
+        }
+        uint32_t* const L = P.lut + base;
+        for (uint32_t i = tid; i < nb; i += kStep) L[i] = 0;
+        if (threadIdx.x == 0) total = 0;
+        cluster.sync();
+        count_rows<true>(P, s, e, tid, kStep, B, b0, L);
+        cluster.sync();
+        // each block's share of the buckets, after the sums of those before it
+        const uint32_t share = (nb + kGiantBlocks - 1) / kGiantBlocks;
+        const uint32_t l0 = min(nb, rank * share), l1 = min(nb, l0 + share);
+        uint32_t sum = 0;
+        for (uint32_t i = l0 + threadIdx.x; i < l1; i += kGiantThreads) sum += __ldcg(L + i);
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&total, sum);
+        cluster.sync();
+        uint32_t before = s;
+        for (uint32_t k = 0; k < rank; k++) before += *cluster.map_shared_rank(&total, k);
+        scan_counters<true, kGiantThreads>(L + l0, l1 - l0, before, warp_tot);
+        cluster.sync();
+        move_rows<true>(P, s, e, tid, kStep, B, b0, L);
+    }
+    cluster.sync();  // (no block ends while another reads its shared memory)
 }
 
 // Zone geometry depends only on the zone count: it is computed once per
@@ -1214,6 +1407,7 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
     const size_t o_cunit = W.add<uint32_t>(cells_cap);
     const size_t o_unit = W.add<uint4>(units_cap + 1);
     const size_t o_ucur = W.add<uint32_t>(units_cap * kCursorStep);
+    const size_t o_giants = W.add<uint32_t>(n / kGiantZone + 1);
     double *d_lon = nullptr, *d_lat = nullptr;
     unsigned char* work = nullptr;
     uint4* tmp = nullptr;
@@ -1278,7 +1472,7 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
             uint32_t* const zcnt = at32(o_zcnt);
             uint64_t* const status = (uint64_t*)(work + o_status);
             // [0..2] tile counters, [4] cells, [5] units,
-            // [6..7] range of the RA keys
+            // [6..7] range of the RA keys, [8] units listed
             uint32_t* const small = at32(o_small);
             KeyRange* const range = (KeyRange*)(small + 6);
             uint32_t* const cstart = at32(o_cstart);
@@ -1363,10 +1557,17 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
             if (X->p64 && n > 0)
                 XM_LAUNCH("k_unit_b", (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, k_unit_b,
                           X->pos, n, X->p64, err);
+            const uint32_t giant_rows = n <= kGiantRows ? (uint32_t)n  // (a launch saved: no list)
+                                        : !two          ? kGiantZone
+                                        : n >> 11 > kGiantRows ? (uint32_t)(n >> 11)
+                                                               : kGiantRows;
             const PlaceArgs P{tmp, unit, small + 5, cstart, czone, zcells, range, geo, nz, n,
-                              X->rec, X->lut, X->zhot, err};
+                              X->rec, X->lut, X->zhot, err, giant_rows, at32(o_giants), small + 8};
             XM_LAUNCH("k_place_b", (unsigned)(units_cap < kPlaceBlocks * 152 ? units_cap : kPlaceBlocks * 152),
                       kPlaceThreads, sizeof(PlaceSmem), s, k_place_b, P);
+            if (n > giant_rows)
+                XM_LAUNCH("k_place_giant", 152 / kGiantBlocks * kGiantBlocks, kGiantThreads, 0, s,
+                          k_place_giant, P);
             return XM_OK;
         };
         st = body();
