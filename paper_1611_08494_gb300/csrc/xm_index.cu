@@ -118,12 +118,14 @@ __device__ __forceinline__ bool build_failed(const int32_t* err) {
 }
 
 // Sources per zone. WIDE 0: counters in global memory (few sources, or more
-// zones than shared memory holds counters for); 1: a 32-bit counter per zone
-// in shared memory; 2: 16-bit counters, folded into the global ones before
-// they can overflow. On 2e8 sources in 27,000 zones the shared form takes
-// 0.41 ms (the 8 bytes it reads per source), global atomics 2.1 ms.
+// zones than shared memory holds counters for), one atomic for a warp whose
+// sources share a zone; 1: a 32-bit counter per zone in shared memory; 2: 16-bit
+// counters, two a word, folded into the global ones by the thread whose source
+// takes one to 0x8000. A barrier every kFoldLoops loads bounds what is added
+// before that thread's subtraction. On 2e8 sources in 27,000 zones the shared
+// form takes 0.41 ms (the 8 bytes it reads per source), global atomics 2.1 ms.
 template <int WIDE>
-__global__ void __launch_bounds__(1024) k_zone_count(const double* __restrict__ lat, int64_t n,
+__global__ void __launch_bounds__(kCountThreads) k_zone_count(const double* __restrict__ lat, int64_t n,
                                                      int32_t nz, uint32_t* __restrict__ zcnt) {
     pdl_wait();
     extern __shared__ uint32_t h[];
@@ -131,18 +133,27 @@ __global__ void __launch_bounds__(1024) k_zone_count(const double* __restrict__ 
         for (int i = threadIdx.x; i < (WIDE == 1 ? nz : (nz + 1) / 2); i += blockDim.x) h[i] = 0;
         __syncthreads();
     }
-    const int64_t step = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * step) {
-        double la[4];
+    const int64_t step = (int64_t)gridDim.x * kCountThreads;
+    int loads = 0;
+    for (int64_t b0 = (int64_t)blockIdx.x * kCountThreads; b0 < n; b0 += kCountLoads * step) {
+        const int64_t i0 = b0 + threadIdx.x;
+        double la[kCountLoads];
 #pragma unroll
-        for (int k = 0; k < 4; k++) la[k] = i0 + k * step < n ? lat[i0 + k * step] : 0.0;
+        for (int k = 0; k < kCountLoads; k++) la[k] = i0 + k * step < n ? lat[i0 + k * step] : 0.0;
 #pragma unroll
-        for (int k = 0; k < 4; k++) {
-            if (i0 + k * step >= n) break;
+        for (int k = 0; k < kCountLoads; k++) {
             const int32_t z = zone_of_lat(lat_or_zero(la[k]), nz);
             if (WIDE == 0) {
-                atomicAdd(&zcnt[z], 1u);
-            } else if (WIDE == 1) {
+                const bool on = i0 + k * step < n;
+                if (__all_sync(0xffffffffu, on && z == __shfl_sync(0xffffffffu, z, 0))) {
+                    if ((threadIdx.x & 31) == 0) atomicAdd(&zcnt[z], 32u);
+                } else if (on) {
+                    atomicAdd(&zcnt[z], 1u);
+                }
+                continue;
+            }
+            if (i0 + k * step >= n) break;
+            if (WIDE == 1) {
                 atomicAdd(&h[z], 1u);
             } else {
                 const int sh = 16 * (z & 1);
@@ -152,6 +163,7 @@ __global__ void __launch_bounds__(1024) k_zone_count(const double* __restrict__ 
                 }
             }
         }
+        if (WIDE == 2 && ++loads % kFoldLoops == 0) __syncthreads();
     }
     if (!WIDE) return;
     __syncthreads();
@@ -1497,12 +1509,12 @@ extern "C" xm_status xm_build_index(const xm_columns* B, const xm_index_opts* op
             // (counters in shared memory are worth their set-up from about 1e5 sources)
             const size_t wide1 = (size_t)nz * 4, wide2 = ((size_t)nz + 1) / 2 * 4;
             if (n >= (1 << 17) && wide1 <= kCountSmem) {
-                XM_LAUNCH("k_zone_count", 152, 1024, wide1, s, k_zone_count<1>, lat, n, nz, zcnt);
+                XM_LAUNCH("k_zone_count", 152, kCountThreads, wide1, s, k_zone_count<1>, lat, n, nz, zcnt);
             } else if (n >= (1 << 17) && wide2 <= kCountSmem) {
-                XM_LAUNCH("k_zone_count", 152, 1024, wide2, s, k_zone_count<2>, lat, n, nz, zcnt);
+                XM_LAUNCH("k_zone_count", 152, kCountThreads, wide2, s, k_zone_count<2>, lat, n, nz, zcnt);
             } else if (n > 0) {
-                const int64_t g = (n + 1023) / 1024;
-                XM_LAUNCH("k_zone_count", (unsigned)(g < 8 * 152 ? g : 8 * 152), 1024, 0, s,
+                const int64_t g = (n + kCountThreads - 1) / kCountThreads;
+                XM_LAUNCH("k_zone_count", (unsigned)(g < 8 * 152 ? g : 8 * 152), kCountThreads, 0, s,
                           k_zone_count<0>, lat, n, nz, zcnt);
             }
             const int64_t tiles = (n + kTile - 1) / kTile;

@@ -23,6 +23,13 @@ constexpr int kBinZoneBits = 11;
 constexpr int kMaxZones = 648000;  // of at least 1 arcsec
 static_assert((kMaxZones >> kBinZoneBits) + 2 <= kMaxBins, "bins of a few rows fit every zone count");
 
+// The zone count's 16-bit counters: a block adds kCountThreads * kCountLoads
+// sources a loop, a barrier every kFoldLoops loops. A counter is below 0x8000
+// after a barrier; before the next it takes at most all that is added between
+// them, stays below 2^16 (no carry into its neighbour) and reaches 0x8000 once.
+constexpr int kCountThreads = 1024, kCountLoads = 4, kFoldLoops = 7;
+static_assert(kCountThreads * kCountLoads * kFoldLoops < 0x8000, "16-bit counters of zones hold");
+
 struct BuildPlan {
     bool two;            // two splits: into bins, and those into units
     int kb;              // a bin's window holds 2^kb rows

@@ -52,3 +52,27 @@ def test_more_units_in_a_bin_than_a_tile_counts():
     n = 1_400_000  # in one zone, whose parts are 1750 units or more
     lat = (4500.5 * 20.0 + g.uniform(-9.0, 9.0, n)) / 3600.0
     _check(g, g.uniform(0, 360, n), lat, 20.0, dict(shape=0, a=0.8))
+
+
+def test_two_zones_of_one_counter_word():
+    """Millions of sources in two zones whose 16-bit counters share a word:
+    every block folds both counters."""
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1611_08494_gb300 import xm
+
+    g = synth.rng(1460)
+    n = 12_000_000
+    lon = g.uniform(0, 360, n)
+    lat = 16.0 / 3600.0 * g.uniform(2000.02, 2000.98, n)  # zones 2 k and 2 k + 1 of 8 arcsec
+    idx = xm.Index(_cuda(lon), _cuda(lat), zone_height_arcsec=8.0)
+    pick = g.integers(0, n, 40)
+    a_lon, a_lat = lon[pick], lat[pick] + 0.1 / 3600.0
+    res = xm.Result(idx, _cuda(a_lon), _cuda(a_lat), a=1.0)
+    near = np.unique(np.concatenate([np.nonzero(np.abs(lon - x) < 0.001)[0] for x in a_lon]))
+    ref = oracle.match(a_lon, a_lat, lon[near], lat[near], a=1.0)
+    assert ref["border_a"].size == 0 and ref["a_row"].size > 40
+    np.testing.assert_array_equal(res.a_row.cpu().numpy(), ref["a_row"])
+    np.testing.assert_array_equal(res.b_row.cpu().numpy(), near[ref["b_row"]])

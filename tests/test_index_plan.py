@@ -62,3 +62,53 @@ def test_bins_fit_their_arrays(tmp_path):
     subprocess.run([cxx, "-std=c++17", "-O2", "-I" + CSRC, "-o", exe, str(src)], check=True)
     r = subprocess.run([exe], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+FOLD = r"""
+#include <stdio.h>
+#include "xm_plan.cuh"
+using namespace xm;
+// Two 16-bit counters of a word under the order of events that holds a fold back
+// the longest: all that is added between two barriers, then the folds.
+int main() {
+    const uint32_t per = kCountThreads * kCountLoads * kFoldLoops;
+    for (int which = 0; which < 2; which++)
+        for (uint32_t step = 1; step <= per; step = step < 3 ? step + 1 : step * 3) {
+            uint32_t word = 0, other = 0x7FFF;
+            word += other << (16 * !which);  // the neighbour's count, which must not change
+            uint64_t added = 0, folded = 0;
+            const int sh = 16 * which;
+            for (int window = 0; window < 40; window++) {
+                const uint32_t n = per - (window * step) % per;
+                uint32_t folds = 0;
+                for (uint32_t k = 0; k < n; k++) {
+                    folds += ((word >> sh) & 0xFFFFu) == 0x7FFFu;
+                    word += 1u << sh;
+                }
+                added += n;
+                for (uint32_t k = 0; k < folds; k++) {
+                    word -= 0x8000u << sh;
+                    folded += 0x8000;
+                }
+                if (((word >> (16 * !which)) & 0xFFFFu) != other ||
+                    folded + ((word >> sh) & 0xFFFFu) != added) {
+                    printf("window %d of %u sources\n", window, n);
+                    return 1;
+                }
+            }
+        }
+    return 0;
+}
+"""
+
+
+def test_counters_of_zones_hold(tmp_path):
+    cxx = shutil.which("g++")
+    if not cxx:
+        pytest.skip("no C++ compiler")
+    src = tmp_path / "fold.cpp"
+    src.write_text(FOLD)
+    exe = str(tmp_path / "fold")
+    subprocess.run([cxx, "-std=c++17", "-O2", "-I" + CSRC, "-o", exe, str(src)], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
