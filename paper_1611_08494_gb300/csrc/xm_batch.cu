@@ -66,6 +66,7 @@ struct BatchConst {
     int32_t index_frame;
     int32_t nz;
     float h_f;  // zone height of the index (rad)
+    float sparse_r;  // sources of larger regions are not offered to the sparse pass
 };
 
 __device__ __forceinline__ int32_t find_req(const int64_t* __restrict__ off, int32_t n_req,
@@ -112,36 +113,71 @@ __global__ void k_batch_ingest(BatchConst C, uint64_t* __restrict__ keys,
     vals[g] = (uint32_t)g;
 }
 
-// err, bad_req: also validates (input order, which needs no sort keys).
-__global__ void k_batch_prep(BatchConst C, const uint32_t* __restrict__ vals,
-                             APrep* __restrict__ out, ACold* __restrict__ cold,
-                             int32_t* __restrict__ lrow, int32_t* err, int32_t* bad_req) {
+// err, bad_req: also validates (input order, which needs no sort keys). Sources
+// too large for the sparse count pass are listed for the general one (left[0]
+// of them), and the chunks of 32 with another one for the sparse pass (left[1];
+// one atomic a block each: the warps' own would take as long as the rest).
+__global__ void __launch_bounds__(kBlock) k_batch_prep(
+    BatchConst C, const uint32_t* __restrict__ vals, APrep* __restrict__ out,
+    ACold* __restrict__ cold, int32_t* __restrict__ lrow, int32_t* err, int32_t* bad_req,
+    int32_t* __restrict__ large, int32_t* __restrict__ chunks, int32_t* left) {
     pdl_wait();
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= C.total) return;
-    const int64_t g = vals ? (int64_t)vals[s] : s;
-    const int32_t r = find_req(C.off, C.n_req, g);
-    const ReqDev& R = C.req[r];
-    const int64_t i = g - R.off;
-    double lon, lat, gamma;
-    bool ok;
-    batch_position(C, R, i, &lon, &lat, &gamma, &ok);
-    const double a = col_or(R.a_col, i, R.a);
-    const double b = R.shape == XM_CIRCLE ? a : col_or(R.b_col, i, R.b);
-    const double pa = col_or(R.pa_col, i, R.pa);
-    if (err) {
-        if (!ok) atomicOr(err, kErrCoord);
-        if (!size_ok(a, b, pa)) atomicOr(err, kErrSize);
-        if (!ok || !size_ok(a, b, pa)) atomicMin(bad_req, r);
+    const int64_t s = (int64_t)blockIdx.x * kBlock + threadIdx.x;
+    const bool on = s < C.total;
+    bool small = false;
+    if (on) {
+        const int64_t g = vals ? (int64_t)vals[s] : s;
+        const int32_t r = find_req(C.off, C.n_req, g);
+        const ReqDev& R = C.req[r];
+        const int64_t i = g - R.off;
+        double lon, lat, gamma;
+        bool ok;
+        batch_position(C, R, i, &lon, &lat, &gamma, &ok);
+        const double a = col_or(R.a_col, i, R.a);
+        const double b = R.shape == XM_CIRCLE ? a : col_or(R.b_col, i, R.b);
+        const double pa = col_or(R.pa_col, i, R.pa);
+        if (err) {
+            if (!ok) atomicOr(err, kErrCoord);
+            if (!size_ok(a, b, pa)) atomicOr(err, kErrSize);
+            if (!ok || !size_ok(a, b, pa)) atomicMin(bad_req, r);
+        }
+        APrep P;
+        ACold C64;
+        make_aprep(lon, lat, gamma, ok, a, b, pa, R.shape, R.pa_dir, R.size_k, R.pa_zero, C.nz, C.h_f,
+                   (int32_t)g, &P, &C64);
+        if (R.rotate) P.shape |= kRotated;
+        out[s] = P;
+        cold[s] = C64;
+        lrow[g] = (int32_t)i;
+        small = P.R <= C.sparse_r;
     }
-    APrep P;
-    ACold C64;
-    make_aprep(lon, lat, gamma, ok, a, b, pa, R.shape, R.pa_dir, R.size_k, R.pa_zero, C.nz, C.h_f,
-               (int32_t)g, &P, &C64);
-    if (R.rotate) P.shape |= kRotated;
-    out[s] = P;
-    cold[s] = C64;
-    lrow[g] = (int32_t)i;
+    constexpr int kWarps = kBlock / 32;
+    __shared__ int32_t n_large[kWarps], n_chunk[kWarps], first[2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t big = __ballot_sync(0xffffffffu, on && !small);
+    const bool chunk = __any_sync(0xffffffffu, small);
+    if (lane == 0) {
+        n_large[warp] = __popc(big);
+        n_chunk[warp] = chunk;
+    }
+    __syncthreads();
+    int32_t at = 0, at_chunk = 0, sum = 0, sum_chunk = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; w++) {
+        if (w < warp) {
+            at += n_large[w];
+            at_chunk += n_chunk[w];
+        }
+        sum += n_large[w];
+        sum_chunk += n_chunk[w];
+    }
+    if (threadIdx.x == 0) {
+        if (sum) first[0] = atomicAdd(left, sum);
+        if (sum_chunk) first[1] = atomicAdd(left + 1, sum_chunk);
+    }
+    __syncthreads();
+    if (on && !small) large[first[0] + at + __popc(big & ((1u << lane) - 1u))] = (int32_t)s;
+    if (chunk && lane == 0) chunks[first[1] + at_chunk] = (int32_t)(s >> 5);
 }
 
 __device__ __forceinline__ bool jt_pairs(int t) {
@@ -372,9 +408,9 @@ struct BatchBufs {
 };
 
 // small[]: 0 total pairs, 1 total rows, 2 arena records, 3 (int32 x2) error
-// bits and first bad request, 4 (int32 x4) list counts + chunk queue, 6 (int32)
-// largest member count and sources the sparse pass leaves, 7 (int32) the sparse
-// pass's queue, per-request counters follow at small + 8: unmatched A [n], matched B [n]
+// bits and first bad request, 4 (int32 x4) list counts + chunk queue, 6 (int32
+// x2) largest member count and the sparse pass's queue, 7 (int32 x2) sources the
+// sparse pass leaves and chunks it takes, per-request counters follow at small + 8: unmatched A [n], matched B [n]
 constexpr int kSmallWords = 8;
 
 }  // namespace
@@ -498,7 +534,7 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
     B.prep = (APrep*)dev_alloc(nn * sizeof(APrep), s);
     B.cold = (ACold*)dev_alloc(nn * sizeof(ACold), s);
     B.lrow = (int32_t*)dev_alloc(nn * sizeof(int32_t), s);
-    B.lists = (int32_t*)dev_alloc(4 * nn * sizeof(int32_t), s);
+    B.lists = (int32_t*)dev_alloc((4 * nn + (nn + 31) / 32) * sizeof(int32_t), s);
     B.arena = (MemberRec*)dev_alloc(arena_cap * sizeof(MemberRec), s);
     B.rows = (int32_t*)dev_alloc(nn * sizeof(int32_t), s);
     B.row_off = (int64_t*)dev_alloc((nn + sum_words) * sizeof(int64_t), s);
@@ -536,11 +572,13 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
     C.index_frame = X->frame;
     C.nz = X->nz;
     C.h_f = (float)X->h;
+    C.sparse_r = sparse_limit(prec == XM_PREC_FP64 ? kPrecFP64 : kPrecFP32, C.h_f);
     int32_t* err = (int32_t*)(B.small + 3);
     int32_t* bad_req = err + 1;
     int32_t* list_n = (int32_t*)(B.small + 4);
     unsigned long long* arena_n = (unsigned long long*)(B.small + 2);
     unsigned int* queue = (unsigned int*)(list_n + 3);
+    int32_t* const left = (int32_t*)(B.small + 7);
     unsigned long long* req_un_a = (unsigned long long*)(B.small + kSmallWords);
     unsigned long long* req_mb = req_un_a + n;
 
@@ -576,7 +614,8 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
             // (input order: the scan takes the sources request by request)
             XM_LAUNCH("k_batch_prep", grid_for(total), kBlock, 0, s, k_batch_prep, C,
                       sorted_a ? (const uint32_t*)B.vals : (const uint32_t*)nullptr, B.prep, B.cold,
-                      B.lrow, sorted_a ? (int32_t*)nullptr : err, bad_req);
+                      B.lrow, sorted_a ? (int32_t*)nullptr : err, bad_req, B.lists + 3 * nn,
+                      B.lists + 4 * nn, left);
         }
         ScanArgs a{};
         a.G = X->geom();
@@ -603,9 +642,10 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
         if (total > 0) {
             // sources whose regions are small against the zones, then the
             // rest of them, as in a single match
-            int32_t* const left = (int32_t*)(B.small + 6) + 1;
             ScanArgs q = a;
-            q.queue = (unsigned int*)(B.small + 7);
+            q.queue = (unsigned int*)(B.small + 6) + 1;
+            q.list = B.lists + 4 * nn;
+            q.nlist_dev = left + 1;
             const unsigned gs = (unsigned)std::min<int64_t>(8LL * sms, (total + 127) / 128);
             if (prec == XM_PREC_FP32_RECHECK)
                 XM_LAUNCH("k_scan_src", gs, kScanThreads, (kSrcSmem<kPrecFP32, true>), s,

@@ -1010,8 +1010,20 @@ __device__ __noinline__ bool recheck64(double lon, double lat, double theta, dou
     return test64(a64, shape, px, py, pz, &rho);
 }
 
+// The largest radius of a region that a batch offers to the sparse pass: half a
+// zone meets two zones at most; up to a zone some do, and on the float64 path,
+// where the pass gains more, three quarters pay. (64 requests of 2e4 sources,
+// limits of half, three quarters and a whole zone: sizes from 0.5 to 1.5 zones
+// 1.19, 1.21, 1.19 ms in float32, where every source offered took 1.22; from
+// 0.025 to 1.5 zones 1.06, 1.04, 1.02 there and 1.13, 1.10, 1.07 in float64.)
+__host__ __device__ __forceinline__ float sparse_limit(int prec, float h_f) {
+    return (prec == kPrecFP64 ? 0.75f : 0.5f) * h_f;
+}
+
 // PREP: the sources are prepared records (P.A, P.Ac: the requests of a batch,
-// of any shapes and sizes) instead of the caller's columns with one size. The
+// of any shapes and sizes) instead of the caller's columns with one size, in
+// the chunks of P.list that hold one within sparse_limit (those too large are in
+// `defer` already). The
 // 3.1e7 sources of a batch, half of them with sizes of their own, two thirds of
 // the others small enough: 1.9 ms and 1.0 for k_scan over the rest (4.0 with
 // k_scan alone).
@@ -1059,7 +1071,12 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_
     // its positions loaded
     unsigned int next = 0;
     if (lane == 0) next = atomicAdd(P.queue, 1u);
-    int64_t this_first = (int64_t)__shfl_sync(0xffffffffu, next, 0) * 32;
+    const unsigned int n_listed = PREP ? (unsigned int)*P.nlist_dev : 0;
+    auto first_of = [&](unsigned int chunk) {
+        if (!PREP) return (int64_t)chunk * 32;
+        return chunk < n_listed ? (int64_t)__ldg(P.list + chunk) * 32 : P.nA;
+    };
+    int64_t this_first = first_of(__shfl_sync(0xffffffffu, next, 0));
     double lon0 = 0.0, lat0 = 0.0;
     if (!PREP && this_first + lane < P.nA) {
         lon0 = I.lon[this_first + lane];
@@ -1071,6 +1088,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_
 
         // ---- preparation, window and bucket ranges (lane = source)
         bool mine = false;  // this lane's source is counted here
+        bool leave = false;  // it goes to k_scan
         int n0 = 0, nrec = 0;  // records of item 0, of both items
         if (this_first + lane < P.nA) {
             const int64_t s = this_first + lane;
@@ -1121,7 +1139,9 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_
                 W.theta[lane] = C.theta;
             }
             // (float32 separations, on that path)
-            mine = PREC == kPrecFP64 || 16.0f * kEps32 * (A.R + 2.0f * G.h_f) * 206264.8f <= 9e-5f;
+            const bool offered = !PREP || A.R <= sparse_limit(PREC, G.h_f);
+            mine = offered &&
+                   (PREC == kPrecFP64 || 16.0f * kEps32 * (A.R + 2.0f * G.h_f) * 206264.8f <= 9e-5f);
             if (mine && A.R > 0.0f) {
                 const Window w = a_window(A, G);
                 const int items = (w.z1 - w.z0 + 1) * w.nseg;
@@ -1151,9 +1171,16 @@ __global__ void __launch_bounds__(kScanThreads, 6) k_scan_src(ScanArgs P, int32_
                     }
                 }
             }
-            if (!mine) defer[atomicAdd(n_defer, 1)] = (int32_t)s;
+            leave = offered && !mine;
         }
-        const int64_t next_first = (int64_t)__shfl_sync(0xffffffffu, next, 0) * 32;
+        const uint32_t left = __ballot_sync(0xffffffffu, leave);
+        if (left) {
+            int32_t at = 0;
+            if (lane == 0) at = atomicAdd(n_defer, __popc(left));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (leave) defer[at + __popc(left & lt_mask)] = (int32_t)this_first + lane;
+        }
+        const int64_t next_first = first_of(__shfl_sync(0xffffffffu, next, 0));
         if (!PREP && next_first + lane < P.nA) {
             lon0 = I.lon[next_first + lane];
             lat0 = I.lat[next_first + lane];
