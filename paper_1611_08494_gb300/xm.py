@@ -657,22 +657,25 @@ class _BatchMem:
 class Batch:
     """Many requests against one index in one pass. ``xm_match_batch``."""
 
-    # view's tensors: name, pointer and length in the C view, type
-    _FIELDS = (("a_row", "a_row", "n_pairs", "<i8"), ("b_row", "b_row", "n_pairs", "<i8"),
-               ("sep", "sep_arcsec", "n_pairs", "<f8"), ("count", "count", "n_a", "<i4"),
-               ("best_b", "best_b_row", "n_a", "<i8"), ("best_sep", "best_sep_arcsec", "n_a", "<f8"),
-               ("row_a", "row_a", "n_rows", "<i8"), ("row_b", "row_b", "n_rows", "<i8"),
-               ("row_sep", "row_sep", "n_rows", "<f8"))
+    # view's tensors in groups that a request has all or none of (by its
+    # selection and join): length in the C view, then name, pointer there and
+    # type of each
+    _FIELDS = (("n_pairs", (("a_row", "a_row", "<i8"), ("b_row", "b_row", "<i8"), ("sep", "sep_arcsec", "<f8"))),
+               ("n_a", (("count", "count", "<i4"),)),
+               ("n_a", (("best_b", "best_b_row", "<i8"), ("best_sep", "best_sep_arcsec", "<f8"))),
+               ("n_rows", (("row_a", "row_a", "<i8"), ("row_b", "row_b", "<i8"), ("row_sep", "row_sep", "<f8"))))
 
     def __init__(self, index: Index, requests, precision=PREC_FP32, use_graph=False,
                  persistent_blocks=0, pair_capacity=0, row_capacity=0, a_order=A_ORDER_DEFAULT,
                  stream=None):
         keep = []
+        kinds = []
         arr = (Request * max(len(requests), 1))()
         for k, rq in enumerate(requests):
             rq = dict(rq)
             r, keep = request(rq.pop("lon"), rq.pop("lat"), keep=keep, **rq)
             arr[k] = r
+            kinds.append((r.selection, r.join_type))
         opts = BatchOpts(int(precision), int(bool(use_graph)), int(persistent_blocks),
                          int(a_order), int(pair_capacity), int(row_capacity))
         h = _p()
@@ -680,7 +683,12 @@ class Batch:
                              _stream_handle(stream), ctypes.byref(h)), "xm_match_batch")
         self.handle = h.value
         self._mem = _BatchMem(h.value)
-        self._views = None
+        self._base = None
+        # the first and last request that has each group of _FIELDS
+        has = ([k for k, (s, _) in enumerate(kinds) if s & SEL_ALL], range(len(kinds)),
+               [k for k, (s, _) in enumerate(kinds) if s & SEL_BEST],
+               [k for k, (_, j) in enumerate(kinds) if j >= 0])
+        self._ends = [(h[0], h[-1]) if h else None for h in has]
         self.index = index
         self.n = len(requests)
         self._keep = keep
@@ -691,31 +699,31 @@ class Batch:
               "xm_batch_info")
         return {"total_a": a.value, "total_pairs": p.value, "device_ms": ms.value}
 
-    def _all_views(self):
-        """Every request's C view, and per field the tensor over all requests' values (they are
-        consecutive) with its address. A slice of it costs half of a tensor made from an
-        address: 1.2 against 2.6 ms for the views of 64 requests."""
-        views = (BatchView * self.n)()
-        for r in range(self.n):
-            check(xm_batch_get(self.handle, r, ctypes.byref(views[r])), "xm_batch_get")
-        base = {}
-        for name, ptr, num, typestr in self._FIELDS:
-            size = int(typestr[2])
-            ends = [(getattr(v, ptr), getattr(v, num)) for v in views if getattr(v, ptr)]
-            lo = min((p for p, _ in ends), default=0)
-            hi = max((p + size * n for p, n in ends), default=0)
-            base[name] = (_tensor(lo, (hi - lo) // size, typestr, self._mem), lo, ptr, num, size)
-        return views, base
+    def _get(self, r: int) -> BatchView:
+        v = BatchView()
+        check(xm_batch_get(self.handle, r, ctypes.byref(v)), "xm_batch_get")
+        return v
+
+    def _bases(self):
+        """Per field the tensor over all requests' values with its address: they are consecutive,
+        from those of the first request that has them to the last one's. A slice of it costs half
+        of a tensor made from an address: 1.2 against 2.6 ms for the views of 64 requests."""
+        out = []
+        for (num, fields), ends in zip(self._FIELDS, self._ends):
+            v0, v1 = (self._get(ends[0]), self._get(ends[1])) if ends else (None, None)
+            for name, ptr, typestr in fields:
+                size = int(typestr[2])
+                lo = getattr(v0, ptr) if ends else 0
+                hi = getattr(v1, ptr) + size * getattr(v1, num) if ends else 0
+                out.append((name, _tensor(lo, (hi - lo) // size, typestr, self._mem), lo, ptr, num, size))
+        return out
 
     def view(self, r: int) -> dict:
-        if not 0 <= r < self.n:
-            check(xm_batch_get(self.handle, r, ctypes.byref(BatchView())), "xm_batch_get")
-        if self._views is None:
-            self._views = self._all_views()
-        views, base = self._views
-        v = views[r]
+        v = self._get(r)
+        if self._base is None:
+            self._base = self._bases()
         out = {}
-        for name, (t, lo, ptr, num, size) in base.items():
+        for name, t, lo, ptr, num, size in self._base:
             p = getattr(v, ptr)
             first = (p - lo) // size if p else 0
             out[name] = t[first:first + (getattr(v, num) if p else 0)]
