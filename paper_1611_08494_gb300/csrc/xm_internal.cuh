@@ -790,6 +790,7 @@ struct xm_result {
     int device;
     int32_t selection, precision, shape;
     int32_t max_count;    // largest member count of any source (0: not known)
+    int32_t rotated;      // the A sources came in another frame than the index
     int64_t n_a, n_b, n_pairs;
     int32_t* count;       // [n_a]
     int64_t* pair_off;    // [n_a] exclusive scan of count

@@ -329,6 +329,7 @@ xm_status xm_pending::begin() {
     I.lat = lat;
     I.n = nA;
     I.rotate = A.frame != X->frame;
+    R->rotated = I.rotate;
     double m[9];
     gal_to_eq(m);
     for (int r = 0; r < 3; r++)

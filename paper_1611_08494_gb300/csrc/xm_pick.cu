@@ -50,13 +50,14 @@ __global__ void k_pick_cont(const int64_t* __restrict__ pb, const double* __rest
     }
 }
 
-// Float64 separation (arcsec) of pair p from the exact positions.
+// Float64 separation (arcsec) of pair p from the exact positions, the one that
+// the match computes (rotated: its A sources came in another frame).
 __device__ __forceinline__ double sep64_of(const IndexGeom& G, const ACold* __restrict__ acold,
-                                           const int32_t* __restrict__ a_slot, int64_t a,
-                                           int64_t b) {
+                                           const int32_t* __restrict__ a_slot, bool rotated,
+                                           int64_t a, int64_t b) {
     ACold C = acold[a_slot ? a_slot[a] : a];
     C.theta = 0.0;  // (the separation does not depend on the orientation)
-    const A64 A = make_a64(C, false);
+    const A64 A = make_a64(C, rotated);
     double px, py, pz, rho;
     load_p64(G, (int32_t)b, &px, &py, &pz);
     test64(A, XM_CIRCLE, px, py, pz, &rho);
@@ -64,7 +65,7 @@ __device__ __forceinline__ double sep64_of(const IndexGeom& G, const ACold* __re
 }
 
 __global__ void k_pick_exact(IndexGeom G, const ACold* __restrict__ acold,
-                             const int32_t* __restrict__ a_slot, const int64_t* __restrict__ pa,
+                             const int32_t* __restrict__ a_slot, bool rotated, const int64_t* __restrict__ pa,
                              const int64_t* __restrict__ pb, const double* __restrict__ ps, int64_t n,
                              const unsigned long long* __restrict__ minbits,
                              const int32_t* __restrict__ ncont,
@@ -76,11 +77,11 @@ __global__ void k_pick_exact(IndexGeom G, const ACold* __restrict__ acold,
     if (ncont[b] < 2) return;
     const double m = __longlong_as_double((long long)minbits[b]);
     if (!(ps[p] <= m + kBandArcsec + 1e-9 * m)) return;
-    atomicMin(&min64[b], (unsigned long long)dbits(sep64_of(G, acold, a_slot, pa[p], b)));
+    atomicMin(&min64[b], (unsigned long long)dbits(sep64_of(G, acold, a_slot, rotated, pa[p], b)));
 }
 
 __global__ void k_pick_first(IndexGeom G, const ACold* __restrict__ acold,
-                             const int32_t* __restrict__ a_slot, const int64_t* __restrict__ pa,
+                             const int32_t* __restrict__ a_slot, bool rotated, const int64_t* __restrict__ pa,
                              const int64_t* __restrict__ pb, const double* __restrict__ ps, int64_t n,
                              const unsigned long long* __restrict__ minbits,
                              const int32_t* __restrict__ ncont,
@@ -94,7 +95,7 @@ __global__ void k_pick_first(IndexGeom G, const ACold* __restrict__ acold,
     const double m = __longlong_as_double((long long)minbits[b]);
     if (!(ps[p] <= m + kBandArcsec + 1e-9 * m)) return;
     // the same computation as k_pick_exact, so equal values compare equal
-    if (dbits(sep64_of(G, acold, a_slot, pa[p], b)) == (uint64_t)min64[b])
+    if (dbits(sep64_of(G, acold, a_slot, rotated, pa[p], b)) == (uint64_t)min64[b])
         atomicMin(&first_exact[b], (unsigned long long)p);
 }
 
@@ -176,9 +177,10 @@ extern "C" xm_status xm_pick_pairs(const xm_index* X, const xm_result* R, int32_
             XM_LAUNCH("k_pick_cont", grid_of(n), kBlock, 0, s, k_pick_cont, R->b_row, R->sep, n,
                       minbits, ncont, first);
             XM_LAUNCH("k_pick_exact", grid_of(n), kBlock, 0, s, k_pick_exact, G, R->acold, R->a_slot,
-                      R->a_row, R->b_row, R->sep, n, minbits, ncont, min64);
+                      R->rotated != 0, R->a_row, R->b_row, R->sep, n, minbits, ncont, min64);
             XM_LAUNCH("k_pick_first", grid_of(n), kBlock, 0, s, k_pick_first, G, R->acold,
-                      R->a_slot, R->a_row, R->b_row, R->sep, n, minbits, ncont, min64, first_exact);
+                      R->a_slot, R->rotated != 0, R->a_row, R->b_row, R->sep, n, minbits, ncont, min64,
+                      first_exact);
             XM_LAUNCH("k_pick_flag", grid_of(n), kBlock, 0, s, k_pick_flag, R->a_row, R->b_row, n,
                       ncont, first, first_exact, R->best_b, pick == XM_PICK_MUTUAL ? 1 : 0, flag);
         }
