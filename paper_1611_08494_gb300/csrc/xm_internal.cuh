@@ -741,6 +741,7 @@ xm_status exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t
 // zeros[t]: the counts of zero before element kCountTile * t (a join's
 // unmatched sources), count_scan_words(n) words (0 below kCountScanMin).
 constexpr int kCountTile = 1024;
+constexpr int kRowsThread = 16;  // pairs of a source that a thread of the join writes by itself
 constexpr int64_t kCountScanMin = 1 << 18;
 int64_t count_scan_words(int64_t n);
 xm_status count_scan(const int32_t* count, int64_t* out, int64_t n, int64_t* total, int64_t* zeros,
@@ -789,7 +790,7 @@ struct xm_index {
 struct xm_result {
     int device;
     int32_t selection, precision, shape;
-    int32_t max_count;    // largest member count of any source (0: not known)
+    int32_t max_count;    // no source has more members than this (0: not known)
     int32_t rotated;      // the A sources came in another frame than the index
     int64_t n_a, n_b, n_pairs;
     int32_t* count;       // [n_a]

@@ -139,7 +139,6 @@ __global__ void k_write_b(const uint32_t* __restrict__ bits, const int64_t* __re
 constexpr int kRowsA = 4;  // A sources per thread: 128 in a row per warp
 constexpr int kTileA = kRowsA * kBlock;
 static_assert(kTileA == kCountTile, "the match counts unmatched sources per tile");
-constexpr int kRowsThread = 16;  // pairs that a thread writes for its source
 constexpr int kRowsWarp = 512;   // pairs that a warp writes for its 32 sources
 constexpr int kRowsChunk = 4 * kBlock;  // pairs of a listed chunk
 

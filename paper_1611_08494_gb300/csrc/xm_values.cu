@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kBlock) k_val_probe(
         }
         const int32_t c32 = (int32_t)(m < 2147483647 ? m : 2147483647);
         count[i] = c32;
-        if (c32 > 1 && c32 > *(volatile const int32_t*)max_count) atomicMax(max_count, c32);
+        if (c32 > kRowsThread && c32 > *(volatile const int32_t*)max_count) atomicMax(max_count, c32);
         first[i] = m == 1 ? best : f;
         if (best_b) {
             best_b[i] = best;
@@ -366,7 +366,7 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
             bk = d_b;
         }
         // small: [0] AND of codes, [1] OR, [2] pair total, [3] error bits, [4]
-        // largest count above 1
+        // largest count above kRowsThread
         const unsigned long long init[5] = {~0ull, 0ull, 0ull, 0ull, 0ull};
         e = cudaMemcpyAsync(small, init, sizeof(init), cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return cuda_fail(e, "xm_match_values: init");
@@ -431,7 +431,7 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
         if (e != cudaSuccess) return cuda_fail(e, "xm_match_values sync");
         if ((int32_t)h[1] & kErrTimeout) return set_error(XM_ETIMEOUT, "xm_match_values: look-back timed out");
         if ((int32_t)h[1] & kErrOverflow) return set_error(XM_ECUDA, "xm_match_values: run list overflow");
-        R->max_count = h[2] ? (int32_t)h[2] : 1;
+        R->max_count = h[2] ? (int32_t)h[2] : kRowsThread;
         R->n_pairs = (selection & XM_SEL_ALL) ? (int64_t)h[0] : 0;
         if (selection & XM_SEL_ALL) {
             const int64_t np = R->n_pairs > 0 ? R->n_pairs : 1;
