@@ -129,8 +129,10 @@ typedef struct {
 /* Options of the B index (the sky partition of paper §2.3). The index cuts
  * the sphere into declination zones of height zone_height_arcsec, each zone
  * into RA cells about as wide as they are high; B sources are filed by zone
- * and RA. 0 selects 20 arcsec. build_fp64 also stores float64 unit
- * vectors, which the FP64 path reads (it falls back to computing them). */
+ * and RA. 0 selects 20 arcsec. An index holds 32 bytes a source, 8 to 12 of
+ * bucket tables (xm_index_info has the sum), and 8 with ids. build_fp64 adds
+ * 32: it also stores float64 unit vectors, which the FP64 path reads (it falls
+ * back to computing them). */
 typedef struct {
     double zone_height_arcsec;
     int32_t build_fp64;
@@ -646,9 +648,10 @@ XM_API xm_status xm_measure_peak(int32_t what, double* value, void* stream);
 
 /* ---- test hook (no counterpart in the paper) ----------------------------- */
 
-/* Sets the look-backs of the radix sort's counting passes and of the index
- * build's prefix sums for tests of their bounded waits: spin_limit is the number of polls after which a look-back
- * gives up (0 restores the default, one to two seconds of polling), and
+/* Sets the look-backs of the radix sort's counting passes and of the prefix
+ * sums of the index build and of xm_join (whose xm_rows_get returns the error)
+ * for tests of their bounded waits: spin_limit is the number of polls after
+ * which a look-back gives up (0 restores the default, one to two seconds of polling), and
  * silent_tile (-1 = none) is a tile that publishes none of its status words,
  * so the look-backs after it wait on words nobody writes. A look-back that
  * gives up lets its kernel finish (what it computes is then not used) and

@@ -66,10 +66,10 @@ xm_status launch_scan_fused(int prec, const ScanArgs& a, int mode, int64_t n_uni
 
 // The sparse count pass (k_scan_src): persistent warps, at most the blocks
 // resident at once.
-// Whether the count pass takes the sparse form: float32 tests in input order,
-// and a region of fixed size whose bounding radius is under 0.4 zone heights,
-// so a source meets at most two zones (sources with more items are left to
-// k_scan by the pass itself).
+// Whether the count pass takes the sparse form: input order, either precision,
+// and a region of fixed size (with one angle or an angle by source) whose
+// bounding radius is under 0.4 zone heights, so a source meets at most two
+// zones (sources with more items are left to k_scan by the pass itself).
 bool sparse_scan(bool sorted_a, const xm_region* region, const xm_index* X) {
     if (sorted_a || region->a_col || region->b_col) return false;
     const double k = region->size_scale * region->size_unit_arcsec * kArcsec;
