@@ -58,6 +58,8 @@ void drain_locked() {
             auto& t = g_prof_tot[p.name];
             t.first += ms;
             t.second += 1;
+        } else {  // (events recorded into a graph have no time; the next launch must not see it)
+            cudaGetLastError();
         }
         g_event_pool.push_back(p.a);
         g_event_pool.push_back(p.b);

@@ -62,3 +62,25 @@ def test_one_view_of_many(monkeypatch, first):
     for bad in (-1, 300):
         with pytest.raises(xm.XMError):
             batch.view(bad)
+
+
+def test_profiling_a_graph_batch_fails_no_later_call():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1611_08494_gb300 import xm
+
+    g = synth.rng(1910)
+    lon, lat = _cuda(g.uniform(20.0, 21.0, 5_000)), _cuda(g.uniform(-0.5, 0.5, 5_000))
+    idx = xm.Index(lon, lat)
+    xm.prof_enable(True)
+    try:
+        batch = xm.Batch(idx, [dict(lon=lon[:500], lat=lat[:500], a=5.0)], use_graph=True)
+        prof = xm.prof_all()
+    finally:
+        xm.prof_enable(False)
+    assert "batch_graph" in prof
+    res = xm.Result(xm.Index(lon, lat), lon[:500], lat[:500], a=5.0)  # (the build's first launch failed)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(batch.view(0)["b_row"].cpu().numpy(), res.b_row.cpu().numpy())
