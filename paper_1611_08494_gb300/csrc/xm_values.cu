@@ -163,15 +163,17 @@ __device__ __forceinline__ int64_t bound(const uint64_t* __restrict__ sorted, in
     return lo;
 }
 
-constexpr int kProbeKeys = 4;  // A keys per thread
-constexpr int kProbeRun = 4;   // words of a bucket read at once
+constexpr int kProbeRun = 4;  // words of a bucket read at once
 
 // Per A key the B rows of equal keys. Bound by the latency of dependent loads
-// (bucket table, bucket, B's key under the hash), kept in flight for four keys
-// at a time. first: the only match's row, or the place of the first of several
-// (k_val_emit then reads no list for most keys: 0.45 ms for 2.5e7 against 0.81
-// when each went through its place to a row). 1.8 ms for 2.5e7 keys among 1e8;
-// 2.0 a key per thread with codes and rows apart from the sorted hashes.
+// (bucket table, bucket, B's key under the hash), which many threads of few
+// registers overlap. first: the only match's row, or the place of the first of
+// several (k_val_emit then reads no list for most keys: 0.45 ms for 2.5e7
+// against 0.81 when each went through its place to a row). 1.46 ms for 2.5e7
+// keys among 1e8, and 0.55 for 3e6 keys with 20 matches each among 1e7; with four
+// keys per thread 1.73 and 0.94, since a thread then walks four runs one after
+// the other, and 1.93 and 1.22 with their walks side by side, whose registers
+// halve the threads.
 template <bool HASHED>
 __global__ void __launch_bounds__(kBlock) k_val_probe(
     const void* __restrict__ a_keys, int64_t n_a, int32_t type, const uint64_t* __restrict__ sorted,
@@ -179,88 +181,65 @@ __global__ void __launch_bounds__(kBlock) k_val_probe(
     int64_t* __restrict__ first, int64_t* __restrict__ best_b, double* __restrict__ best_sep,
     int32_t* max_count) {
     pdl_wait();
-    const int64_t i0 = (int64_t)blockIdx.x * (kProbeKeys * kBlock) + threadIdx.x;
-    uint64_t c[kProbeKeys];
-    uint32_t w[kProbeKeys], lo[kProbeKeys], hi[kProbeKeys];
-    uint64_t e[kProbeKeys][kProbeRun];
+    const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
+    if (i >= n_a) return;
+    const uint64_t c = key_code(a_keys, i, type);
+    // (NaN never matches; the int64 maximum has the same code and does)
+    const bool any = n_b > 0 && !(type == XM_KEY_FLOAT64 && c == kNaNCode) &&
+                     (HASHED || (c & ~V.mask) == V.prefix);
+    const uint32_t w = (uint32_t)(HASHED ? code_hash(c) : c & V.mask);
+    uint32_t lo = any ? __ldg(&V.lut[w >> V.shift]) : 0;
+    const uint32_t hi = any ? __ldg(&V.lut[(w >> V.shift) + 1]) : 0;
+    if (hi - lo > 2 * kProbeRun) lo = (uint32_t)bound(sorted, lo, hi, w, false);
+    uint64_t e[kProbeRun];
 #pragma unroll
-    for (int k = 0; k < kProbeKeys; k++) {
-        const int64_t i = i0 + k * kBlock;
-        c[k] = i < n_a ? key_code(a_keys, i, type) : 0;
-        // (NaN never matches; the int64 maximum has the same code and does)
-        const bool any = i < n_a && n_b > 0 && !(type == XM_KEY_FLOAT64 && c[k] == kNaNCode) &&
-                         (HASHED || (c[k] & ~V.mask) == V.prefix);
-        w[k] = (uint32_t)(HASHED ? code_hash(c[k]) : c[k] & V.mask);
-        const uint32_t b = w[k] >> V.shift;
-        lo[k] = any ? __ldg(&V.lut[b]) : 0;
-        hi[k] = any ? __ldg(&V.lut[b + 1]) : 0;
-    }
+    for (int j = 0; j < kProbeRun; j++) e[j] = lo + j < hi ? __ldg(&sorted[lo + j]) : 0;
+    int at = -1;  // the first word equal to w among those read, or -1
+    uint32_t row = 0;
 #pragma unroll
-    for (int k = 0; k < kProbeKeys; k++) {
-        if (hi[k] - lo[k] > 2 * kProbeRun) lo[k] = (uint32_t)bound(sorted, lo[k], hi[k], w[k], false);
-#pragma unroll
-        for (int j = 0; j < kProbeRun; j++)
-            e[k][j] = lo[k] + j < hi[k] ? __ldg(&sorted[lo[k] + j]) : 0;
-    }
-    int32_t at[kProbeKeys];  // the first word equal to w among those read, or -1
-    bool eq[kProbeKeys];
-#pragma unroll
-    for (int k = 0; k < kProbeKeys; k++) {
-        at[k] = -1;
-        uint32_t row = 0;
-#pragma unroll
-        for (int j = kProbeRun - 1; j >= 0; j--)
-            if (lo[k] + j < hi[k] && (uint32_t)(e[k][j] >> 32) == w[k]) {
-                at[k] = j;
-                row = (uint32_t)e[k][j];
-            }
-        eq[k] = at[k] >= 0 && (!HASHED || key_code(b_keys, row, type) == c[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < kProbeKeys; k++) {
-        const int64_t i = i0 + k * kBlock;
-        if (i >= n_a) break;
-        int64_t m = 0, f = 0, best = -1, p = lo[k];
-        if (at[k] < 0 && hi[k] - lo[k] > kProbeRun && (uint32_t)(e[k][kProbeRun - 1] >> 32) < w[k])
-            p = bound(sorted, lo[k] + kProbeRun, hi[k], w[k], false);
-        else if (at[k] < 0)
-            p = hi[k];
-        else
-            p += at[k];
-        // (p: the first word equal to w, or one past those below it)
-        bool known = at[k] >= 0;
-        for (; p < hi[k]; p++) {
-            const int64_t j = p - lo[k];
-            uint64_t v = 0;
-            if (j < kProbeRun) {
-#pragma unroll
-                for (int q = 0; q < kProbeRun; q++) v = q == j ? e[k][q] : v;
-            } else {
-                v = __ldg(&sorted[p]);
-            }
-            if ((uint32_t)(v >> 32) != w[k]) break;
-            const uint32_t r = (uint32_t)v;
-            const bool match = known ? eq[k] : !HASHED || key_code(b_keys, r, type) == c[k];
-            known = false;
-            if (!match) continue;
-            if (m == 0) {
-                best = r;
-                f = p;
-            }
-            m++;
-            if (!HASHED && p - f >= 2 * kProbeRun) {  // a long run of equal keys
-                m = bound(sorted, p, hi[k], w[k], true) - f;
-                break;
-            }
+    for (int j = kProbeRun - 1; j >= 0; j--)
+        if (lo + j < hi && (uint32_t)(e[j] >> 32) == w) {
+            at = j;
+            row = (uint32_t)e[j];
         }
-        const int32_t c32 = (int32_t)(m < 2147483647 ? m : 2147483647);
-        count[i] = c32;
-        if (c32 > kRowsThread && c32 > *(volatile const int32_t*)max_count) atomicMax(max_count, c32);
-        first[i] = m == 1 ? best : f;
-        if (best_b) {
-            best_b[i] = best;
-            best_sep[i] = m > 0 ? 0.0 : NAN;
+    bool known = at >= 0;  // (the first word's key is compared before the walk)
+    const bool eq = known && (!HASHED || key_code(b_keys, row, type) == c);
+    uint32_t p = known ? lo + at : hi;  // the first word equal to w, or one past those below it
+    if (!known && hi - lo > kProbeRun && (uint32_t)(e[kProbeRun - 1] >> 32) < w)
+        p = (uint32_t)bound(sorted, lo + kProbeRun, hi, w, false);
+    uint32_t m = 0, f = 0;
+    int64_t best = -1;
+    for (; p < hi; p++) {
+        const uint32_t j = p - lo;
+        uint64_t v = 0;
+        if (j < kProbeRun) {
+#pragma unroll
+            for (int q = 0; q < kProbeRun; q++) v = q == j ? e[q] : v;
+        } else {
+            v = __ldg(&sorted[p]);
         }
+        if ((uint32_t)(v >> 32) != w) break;
+        const uint32_t r = (uint32_t)v;
+        const bool match = known ? eq : !HASHED || key_code(b_keys, r, type) == c;
+        known = false;
+        if (!match) continue;
+        if (m == 0) {
+            best = r;
+            f = p;
+        }
+        m++;
+        if (!HASHED && p - f >= 2 * kProbeRun) {  // a long run of equal keys
+            m = (uint32_t)bound(sorted, p, hi, w, true) - f;
+            break;
+        }
+    }
+    const int32_t c32 = (int32_t)m;  // (there are at most 2^31 - 1 rows)
+    count[i] = c32;
+    if (c32 > kRowsThread && c32 > *(volatile const int32_t*)max_count) atomicMax(max_count, c32);
+    first[i] = m == 1 ? best : (int64_t)f;
+    if (best_b) {
+        best_b[i] = best;
+        best_sep[i] = m > 0 ? 0.0 : NAN;
     }
 }
 
@@ -414,7 +393,7 @@ extern "C" xm_status xm_match_values(const void* a_keys, int64_t n_a, const void
                       n_runs, run_cap, err);
             XM_LAUNCH("k_val_runs", 4 * 152, kBlock, 0, s, k_val_runs, runs, n_runs, run_cap, lut);
         }
-        const unsigned gp = grid_of((n_a + kProbeKeys - 1) / kProbeKeys);
+        const unsigned gp = grid_of(n_a);
         if (n_a > 0 && hashed)
             XM_LAUNCH("k_val_probe", gp, kBlock, 0, s, k_val_probe<true>, ak, n_a, key_type, packed, bk,
                       n_b, V, R->count, first, R->best_b, R->best_sep, (int32_t*)(small + 4));
