@@ -669,13 +669,11 @@ class Batch:
                  persistent_blocks=0, pair_capacity=0, row_capacity=0, a_order=A_ORDER_DEFAULT,
                  stream=None):
         keep = []
-        kinds = []
         arr = (Request * max(len(requests), 1))()
         for k, rq in enumerate(requests):
             rq = dict(rq)
             r, keep = request(rq.pop("lon"), rq.pop("lat"), keep=keep, **rq)
             arr[k] = r
-            kinds.append((r.selection, r.join_type))
         opts = BatchOpts(int(precision), int(bool(use_graph)), int(persistent_blocks),
                          int(a_order), int(pair_capacity), int(row_capacity))
         h = _p()
@@ -684,11 +682,7 @@ class Batch:
         self.handle = h.value
         self._mem = _BatchMem(h.value)
         self._base = None
-        # the first and last request that has each group of _FIELDS
-        has = ([k for k, (s, _) in enumerate(kinds) if s & SEL_ALL], range(len(kinds)),
-               [k for k, (s, _) in enumerate(kinds) if s & SEL_BEST],
-               [k for k, (_, j) in enumerate(kinds) if j >= 0])
-        self._ends = [(h[0], h[-1]) if h else None for h in has]
+        self._requests = arr
         self.index = index
         self.n = len(requests)
         self._keep = keep
@@ -708,13 +702,20 @@ class Batch:
         """Per field the tensor over all requests' values with its address: they are consecutive,
         from those of the first request that has them to the last one's. A slice of it costs half
         of a tensor made from an address: 1.2 against 2.6 ms for the views of 64 requests."""
+        rq = np.frombuffer(self._requests, np.uint8).reshape(-1, ctypes.sizeof(Request))[:self.n]
+
+        def column(field):
+            return rq[:, field.offset:field.offset + 4].copy().view(np.int32)[:, 0]
+
+        sel, join = column(Request.selection), column(Request.join_type)
         out = []
-        for (num, fields), ends in zip(self._FIELDS, self._ends):
-            v0, v1 = (self._get(ends[0]), self._get(ends[1])) if ends else (None, None)
+        for (num, fields), has in zip(self._FIELDS, (sel & SEL_ALL, sel >= 0, sel & SEL_BEST, join >= 0)):
+            ends = np.flatnonzero(has)
+            v0, v1 = (self._get(int(ends[0])), self._get(int(ends[-1]))) if ends.size else (None, None)
             for name, ptr, typestr in fields:
                 size = int(typestr[2])
-                lo = getattr(v0, ptr) if ends else 0
-                hi = getattr(v1, ptr) + size * getattr(v1, num) if ends else 0
+                lo = getattr(v0, ptr) if v0 else 0
+                hi = getattr(v1, ptr) + size * getattr(v1, num) if v1 else 0
                 out.append((name, _tensor(lo, (hi - lo) // size, typestr, self._mem), lo, ptr, num, size))
         return out
 
