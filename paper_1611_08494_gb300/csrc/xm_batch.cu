@@ -115,69 +115,94 @@ __global__ void k_batch_ingest(BatchConst C, uint64_t* __restrict__ keys,
 
 // err, bad_req: also validates (input order, which needs no sort keys). Sources
 // too large for the sparse count pass are listed for the general one (left[0]
-// of them), and the chunks of 32 with another one for the sparse pass (left[1];
-// one atomic a block each: the warps' own would take as long as the rest).
+// of them), and the chunks of 32 with another one for the sparse pass (left[1]).
+// A block takes its places in the lists with one atomic each after ROUNDS
+// sources a thread and waits for them, so batches of 2^19 sources and more take
+// four rounds: 0.16 ms for 3.8e6 sources, 0.205 with one (0.183 without the
+// lists), 1.10 for 3.2e7.
+template <int ROUNDS>
 __global__ void __launch_bounds__(kBlock) k_batch_prep(
     BatchConst C, const uint32_t* __restrict__ vals, APrep* __restrict__ out,
     ACold* __restrict__ cold, int32_t* __restrict__ lrow, int32_t* err, int32_t* bad_req,
     int32_t* __restrict__ large, int32_t* __restrict__ chunks, int32_t* left) {
     pdl_wait();
-    const int64_t s = (int64_t)blockIdx.x * kBlock + threadIdx.x;
-    const bool on = s < C.total;
-    bool small = false;
-    if (on) {
-        const int64_t g = vals ? (int64_t)vals[s] : s;
-        const int32_t r = find_req(C.off, C.n_req, g);
-        const ReqDev& R = C.req[r];
-        const int64_t i = g - R.off;
-        double lon, lat, gamma;
-        bool ok;
-        batch_position(C, R, i, &lon, &lat, &gamma, &ok);
-        const double a = col_or(R.a_col, i, R.a);
-        const double b = R.shape == XM_CIRCLE ? a : col_or(R.b_col, i, R.b);
-        const double pa = col_or(R.pa_col, i, R.pa);
-        if (err) {
-            if (!ok) atomicOr(err, kErrCoord);
-            if (!size_ok(a, b, pa)) atomicOr(err, kErrSize);
-            if (!ok || !size_ok(a, b, pa)) atomicMin(bad_req, r);
-        }
-        APrep P;
-        ACold C64;
-        make_aprep(lon, lat, gamma, ok, a, b, pa, R.shape, R.pa_dir, R.size_k, R.pa_zero, C.nz, C.h_f,
-                   (int32_t)g, &P, &C64);
-        if (R.rotate) P.shape |= kRotated;
-        out[s] = P;
-        cold[s] = C64;
-        lrow[g] = (int32_t)i;
-        small = P.R <= C.sparse_r;
-    }
-    constexpr int kWarps = kBlock / 32;
-    __shared__ int32_t n_large[kWarps], n_chunk[kWarps], first[2];
+    constexpr int kGroups = ROUNDS * kBlock / 32;  // of 32 sources
+    static_assert(kGroups <= 32, "a lane per group");
+    __shared__ uint32_t s_big[kGroups], s_small[kGroups];  // masks
+    __shared__ int32_t at_large[kGroups], at_chunk[kGroups];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t big = __ballot_sync(0xffffffffu, on && !small);
-    const bool chunk = __any_sync(0xffffffffu, small);
-    if (lane == 0) {
-        n_large[warp] = __popc(big);
-        n_chunk[warp] = chunk;
-    }
-    __syncthreads();
-    int32_t at = 0, at_chunk = 0, sum = 0, sum_chunk = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; w++) {
-        if (w < warp) {
-            at += n_large[w];
-            at_chunk += n_chunk[w];
+    const int64_t base = (int64_t)blockIdx.x * (ROUNDS * kBlock);
+#pragma unroll 1
+    for (int round = 0; round < ROUNDS; round++) {
+        const int64_t s = base + round * kBlock + threadIdx.x;
+        const bool on = s < C.total;
+        bool small = false;
+        if (on) {
+            const int64_t g = vals ? (int64_t)vals[s] : s;
+            const int32_t r = find_req(C.off, C.n_req, g);
+            const ReqDev& R = C.req[r];
+            const int64_t i = g - R.off;
+            double lon, lat, gamma;
+            bool ok;
+            batch_position(C, R, i, &lon, &lat, &gamma, &ok);
+            const double a = col_or(R.a_col, i, R.a);
+            const double b = R.shape == XM_CIRCLE ? a : col_or(R.b_col, i, R.b);
+            const double pa = col_or(R.pa_col, i, R.pa);
+            if (err) {
+                if (!ok) atomicOr(err, kErrCoord);
+                if (!size_ok(a, b, pa)) atomicOr(err, kErrSize);
+                if (!ok || !size_ok(a, b, pa)) atomicMin(bad_req, r);
+            }
+            APrep P;
+            ACold C64;
+            make_aprep(lon, lat, gamma, ok, a, b, pa, R.shape, R.pa_dir, R.size_k, R.pa_zero, C.nz,
+                       C.h_f, (int32_t)g, &P, &C64);
+            if (R.rotate) P.shape |= kRotated;
+            out[s] = P;
+            cold[s] = C64;
+            lrow[g] = (int32_t)i;
+            small = P.R <= C.sparse_r;
         }
-        sum += n_large[w];
-        sum_chunk += n_chunk[w];
-    }
-    if (threadIdx.x == 0) {
-        if (sum) first[0] = atomicAdd(left, sum);
-        if (sum_chunk) first[1] = atomicAdd(left + 1, sum_chunk);
+        const uint32_t big = __ballot_sync(0xffffffffu, on && !small);
+        const uint32_t fit = __ballot_sync(0xffffffffu, small);
+        if (lane == 0) {
+            s_big[round * (kBlock / 32) + warp] = big;
+            s_small[round * (kBlock / 32) + warp] = fit;
+        }
     }
     __syncthreads();
-    if (on && !small) large[first[0] + at + __popc(big & ((1u << lane) - 1u))] = (int32_t)s;
-    if (chunk && lane == 0) chunks[first[1] + at_chunk] = (int32_t)(s >> 5);
+    if (warp == 0) {
+        const int32_t n = lane < kGroups ? __popc(s_big[lane]) : 0;
+        const int32_t c = lane < kGroups ? s_small[lane] != 0 : 0;
+        int32_t sn = n, sc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t t = __shfl_up_sync(0xffffffffu, sn, o), u = __shfl_up_sync(0xffffffffu, sc, o);
+            if (lane >= o) {
+                sn += t;
+                sc += u;
+            }
+        }
+        int32_t b0 = 0, b1 = 0;
+        if (lane == 31) {
+            if (sn) b0 = atomicAdd(left, sn);
+            if (sc) b1 = atomicAdd(left + 1, sc);
+        }
+        b0 = __shfl_sync(0xffffffffu, b0, 31);
+        b1 = __shfl_sync(0xffffffffu, b1, 31);
+        if (lane < kGroups) {
+            at_large[lane] = b0 + sn - n;
+            at_chunk[lane] = b1 + sc - c;
+        }
+    }
+    __syncthreads();
+    for (int q = warp; q < kGroups; q += kBlock / 32) {
+        const int64_t s0 = base + 32 * q;
+        const uint32_t big = s_big[q];
+        if ((big >> lane) & 1u)
+            large[at_large[q] + __popc(big & ((1u << lane) - 1u))] = (int32_t)s0 + lane;
+        if (lane == 0 && s_small[q]) chunks[at_chunk[q]] = (int32_t)(s0 >> 5);
+    }
 }
 
 __device__ __forceinline__ bool jt_pairs(int t) {
@@ -612,10 +637,15 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
                 if (r != XM_OK) return r;
             }
             // (input order: the scan takes the sources request by request)
-            XM_LAUNCH("k_batch_prep", grid_for(total), kBlock, 0, s, k_batch_prep, C,
-                      sorted_a ? (const uint32_t*)B.vals : (const uint32_t*)nullptr, B.prep, B.cold,
-                      B.lrow, sorted_a ? (int32_t*)nullptr : err, bad_req, B.lists + 3 * nn,
-                      B.lists + 4 * nn, left);
+            auto prep = [&](auto kernel, int rounds) -> xm_status {
+                XM_LAUNCH("k_batch_prep", grid_for((total + rounds - 1) / rounds), kBlock, 0, s, kernel,
+                          C, sorted_a ? (const uint32_t*)B.vals : (const uint32_t*)nullptr, B.prep,
+                          B.cold, B.lrow, sorted_a ? (int32_t*)nullptr : err, bad_req,
+                          B.lists + 3 * nn, B.lists + 4 * nn, left);
+                return XM_OK;
+            };
+            const xm_status rp = total >= (1 << 19) ? prep(k_batch_prep<4>, 4) : prep(k_batch_prep<1>, 1);
+            if (rp != XM_OK) return rp;
         }
         ScanArgs a{};
         a.G = X->geom();

@@ -52,3 +52,29 @@ def test_batch_of_sizes(prec, order, kind, sizes):
             np.testing.assert_array_equal(v[f].cpu().numpy(), getattr(ref, f).cpu().numpy(), err_msg=f)
         for f in ("sep", "best_sep"):
             np.testing.assert_allclose(v[f].cpu().numpy(), getattr(ref, f).cpu().numpy(), rtol=0, atol=tol)
+
+
+def test_large_batch():
+    """As many sources as take several rounds a thread in the preparation."""
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1611_08494_gb300 import xm
+
+    g = synth.rng(1850)
+    lon, lat = g.uniform(0.0, 360.0, 300_000), g.uniform(-60.0, 60.0, 300_000)
+    idx = xm.Index(_cuda(lon), _cuda(lat), zone_height_arcsec=ZONE_H)
+    reqs = []
+    for k, n in enumerate((1_500_001, 2_000_000, 700_077)):
+        pick = g.integers(0, lon.size, n)
+        q = dict(lon=_cuda(lon[pick]), lat=_cuda(np.clip(lat[pick] + g.normal(0, 5e-4, n), -90, 90)))
+        a = 0.5 * 100.0 ** g.uniform(0, 1, n)
+        q.update((dict(a=30.0), dict(a_col=_cuda(a)), dict(a=2.0))[k])
+        reqs.append(q)
+    batch = xm.Batch(idx, reqs)
+    for r, q in enumerate(reqs):
+        v, q = batch.view(r), dict(q)
+        ref = xm.Result(idx, q.pop("lon"), q.pop("lat"), **q)
+        for f in ("a_row", "b_row", "count", "best_b"):
+            assert torch.equal(v[f], getattr(ref, f)), f
