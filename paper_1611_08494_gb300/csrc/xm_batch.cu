@@ -117,9 +117,11 @@ __global__ void k_batch_ingest(BatchConst C, uint64_t* __restrict__ keys,
 // too large for the sparse count pass are listed for the general one (left[0]
 // of them), and the chunks of 32 with another one for the sparse pass (left[1]).
 // A block takes its places in the lists with one atomic each after ROUNDS
-// sources a thread and waits for them, so batches of 2^19 sources and more take
-// four rounds: 0.16 ms for 3.8e6 sources, 0.205 with one (0.183 without the
-// lists), 1.10 for 3.2e7.
+// sources a thread and waits for them, so batches of 2^22 sources and more take
+// four rounds: 0.245 ms for 6.4e6 sources and 1.10 for 3.2e7 (0.27 and 1.21 with
+// one and no lists; 4.2e8: 16.9, 20.6 with one and lists). Below, blocks of
+// rotated sources, some ten times the work, would end long after the others: 24
+// requests of 3.5e6 sources in three batches took 4 % longer with four rounds.
 template <int ROUNDS>
 __global__ void __launch_bounds__(kBlock) k_batch_prep(
     BatchConst C, const uint32_t* __restrict__ vals, APrep* __restrict__ out,
@@ -644,7 +646,7 @@ static xm_status batch_pass(const xm_index* X, const xm_request* reqs, int64_t n
                           B.lists + 3 * nn, B.lists + 4 * nn, left);
                 return XM_OK;
             };
-            const xm_status rp = total >= (1 << 19) ? prep(k_batch_prep<4>, 4) : prep(k_batch_prep<1>, 1);
+            const xm_status rp = total >= (1 << 22) ? prep(k_batch_prep<4>, 4) : prep(k_batch_prep<1>, 1);
             if (rp != XM_OK) return rp;
         }
         ScanArgs a{};
