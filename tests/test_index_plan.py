@@ -11,7 +11,7 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
                     "paper_1611_08494_gb300", "csrc")
 
-DRIVER = r"""
+PLAN = r"""
 #include <stdio.h>
 #include <vector>
 #include "xm_plan.cuh"
@@ -57,7 +57,7 @@ def test_bins_fit_their_arrays(tmp_path):
     if not cxx:
         pytest.skip("no C++ compiler")
     src = tmp_path / "plan.cpp"
-    src.write_text(DRIVER)
+    src.write_text(PLAN)
     exe = str(tmp_path / "plan")
     subprocess.run([cxx, "-std=c++17", "-O2", "-I" + CSRC, "-o", exe, str(src)], check=True)
     r = subprocess.run([exe], capture_output=True, text=True)
